@@ -5,13 +5,10 @@
 // Kernel 1 (route_topk), bf16 tokens: route_mma_kernel below (or, with
 // VMOE_ROUTE_TC=1, route_tc_kernel in route_tc.cu on tcgen05) -- the router
 // product on the tensor cores (mma.sync) with the fp32 weights split into
-// three bf16 parts.  fp32 tokens or given logits: one CTA per (task, tile of
-// TOK tokens) on the CUDA cores.  The logits
-// tile [TOK x E] = x_tile [TOK x d] * W_r[t] [d x E] is accumulated in fp32
-// registers (4 tokens x 4 experts per thread, d swept in chunks of 32 staged
-// in shared memory, one FMA chain per output in increasing i), then written to
-// shared memory and to `logits`.  One thread per token then takes the max,
-// the softmax denominator and the k largest logits (ties to the lower expert
+// three bf16 parts.  fp32 tokens: route_f32_kernel on the CUDA cores; given
+// logits: route_given_kernel.  One CTA per (task, tile of tokens); the logits
+// tile goes through shared memory, and one thread per token takes the max, the
+// softmax denominator and the k largest logits (ties to the lower expert
 // index).
 //
 // Kernel 2 (capacity_scan): one CTA per task.  The choice-major assignment
@@ -29,7 +26,6 @@ namespace vmoe {
 namespace {
 
 constexpr int RT_THREADS = 256;
-constexpr int RT_KC = 32;  // d-chunk staged per iteration
 
 // Softmax + top-k of `ntok` logit rows held in shared memory (row pitch ldl,
 // odd, so the per-thread rows hit distinct banks), one thread per row.
@@ -40,110 +36,133 @@ __device__ __forceinline__ void topk_rows(const Dims &p, const float *lg, int ld
         topk_row(p, lg + r * ldl, (long long)t * p.N + n0 + r, out_idx, out_gate);
 }
 
-// SIMT router for fp32 tokens (or given logits): ECH experts per pass, TOK
-// tokens per CTA, TOK * ECH = 16 * RT_THREADS.
-template <typename TX, int ECH>
+// Given logits (VMOE_LOGITS_IN): the rows of RT_TOK tokens through shared memory.
+constexpr int RT_TOK = 64;
 __global__ void __launch_bounds__(RT_THREADS)
-route_topk_kernel(Dims p, const TX *__restrict__ x, const float *__restrict__ wr,
-                  const float *__restrict__ bias, float *__restrict__ logits,
-                  int32_t *__restrict__ out_idx, float *__restrict__ out_gate, int logits_in) {
-    constexpr int TOK = 16 * RT_THREADS / ECH;
-    constexpr int TX_THREADS = ECH / 4;  // threads along experts
+route_given_kernel(Dims p, const float *__restrict__ logits, int32_t *__restrict__ out_idx,
+                   float *__restrict__ out_gate) {
+    pdl_wait();
+    extern __shared__ __align__(16) float smem[];  // [RT_TOK][E + 1]
+    const int t = blockIdx.y, n0 = blockIdx.x * RT_TOK, E = p.E;
+    const int ntok = min(RT_TOK, p.N - n0);
+    for (int i = threadIdx.x; i < ntok * E; i += RT_THREADS) {
+        const int r = i / E, e = i - r * E;
+        smem[r * (E + 1) + e] = logits[((long long)t * p.N + n0 + r) * E + e];
+    }
+    __syncthreads();
+    topk_rows(p, smem, E + 1, ntok, t, n0, out_idx, out_gate, RT_THREADS);
+}
+
+// CUDA-core router for fp32 tokens: RF_TOK tokens x ECH experts a pass, 4 x 4
+// logits a thread.  d is swept in chunks of RF_KC staged in shared memory (the
+// next chunk's loads in registers meanwhile); RF_SLICES groups of threads take
+// a slice of every chunk each, and their partial logits are summed in slice
+// order.  A layer's few hundred tokens are a few dozen CTAs, so the chain of
+// chunks is what bounds it, not the arithmetic.
+constexpr int RF_TOK = 16;
+constexpr int RF_KC = 128;
+constexpr int RF_XP = RF_KC + 4;  // x row pitch (floats)
+template <int ECH>
+struct RouteF32 {
+    static constexpr int EG = ECH / 4;                         // threads along experts
+    static constexpr int SLICES = RT_THREADS / (EG * (RF_TOK / 4));
+    static constexpr int KS = RF_KC / SLICES;                  // d per slice and chunk
+    static constexpr int XV = RF_TOK * RF_KC / 4 / RT_THREADS;  // x vectors per thread
+    static constexpr int WV = RF_KC * ECH / RT_THREADS;        // weights per thread
+    static constexpr size_t smem(int E) {
+        return sizeof(float) * ((size_t)RF_TOK * RF_XP + (size_t)RF_KC * ECH +
+                                (size_t)SLICES * RF_TOK * ECH + (size_t)RF_TOK * (E + 1));
+    }
+    static_assert(KS % 4 == 0, "a slice is swept four values of d at a time");
+};
+
+template <int ECH>
+__global__ void __launch_bounds__(RT_THREADS)
+route_f32_kernel(Dims p, const float *__restrict__ x, const float *__restrict__ wr,
+                 const float *__restrict__ bias, float *__restrict__ logits,
+                 int32_t *__restrict__ out_idx, float *__restrict__ out_gate) {
+    using S = RouteF32<ECH>;
+    pdl_wait();
     extern __shared__ __align__(16) float smem[];
-    float *xs = smem;                    // [RT_KC][TOK]  (x chunk, transposed)
-    float *ws = xs + RT_KC * TOK;        // [RT_KC][ECH]
-    float *lg = ws + RT_KC * ECH;        // [TOK][E + 1]
-
-    const int t = blockIdx.y;
-    const int n0 = blockIdx.x * TOK;
-    const int E = p.E, d = p.d, N = p.N;
-    const int ldl = E + 1;
-    const int tid = threadIdx.x;
-    const int ntok = min(TOK, N - n0);
-
-    if (logits_in) {
-        for (int i = tid; i < ntok * E; i += RT_THREADS) {
-            int r = i / E, e = i - r * E;
-            lg[r * ldl + e] = logits[((long long)t * N + n0 + r) * E + e];
-        }
-    } else {
-        const int tg = tid / TX_THREADS;  // token group: tokens 4*tg .. 4*tg+3
-        const int eg = tid % TX_THREADS;  // expert group: experts 4*eg .. 4*eg+3
-        const TX *xt = x + ((long long)t * N + n0) * d;
-        const float *wt = wr + (long long)t * d * E;
-        for (int e0 = 0; e0 < E; e0 += ECH) {
-            float acc[4][4];
+    float *xs = smem;                            // [RF_TOK][RF_XP]
+    float *ws = xs + RF_TOK * RF_XP;             // [RF_KC][ECH]
+    float *part = ws + RF_KC * ECH;              // [SLICES][RF_TOK][ECH]
+    float *lg = part + S::SLICES * RF_TOK * ECH;  // [RF_TOK][E + 1]
+    const int t = blockIdx.y, n0 = blockIdx.x * RF_TOK;
+    const int E = p.E, d = p.d, N = p.N, ldl = E + 1, tid = threadIdx.x;
+    const int ntok = min(RF_TOK, N - n0);
+    const int eg = tid % S::EG, tg = tid / S::EG % (RF_TOK / 4), sl = tid / (S::EG * (RF_TOK / 4));
+    const float *xt = x + ((long long)t * N + n0) * d;
+    const float *wt = wr + (long long)t * d * E;
+    float4 xv[S::XV];
+    float wv[S::WV];
+    for (int e0 = 0; e0 < E; e0 += ECH) {
+        auto load = [&](int k0) {
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = 0.0f;
-            for (int k0 = 0; k0 < d; k0 += RT_KC) {
-                __syncthreads();
-                // 16-byte vector loads along d (d % 8 == 0, so a vector is
-                // either wholly inside the row or wholly past its end).
-                constexpr int VEC = 16 / sizeof(TX);
-                for (int i = tid; i < TOK * (RT_KC / VEC); i += RT_THREADS) {
-                    int r = i / (RT_KC / VEC), c = (i - r * (RT_KC / VEC)) * VEC;
-                    float v[VEC];
-                    if (r < ntok && k0 + c < d) {
-                        uint4 raw = *reinterpret_cast<const uint4 *>(xt + (long long)r * d + k0 + c);
-                        if constexpr (VEC == 8) {
-                            bf16x8_to_f32(raw, v);
-                        } else {
-                            v[0] = __uint_as_float(raw.x);
-                            v[1] = __uint_as_float(raw.y);
-                            v[2] = __uint_as_float(raw.z);
-                            v[3] = __uint_as_float(raw.w);
-                        }
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < VEC; ++q) v[q] = 0.0f;
-                    }
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) xs[(c + q) * TOK + r] = v[q];
-                }
-                for (int i = tid; i < RT_KC * ECH; i += RT_THREADS) {
-                    int r = i / ECH, c = i - r * ECH;
-                    float v = 0.0f;
-                    if (k0 + r < d && e0 + c < E) v = wt[(long long)(k0 + r) * E + e0 + c];
-                    ws[r * ECH + c] = v;
-                }
-                __syncthreads();
-#pragma unroll 8
-                for (int kk = 0; kk < RT_KC; ++kk) {
-                    float4 av = *reinterpret_cast<const float4 *>(&xs[kk * TOK + 4 * tg]);
-                    float4 bv = *reinterpret_cast<const float4 *>(&ws[kk * ECH + 4 * eg]);
-                    float a4[4] = {av.x, av.y, av.z, av.w};
-                    float b4[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-                    for (int a = 0; a < 4; ++a)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(a4[a], b4[b], acc[a][b]);
-                }
+            for (int q = 0; q < S::XV; ++q) {  // d % 8 == 0: a vector is inside its row or past it
+                const int i = tid + q * RT_THREADS, r = i / (RF_KC / 4), c = i % (RF_KC / 4) * 4;
+                xv[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (r < ntok && k0 + c < d)
+                    xv[q] = __ldg(reinterpret_cast<const float4 *>(xt + (long long)r * d + k0 + c));
             }
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                int r = 4 * tg + a;
+            for (int q = 0; q < S::WV; ++q) {
+                const int i = tid + q * RT_THREADS, r = i / ECH, c = i % ECH;
+                wv[q] = k0 + r < d && e0 + c < E ? __ldg(wt + (long long)(k0 + r) * E + e0 + c) : 0.0f;
+            }
+        };
+        float acc[4][4] = {};
+        load(0);
+        for (int k0 = 0; k0 < d; k0 += RF_KC) {
+            __syncthreads();  // the previous chunk has been read
 #pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    int e = e0 + 4 * eg + b;
-                    if (r < ntok && e < E) {
-                        float v = acc[a][b];
-                        if (bias) v += bias[(long long)t * E + e];
-                        lg[r * ldl + e] = v;
+            for (int q = 0; q < S::XV; ++q) {
+                const int i = tid + q * RT_THREADS;
+                *reinterpret_cast<float4 *>(xs + i / (RF_KC / 4) * RF_XP + i % (RF_KC / 4) * 4) = xv[q];
+            }
+#pragma unroll
+            for (int q = 0; q < S::WV; ++q) ws[tid + q * RT_THREADS] = wv[q];
+            __syncthreads();
+            if (k0 + RF_KC < d) load(k0 + RF_KC);
+#pragma unroll 2
+            for (int kk = sl * S::KS; kk < (sl + 1) * S::KS; kk += 4) {
+                float4 a[4], b[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    a[i] = *reinterpret_cast<const float4 *>(xs + (4 * tg + i) * RF_XP + kk);
+                    b[i] = *reinterpret_cast<const float4 *>(ws + (kk + i) * ECH + 4 * eg);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float av[4] = {a[i].x, a[i].y, a[i].z, a[i].w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        acc[i][0] = fmaf(av[q], b[q].x, acc[i][0]);
+                        acc[i][1] = fmaf(av[q], b[q].y, acc[i][1]);
+                        acc[i][2] = fmaf(av[q], b[q].z, acc[i][2]);
+                        acc[i][3] = fmaf(av[q], b[q].w, acc[i][3]);
                     }
                 }
             }
         }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            *reinterpret_cast<float4 *>(part + (sl * RF_TOK + 4 * tg + i) * ECH + 4 * eg) =
+                make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
         __syncthreads();
-        for (int i = tid; i < ntok * E; i += RT_THREADS) {
-            int r = i / E, e = i - r * E;
-            logits[((long long)t * N + n0 + r) * E + e] = lg[r * ldl + e];
+        for (int i = tid; i < RF_TOK * ECH; i += RT_THREADS) {
+            const int r = i / ECH, e = e0 + i % ECH;
+            if (r >= ntok || e >= E) continue;
+            float v = part[i];
+#pragma unroll
+            for (int q = 1; q < S::SLICES; ++q) v += part[q * RF_TOK * ECH + i];
+            if (bias) v += bias[(long long)t * E + e];
+            lg[r * ldl + e] = v;
+            logits[((long long)t * N + n0 + r) * E + e] = v;
         }
     }
     __syncthreads();
-
-    topk_rows(p, lg, E + 1, ntok, t, n0, out_idx, out_gate, RT_THREADS);
+    topk_rows(p, lg, ldl, ntok, t, n0, out_idx, out_gate, RT_THREADS);
 }
 
 // Tensor-core router for bf16 tokens.  x is exactly representable in bf16, so
@@ -393,20 +412,28 @@ capacity_scan_kernel(Dims p, const int32_t *__restrict__ idx, int32_t *__restric
     }
 }
 
-template <typename TX, int ECH>
-int launch_topk(const Dims &p, const TX *x, const float *wr, const float *bias, float *logits,
-                int32_t *idx, float *gate, cudaStream_t s) {
-    constexpr int TOK = 16 * RT_THREADS / ECH;
-    size_t smem = sizeof(float) * ((size_t)RT_KC * TOK + (size_t)RT_KC * ECH + (size_t)TOK * (p.E + 1));
+int launch_given(const Dims &p, const float *logits, int32_t *idx, float *gate, cudaStream_t s) {
+    const size_t smem = sizeof(float) * (size_t)RT_TOK * (p.E + 1);
     static std::atomic<int> smem_limit[64];
-    if (const int st = raise_smem_limit((const void *)route_topk_kernel<TX, ECH>, smem_limit, (int)smem))
-        return st;
-    dim3 grid((p.N + TOK - 1) / TOK, p.T);
+    if (const int st = raise_smem_limit((const void *)route_given_kernel, smem_limit, (int)smem)) return st;
     trace_before(s, "route_topk");
-    route_topk_kernel<TX, ECH><<<grid, RT_THREADS, smem, s>>>(p, x, wr, bias, logits, idx, gate,
-                                                              x == nullptr);
+    const int st = launch_kernel(route_given_kernel, dim3((p.N + RT_TOK - 1) / RT_TOK, p.T), dim3(RT_THREADS),
+                                 smem, s, p, logits, idx, gate);
     trace_after(s);
-    return launch_result();
+    return st;
+}
+
+template <int ECH>
+int launch_f32(const Dims &p, const float *x, const float *wr, const float *bias, float *logits,
+               int32_t *idx, float *gate, cudaStream_t s) {
+    const size_t smem = RouteF32<ECH>::smem(p.E);
+    static std::atomic<int> smem_limit[64];
+    if (const int st = raise_smem_limit((const void *)route_f32_kernel<ECH>, smem_limit, (int)smem)) return st;
+    trace_before(s, "route_topk");
+    const int st = launch_kernel(route_f32_kernel<ECH>, dim3((p.N + RF_TOK - 1) / RF_TOK, p.T), dim3(RT_THREADS),
+                                 smem, s, p, x, wr, bias, logits, idx, gate);
+    trace_after(s);
+    return st;
 }
 
 template <int CS_THREADS>
@@ -439,12 +466,12 @@ int launch_route(const Dims &p, const void *x, const float *w_router, const floa
         else
             st = p.E <= 32 ? launch_mma_router<4>(p, xb, w_router, bias, logits, idx, gate, s)
                            : launch_mma_router<8>(p, xb, w_router, bias, logits, idx, gate, s);
-    } else if (p.bf16) {  // given logits: no GEMV
-        st = launch_topk<__nv_bfloat16, 64>(p, nullptr, w_router, bias, logits, idx, gate, s);
+    } else if (x == nullptr) {
+        st = launch_given(p, logits, idx, gate, s);
     } else {
         const float *xf = (const float *)x;
-        st = p.E <= 32 ? launch_topk<float, 32>(p, xf, w_router, bias, logits, idx, gate, s)
-                       : launch_topk<float, 64>(p, xf, w_router, bias, logits, idx, gate, s);
+        st = p.E <= 32 ? launch_f32<32>(p, xf, w_router, bias, logits, idx, gate, s)
+                       : launch_f32<64>(p, xf, w_router, bias, logits, idx, gate, s);
     }
     if (st != VMOE_OK) return st;
     trace_before(s, "capacity_scan");

@@ -1,0 +1,29 @@
+"""fp32 problems where the CUDA-core kernels change path: 128- and 64-wide tiles with ragged edges, K ranges
+split over a cluster, router chunks and expert passes with remainders, one token.  Held to the fp32 bars of the
+parity tests (1e-5 of an output's RMS: sums of a few hundred to a few thousand fp32 products in any order stay
+under 1e-6)."""
+import pytest
+
+import workloads
+from gpu_helpers import run_step, to_dev
+from test_gpu_parity import _compare_step, _lib  # noqa: F401  (the fixture that builds the library)
+
+pytestmark = pytest.mark.gpu
+
+Config = workloads.Config
+CASES = [
+    # 64 groups: 128 x 128 tiles; d = 72 and f = 1028 end inside a tile and a K chunk
+    Config("f32_wide_tiles", 90, T=2, N=300, d=72, f=1028, E=32, k=2, cf=1.25, dtype="f32", bias="drift"),
+    # 2 groups, K = 516 (33 chunks) over 8 CTAs; row tiles of 64 and of 2 rows
+    Config("f32_split", 91, T=1, N=66, d=128, f=516, E=2, k=2, cf=1.0, dtype="f32", flags=4),
+    # 70 experts (two router passes of 64), d = 136 (a chunk of 8), empty groups
+    Config("f32_experts70", 92, T=2, N=45, d=136, f=64, E=70, k=3, cf=1.0, dtype="f32", bias="zipf", flags=2),
+    Config("f32_one_token", 93, T=1, N=1, d=8, f=4, E=2, k=1, cf=1.0, dtype="f32"),
+]
+
+
+@pytest.mark.parametrize("cfg", CASES, ids=lambda c: c.name)
+def test_f32_step_parity(cfg):
+    inp = workloads.make_inputs(cfg)
+    _, b = run_step(cfg, to_dev(inp))
+    _compare_step(cfg, inp, b, cfg.flags)
