@@ -227,38 +227,110 @@ __device__ __forceinline__ float gelu_deriv_f(float h, bool tanh_form) {
     return 0.5f * (1.0f + erff(h * 0.7071067811865476f)) + h * inv_sqrt_2pi * expf(-0.5f * h * h);
 }
 
-// Fast exact-form GELU for the bf16 epilogues.  erf(x), x >= 0, by the Hastings
-// rational approximation (Abramowitz & Stegun, Handbook of Mathematical
-// Functions, formula 7.1.26): erf(x) = 1 - t (a1 + t (a2 + t (a3 + t (a4 + t a5))))
-// exp(-x^2), t = 1 / (1 + p x), with |error| <= 1.5e-7 -- far below the bf16
-// rounding of the stored outputs.  With x = |h| / sqrt 2 the factor exp(-x^2) =
-// exp(-h^2 / 2) is also the one in the normal density, so GELU' costs one
-// exponential, one reciprocal and a five-term polynomial.
-struct PhiParts {
-    float Phi;  // standard normal CDF at h
-    float E;    // exp(-h^2 / 2)
-};
-__device__ __forceinline__ PhiParts phi_parts(float h) {
-    const float p = 0.3275911f, a1 = 0.254829592f, a2 = -0.284496736f, a3 = 1.421413741f,
-                a4 = -1.453152027f, a5 = 1.061405429f;
-    const float x = fabsf(h) * 0.7071067811865476f;
-    const float t = __fdividef(1.0f, fmaf(p, x, 1.0f));
-    const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, a5, a4), a3), a2), a1);
-    const float E = __expf(-0.5f * h * h);
-    const float tail = 0.5f * poly * E;  // = P(Z > |h|)
-    PhiParts r;
-    r.Phi = h >= 0.0f ? 1.0f - tail : tail;
-    r.E = E;
+// Two fp32 values in one 64-bit register: sm_100 and later run one packed
+// instruction where two scalar ones would issue.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
     return r;
 }
-__device__ __forceinline__ float gelu_fast(float h, bool tanh_form) {
-    if (tanh_form) return gelu_f(h, true);
-    return h * phi_parts(h).Phi;
+__device__ __forceinline__ f32x2 pk2(float v) { return pk2(v, v); }
+__device__ __forceinline__ float2 unpk2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
 }
-__device__ __forceinline__ float gelu_deriv_fast(float h, bool tanh_form) {
-    if (tanh_form) return gelu_deriv_f(h, true);
-    const PhiParts r = phi_parts(h);
-    return fmaf(h * 0.3989422804014327f, r.E, r.Phi);
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 rcp2(f32x2 v) {
+    float2 a = unpk2(v);
+    asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(a.x));
+    asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(a.y));
+    return pk2(a.x, a.y);
+}
+__device__ __forceinline__ f32x2 exp2_2(f32x2 v) {
+    float2 a = unpk2(v);
+    asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(a.x));
+    asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(a.y));
+    return pk2(a.x, a.y);
+}
+// The two bf16 of a 32-bit word, and back (round to nearest even).
+__device__ __forceinline__ f32x2 bf16x2_to_f32x2(uint32_t w) {
+    return pk2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+__device__ __forceinline__ uint32_t f32x2_to_bf16x2(f32x2 v) {
+    const float2 a = unpk2(v);
+    return pack_bf16x2(a.x, a.y);
+}
+
+// GELU and GELU' of two values for the bf16 epilogues, whose issue slots they
+// fill: about 10 instructions a value, where the scalar form with __expf and
+// __fdividef took about 20.
+//
+// Exact form.  erf(x), x >= 0, by the Hastings rational approximation
+// (Abramowitz & Stegun, Handbook of Mathematical Functions, formula 7.1.26):
+// erf(x) = 1 - t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-x^2),
+// t = 1 / (1 + p x), with |error| <= 1.5e-7 -- far below the bf16 rounding of
+// the stored outputs.  With x = |h| / sqrt 2 the factor exp(-x^2) =
+// exp(-h^2 / 2) is also the one in the normal density, so GELU' costs one
+// exponential, one reciprocal and a five-term polynomial.
+struct Phi2 {
+    f32x2 Phi;  // standard normal CDF at h
+    f32x2 E;    // exp(-h^2 / 2)
+};
+__device__ __forceinline__ Phi2 phi2(f32x2 h) {
+    const float p = 0.3275911f, a1 = 0.254829592f, a2 = -0.284496736f, a3 = 1.421413741f,
+                a4 = -1.453152027f, a5 = 1.061405429f;
+    const float2 hv = unpk2(h);
+    const f32x2 t = rcp2(fma2(pk2(fabsf(hv.x), fabsf(hv.y)), pk2(p * 0.7071067811865476f), pk2(1.0f)));
+    f32x2 poly = fma2(t, pk2(0.5f * a5), pk2(0.5f * a4));
+    poly = fma2(t, poly, pk2(0.5f * a3));
+    poly = fma2(t, poly, pk2(0.5f * a2));
+    poly = mul2(t, fma2(t, poly, pk2(0.5f * a1)));
+    Phi2 r;
+    r.E = exp2_2(mul2(mul2(h, h), pk2(-0.5f * 1.4426950408889634f)));
+    const f32x2 tail = mul2(poly, r.E);  // P(Z > |h|)
+    const float2 tv = unpk2(tail), uv = unpk2(fma2(tail, pk2(-1.0f), pk2(1.0f)));
+    r.Phi = pk2(hv.x >= 0.0f ? uv.x : tv.x, hv.y >= 0.0f ? uv.y : tv.y);
+    return r;
+}
+// Tanh form: 0.5 (1 + tanh u) = s(2u) = 1 / (1 + exp(-2u)), the logistic
+// function, u = sqrt(2/pi) (h + 0.044715 h^3); s'(2u) = s (1 - s) with 1 - s =
+// exp(-2u) s, free of cancellation.
+constexpr float GELU_TANH_C = 0.7978845608028654f;  // sqrt(2/pi)
+__device__ __forceinline__ f32x2 gelu2(f32x2 h, bool tanh_form) {
+    if (!tanh_form) return mul2(h, phi2(h).Phi);
+    const float k = -2.0f * 1.4426950408889634f * GELU_TANH_C;
+    const f32x2 z = mul2(h, fma2(mul2(h, h), pk2(k * 0.044715f), pk2(k)));
+    return mul2(h, rcp2(add2(exp2_2(z), pk2(1.0f))));
+}
+__device__ __forceinline__ f32x2 gelu_deriv2(f32x2 h, bool tanh_form) {
+    if (!tanh_form) {
+        const Phi2 r = phi2(h);
+        return fma2(mul2(h, pk2(0.3989422804014327f)), r.E, r.Phi);
+    }
+    const float k = -2.0f * 1.4426950408889634f * GELU_TANH_C;
+    const f32x2 h2 = mul2(h, h);
+    const float2 z = unpk2(mul2(h, fma2(h2, pk2(k * 0.044715f), pk2(k))));
+    // exp(-2u) below overflow, so that (1 - s) s stays 0 and not 0 * inf for large negative h
+    const f32x2 e = exp2_2(pk2(fminf(z.x, 125.0f), fminf(z.y, 125.0f)));
+    const f32x2 s = rcp2(add2(e, pk2(1.0f)));
+    const f32x2 du = fma2(h2, pk2(2.0f * GELU_TANH_C * 3.0f * 0.044715f), pk2(2.0f * GELU_TANH_C));
+    return fma2(mul2(mul2(h, mul2(e, s)), du), s, s);
 }
 
 }  // namespace vmoe

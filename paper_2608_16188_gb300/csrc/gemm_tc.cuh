@@ -379,6 +379,44 @@ __device__ __forceinline__ Tile decode_tile(const Args &a, const int *prefix, in
     return t;
 }
 
+// The elementwise step of a row-mode epilogue on CH accumulator columns of one
+// row (pairs in v, clobbered), packed to bf16: out(words, 0) for the first
+// output and out(words, 1) for the second -- A = GELU(H), or the residual
+// v - bf16(v) of dH, which carries it to about 16 bits.  h: EPI_DGELU's H
+// values of the chunk.
+template <int EPI, int CH, typename Out>
+__device__ __forceinline__ void epilogue_chunk(f32x2 (&v)[CH / 2], const uint4 *h, bool tanh_form, Out out) {
+    uint32_t w[CH / 2];
+    if (EPI == EPI_DGELU) {
+        const uint32_t *hw = reinterpret_cast<const uint32_t *>(h);
+        if (tanh_form) {
+#pragma unroll
+            for (int i = 0; i < CH / 2; ++i) v[i] = mul2(v[i], gelu_deriv2(bf16x2_to_f32x2(hw[i]), true));
+        } else {
+#pragma unroll
+            for (int i = 0; i < CH / 2; ++i) v[i] = mul2(v[i], gelu_deriv2(bf16x2_to_f32x2(hw[i]), false));
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < CH / 2; ++i) w[i] = f32x2_to_bf16x2(v[i]);
+    out(w, 0);
+    if (EPI == EPI_DGELU) {
+#pragma unroll
+        for (int i = 0; i < CH / 2; ++i) w[i] = f32x2_to_bf16x2(fma2(bf16x2_to_f32x2(w[i]), pk2(-1.0f), v[i]));
+        out(w, 1);
+    }
+    if (EPI == EPI_GELU) {
+        if (tanh_form) {
+#pragma unroll
+            for (int i = 0; i < CH / 2; ++i) w[i] = f32x2_to_bf16x2(gelu2(v[i], true));
+        } else {
+#pragma unroll
+            for (int i = 0; i < CH / 2; ++i) w[i] = f32x2_to_bf16x2(gelu2(v[i], false));
+        }
+        out(w, 1);
+    }
+}
+
 template <int BN, int MODE, bool A_MN, bool B_MN, int EPI>
 __global__ void __launch_bounds__(Roles<MODE, EPI>::NT, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -756,10 +794,11 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
             __syncwarp();
         };
-        auto stage = [&](const float *v) {
+        auto stage = [&](const uint32_t(&w)[CH / 2]) {
 #pragma unroll
             for (int i = 0; i < CH / 8; ++i)
-                *reinterpret_cast<uint4 *>(stg + lane * PITCH + i * 16) = f32_to_bf16x8(v + i * 8);
+                *reinterpret_cast<uint4 *>(stg + lane * PITCH + i * 16) =
+                    make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
         };
         int it = 0;
         Tile t = decode_tile<MODE>(args, prefix, blockIdx.x < total ? blockIdx.x : 0);
@@ -788,43 +827,22 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     else if (have_next) load_h(tn, jw, hnxt);
                 }
                 if (nvalid > 0) {
-                    float v[CH];
+                    f32x2 v[CH / 2];
                     if (t.kblocks > 0) {
                         uint32_t r[CH];
-                        if (CH == 32) tmem_ld32(trow + c * CH, *reinterpret_cast<uint32_t(*)[32]>(r));
-                        else tmem_ld16(trow + c * CH, *reinterpret_cast<uint32_t(*)[16]>(r));
+                        tmem_ld32(trow + c * CH, r);
                         tmem_ld_wait();
 #pragma unroll
-                        for (int i = 0; i < CH; ++i) v[i] = __uint_as_float(r[i]);
+                        for (int i = 0; i < CH / 2; ++i)
+                            v[i] = pk2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
                     } else {
 #pragma unroll
-                        for (int i = 0; i < CH; ++i) v[i] = 0.0f;
+                        for (int i = 0; i < CH / 2; ++i) v[i] = pk2(0.0f);
                     }
-                    if (EPI == EPI_DGELU) {
-#pragma unroll
-                        for (int i = 0; i < CH / 8; ++i) {
-                            float hv[8];
-                            bf16x8_to_f32(hcur[i], hv);
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) v[i * 8 + e] *= gelu_deriv_fast(hv[e], tanh_form);
-                        }
-                    }
-                    stage(v);
-                    store_rows(args.D + gofs + c * CH, nvalid);
-                    if (EPI == EPI_DGELU) {  // residual v - bf16(v): dH = hi + lo to ~16 bits
-                        float lv[CH];
-#pragma unroll
-                        for (int i = 0; i < CH; ++i) lv[i] = v[i] - __bfloat162float(__float2bfloat16_rn(v[i]));
-                        stage(lv);
-                        store_rows(args.D2 + gofs2 + c * CH, nvalid);
-                    }
-                    if (EPI == EPI_GELU) {
-                        float gv[CH];
-#pragma unroll
-                        for (int i = 0; i < CH; ++i) gv[i] = gelu_fast(v[i], tanh_form);
-                        stage(gv);
-                        store_rows(args.D2 + gofs2 + c * CH, nvalid);
-                    }
+                    epilogue_chunk<EPI, CH>(v, hcur, tanh_form, [&](const uint32_t(&w)[CH / 2], int out) {
+                        stage(w);
+                        store_rows(out == 0 ? args.D + gofs + c * CH : args.D2 + gofs2 + c * CH, nvalid);
+                    });
                 }
                 if (EPI == EPI_DGELU) {
 #pragma unroll

@@ -924,48 +924,20 @@ row_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     else if (have_next) load_h(tn, 0, hnxt);
                 }
                 if (nvalid > 0) {
-                    float v[32];
+                    f32x2 v[16];
                     uint32_t r[32];
                     tmem_ld32(trow + c * 32, r);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-                    if (EPI == EPI_DGELU) {
+                    for (int i = 0; i < 16; ++i)
+                        v[i] = pk2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+                    epilogue_chunk<EPI, 32>(v, hcur, tanh_form, [&](const uint32_t(&w)[16], int out) {
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            float hv[8];
-                            bf16x8_to_f32(hcur[i], hv);
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) v[i * 8 + e] *= gelu_deriv_fast(hv[e], tanh_form);
-                        }
-                    }
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        *reinterpret_cast<uint4 *>(stg + lane * 80 + i * 16) = f32_to_bf16x8(v + i * 8);
-                    store_rows(args.D + gofs + c * 32, nvalid);
-                    if (EPI == EPI_DGELU) {  // residual v - bf16(v): dH = hi + lo to ~16 bits
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            float lv[8];
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) {
-                                const float x = v[i * 8 + e];
-                                lv[e] = x - __bfloat162float(__float2bfloat16_rn(x));
-                            }
-                            *reinterpret_cast<uint4 *>(stg + lane * 80 + i * 16) = f32_to_bf16x8(lv);
-                        }
-                        store_rows(args.D2 + gofs2 + c * 32, nvalid);
-                    }
-                    if (EPI == EPI_GELU) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            float gv[8];
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) gv[e] = gelu_fast(v[i * 8 + e], tanh_form);
-                            *reinterpret_cast<uint4 *>(stg + lane * 80 + i * 16) = f32_to_bf16x8(gv);
-                        }
-                        store_rows(args.D2 + gofs2 + c * 32, nvalid);
-                    }
+                        for (int i = 0; i < 4; ++i)
+                            *reinterpret_cast<uint4 *>(stg + lane * 80 + i * 16) =
+                                make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+                        store_rows(out == 0 ? args.D + gofs + c * 32 : args.D2 + gofs2 + c * 32, nvalid);
+                    });
                 }
                 if (EPI == EPI_DGELU) {
 #pragma unroll
