@@ -2,16 +2,18 @@
 // sm_103a tensor cores (tcgen05 + TMEM + TMA), one persistent launch over all
 // T*E (task, expert) groups of the merged expert pool.
 //
-// Structure (one CTA per SM, 320 threads):
-//   warp 0      TMA producer: one thread streams 128x64 A tiles and 64xBN B
-//               tiles into a STAGES-deep ring of shared-memory slots
-//               (128-byte swizzle), signalling `full[s]` with the byte count.
+// Structure (one CTA per SM, 352 threads; 608 for the two-output epilogues):
+//   warp 0 and the last warp
+//               TMA producers: one thread streams 128x64 A tiles, another
+//               64xBN B tiles, into a STAGES-deep ring of shared-memory slots
+//               (128-byte swizzle), each signalling `full[s]` with its byte count.
 //   warp 1      MMA issuer: one thread issues tcgen05.mma (M=128, N=BN,
 //               K=16, bf16 in, fp32 accumulate in TMEM), commits each slot
 //               back to `empty[s]` and each finished tile to `tmem_full[a]`.
 //               The whole warp zeroes the K-tail rows of weight-gradient tiles.
-//   warps 2-9   epilogue: tcgen05.ld of the accumulator (one TMEM lane per
-//               thread = one output row; two warps per lane quarter split the
+//   warps 2-9 (2-17)
+//               epilogue: tcgen05.ld of the accumulator (one TMEM lane per
+//               thread = one output row; the warps of a lane quarter split the
 //               columns), the fused elementwise step (GELU, or GELU' of an H
 //               prefetched into registers one chunk ahead), bf16 packing, a
 //               per-warp staging tile in shared memory and coalesced 16-byte
@@ -42,7 +44,7 @@ namespace tc {
 
 constexpr int BM = 128;  // rows of one MMA tile (TMEM lanes)
 constexpr int BK = 64;   // K per pipeline slot = one 128-byte swizzle row of bf16
-constexpr int THREADS = 320;  // warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
+constexpr int THREADS = 320;  // resident-B and SM-pair kernels: warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
 constexpr int EPI_WARP_BYTES = 32 * 80;  // 32 rows x (64 data + 16 pad) bytes
 
 // Row-mode epilogue of the one-SM grouped GEMM: the two-output epilogues
@@ -66,7 +68,7 @@ constexpr int ROW_CH = 32;
 template <int MODE, int EPI>
 struct Roles {
     static constexpr int EW = (MODE == 0 && EPI != EPI_STORE) ? 16 : 8;  // epilogue warps
-    static constexpr int NT = 64 + 32 * EW;  // threads: producer, MMA, epilogue
+    static constexpr int NT = 96 + 32 * EW;  // threads: A producer, MMA, epilogue, B producer
     static constexpr int PITCH = 80;         // staging row pitch (bytes): 64 data + 16 pad
 };
 
@@ -181,11 +183,12 @@ __device__ __forceinline__ unsigned long long global_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-// Bounded wait for the phase of parity `parity` of barrier `bar`.
-static __device__ __noinline__ bool wait_phase(uint32_t bar, uint32_t parity, volatile int *abort_flag,
-                                               int *status,
-                                               unsigned long long limit_ns = TIMEOUT_NS) {
-    if (mbar_try_wait(bar, parity)) return true;
+// Bounded wait for the phase of parity `parity` of barrier `bar`.  The first
+// test is inline: a call for every k-block cost a producer 120 of its 540
+// cycles (measured on a loop of 16 KB copies), which is what bounds the GEMMs of
+// layers that stay in L2.
+static __device__ __noinline__ bool wait_phase_slow(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                                    int *status, unsigned long long limit_ns) {
     const unsigned long long t0 = global_ns();
     for (uint32_t i = 1;; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
@@ -198,6 +201,10 @@ static __device__ __noinline__ bool wait_phase(uint32_t bar, uint32_t parity, vo
             }
         }
     }
+}
+__device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status,
+                                           unsigned long long limit_ns = TIMEOUT_NS) {
+    return mbar_try_wait(bar, parity) || wait_phase_slow(bar, parity, abort_flag, status, limit_ns);
 }
 __device__ __forceinline__ void fence_barrier_init() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -321,6 +328,11 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr, uint32_t lbo, ui
 __device__ __forceinline__ uint64_t operand_desc(uint32_t tile, int kk, bool mn_major) {
     return mn_major ? sdesc_sw128(tile + kk * 2048, 8192, 1024)
                     : sdesc_sw128(tile + kk * 32, 16, 1024);
+}
+// The descriptor kk K-steps of 16 on (the address field counts 16 bytes and does
+// not overflow: shared memory ends below 2^18).
+__device__ __forceinline__ uint64_t desc_step(uint64_t d, int kk, bool mn_major) {
+    return d + (uint64_t)(kk * ((mn_major ? 2048 : 32) >> 4));
 }
 // MN-major k-block of `rows` K rows: its MN chunks are rows x 128 bytes apart.
 __device__ __forceinline__ uint64_t operand_desc_mn(uint32_t tile, int kk, int rows) {
@@ -447,7 +459,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(bar_full(s), 1);
+            mbar_init(bar_full(s), 2);  // the A and the B producer's arrivals
             mbar_init(bar_empty(s), 1);
         }
         for (int a = 0; a < 2; ++a) {
@@ -521,18 +533,27 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     total = (MODE == MODE_ROW) ? misc[2] : args.G * args.tiles_m * args.tiles_n;
     const uint32_t tmem_base = (uint32_t)misc[0];
 
-    if (warp == 0) {
-        // ------------------------------------------------------------ producer
+    if (warp == 0 || warp == Roles<MODE, EPI>::EW + 2) {
+        // ------------------------------------------------------------ producers: A (warp 0), B (the last warp)
+        // One thread each: a copy's wait, expected bytes and issue take it a few
+        // hundred cycles, as long as the MMAs of a k-block, so A and B have their own.
         if (lane == 0) {
+            const bool isA = warp == 0;
             int stage = 0;
             uint32_t phase = 0;
-            int issued[STAGES];
-#pragma unroll
-            for (int s = 0; s < STAGES; ++s) issued[s] = 0;
+            int issued = 0;  // copies so far: slot s has had those of index s, s + STAGES, ...
             bool ok = true;
+            const bool cmpa = (args.compact & CMP_A) != 0, cmpb = (args.compact & CMP_B) != 0;
             for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
                 const Tile t = decode_tile<MODE>(args, prefix, u);
-                if (u + (int)gridDim.x >= total) pdl_launch_dependents();  // this CTA's last tile
+                if (isA && u + (int)gridDim.x >= total) pdl_launch_dependents();  // this CTA's last tile
+                // Row mode, A rows [0, rn): the tile's valid rows rounded up to 16.  The
+                // slot's rows past rn keep stale data, which only reaches output rows
+                // past rows_valid -- never stored.
+                const int rem_rows = t.rows_valid - t.m_blk * BM;
+                const int rn = MODE != MODE_ROW || rem_rows >= BM ? BM : ((rem_rows + 15) & ~15);
+                const int r0 = (cmpa ? t.crow : 0) + t.m_blk * BM, gz = cmpa ? 0 : t.gr;
+                const uint32_t bytes = isA ? (uint32_t)rn * (BK * 2) : S::B_BYTES;
                 for (int kb = 0; kb < t.kblocks; ++kb) {
                     if (!wait_phase(bar_empty(stage), phase ^ 1u, abort_flag, args.status)) {
                         ok = false;
@@ -541,30 +562,25 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     const uint32_t sa = tiles_addr + stage * S::STAGE_BYTES;
                     const uint32_t sb = sa + S::A_BYTES;
                     const uint32_t fb = bar_full(stage);
+                    mbar_expect_tx(fb, bytes);
                     if (MODE == MODE_ROW) {
-                        // A rows [0, rn): the tile's valid rows rounded up to 16.  The
-                        // slot's rows past rn keep stale data, which only reaches
-                        // output rows past rows_valid -- never stored.
-                        const int rem_rows = t.rows_valid - t.m_blk * BM;
-                        const int rn = rem_rows >= BM ? BM : ((rem_rows + 15) & ~15);
-                        const bool cmpa = (args.compact & CMP_A) != 0;
-                        const int r0 = (cmpa ? t.crow : 0) + t.m_blk * BM, gz = cmpa ? 0 : t.gr;
-                        mbar_expect_tx(fb, (uint32_t)rn * (BK * 2) + S::B_BYTES);
-                        if (rn == BM) {
-                            tma_load_3d(sa, &tmA, fb, kb * BK, r0, gz);
-                        } else {
-                            int off = 0;
-                            if (rn & 64) {
-                                tma_load_3d(sa, &tmAt.a[0], fb, kb * BK, r0, gz);
-                                off = 64;
+                        if (isA) {
+                            if (rn == BM) {
+                                tma_load_3d(sa, &tmA, fb, kb * BK, r0, gz);
+                            } else {
+                                int off = 0;
+                                if (rn & 64) {
+                                    tma_load_3d(sa, &tmAt.a[0], fb, kb * BK, r0, gz);
+                                    off = 64;
+                                }
+                                if (rn & 32) {
+                                    tma_load_3d(sa + off * (BK * 2), &tmAt.a[1], fb, kb * BK, r0 + off, gz);
+                                    off += 32;
+                                }
+                                if (rn & 16)
+                                    tma_load_3d(sa + off * (BK * 2), &tmAt.a[2], fb, kb * BK, r0 + off, gz);
                             }
-                            if (rn & 32) {
-                                tma_load_3d(sa + off * (BK * 2), &tmAt.a[1], fb, kb * BK, r0 + off, gz);
-                                off += 32;
-                            }
-                            if (rn & 16) tma_load_3d(sa + off * (BK * 2), &tmAt.a[2], fb, kb * BK, r0 + off, gz);
-                        }
-                        if (B_MN) {  // one 4-D box: BN/64 column chunks of 64 rows
+                        } else if (B_MN) {  // one 4-D box: BN/64 column chunks of 64 rows
                             tma_load_4d(sb, &tmB, fb, 0, kb * BK, t.n_blk * (BN / 64), t.gr);
                         } else {
                             tma_load_3d(sb, &tmB, fb, kb * BK, t.n_blk * BN, t.gr);
@@ -575,18 +591,16 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         // rows, which start at row C of the group.
                         // (Tail-sized boxes for the last k-block, as in the resident-B
                         // kernel, made this streaming kernel slower: full boxes here.)
-                        mbar_expect_tx(fb, S::STAGE_BYTES);
                         const int hi = (kb >= t.khalf) ? 1 : 0;
                         const int ka = (kb - hi * t.khalf) * BK;
-                        const int kbr = hi * args.C + ka;
-                        tma_load_4d(sa, &tmA, fb, 0, ka, t.m_blk * (BM / 64), t.gr);
-                        if (args.compact & CMP_B)  // residual rows follow the entry's load rows
-                            tma_load_4d(sb, &tmB, fb, 0, t.crow + hi * t.kvalid + ka,
-                                        t.n_blk * (BN / 64), 0);
+                        if (isA)
+                            tma_load_4d(sa, &tmA, fb, 0, ka, t.m_blk * (BM / 64), t.gr);
+                        else if (cmpb)  // residual rows follow the entry's load rows
+                            tma_load_4d(sb, &tmB, fb, 0, t.crow + hi * t.kvalid + ka, t.n_blk * (BN / 64), 0);
                         else
-                            tma_load_4d(sb, &tmB, fb, 0, kbr, t.n_blk * (BN / 64), t.gr);
+                            tma_load_4d(sb, &tmB, fb, 0, hi * args.C + ka, t.n_blk * (BN / 64), t.gr);
                     }
-                    issued[stage]++;
+                    ++issued;
                     if (++stage == STAGES) {
                         stage = 0;
                         phase ^= 1u;
@@ -595,13 +609,11 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
             if (*abort_flag) {  // let copies in flight land before the CTA exits
                 int dummy = 0;
-                for (int s = 0; s < STAGES; ++s)
-                    if (issued[s] > 0) {
-                        const unsigned long long t0 = global_ns();
-                        while (!mbar_try_wait(bar_full(s), (uint32_t)((issued[s] - 1) & 1)) &&
-                               global_ns() - t0 < 100000000ull)
-                            ++dummy;
-                    }
+                for (int s = 0; s < STAGES && s < issued; ++s) {
+                    const uint32_t last = (uint32_t)(((issued - 1 - s) / STAGES) & 1);
+                    const unsigned long long t0 = global_ns();
+                    while (!mbar_try_wait(bar_full(s), last) && global_ns() - t0 < 100000000ull) ++dummy;
+                }
             }
         }
         __syncwarp();
@@ -611,7 +623,31 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         uint32_t phase = 0;
         int it = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < total && ok; u += gridDim.x, ++it) {
+        for (int u = blockIdx.x; MODE == MODE_ROW && lane == 0 && u < total && ok; u += gridDim.x, ++it) {
+            const int acc = it & 1;
+            if (!wait_phase(bar_tempty(acc), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag, args.status)) break;
+            tc_fence_after();
+            const uint32_t dtmem = tmem_base + (uint32_t)(acc * BN);
+            for (int kb = 0; kb < args.K_fixed / BK; ++kb) {
+                if (!wait_phase(bar_full(stage), phase, abort_flag, args.status)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t sa = tiles_addr + stage * S::STAGE_BYTES;
+                const uint64_t da = operand_desc(sa, 0, A_MN), db = operand_desc(sa + S::A_BYTES, 0, B_MN);
+#pragma unroll
+                for (int kk = 0; kk < BK / 16; ++kk)
+                    mma_bf16(dtmem, desc_step(da, kk, A_MN), desc_step(db, kk, B_MN), IDESC, (kb | kk) != 0 ? 1u : 0u);
+                mma_commit(bar_empty(stage));
+                if (++stage == STAGES) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
+            }
+            if (ok) mma_commit(bar_tfull(acc));
+        }
+        for (int u = blockIdx.x; MODE == MODE_WGRAD && u < total && ok; u += gridDim.x, ++it) {
             const Tile t = decode_tile<MODE>(args, prefix, u);
             const int acc = it & 1;
             const uint32_t aph = (uint32_t)((it >> 1) & 1);
@@ -632,7 +668,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 const uint32_t sa = tiles_addr + stage * S::STAGE_BYTES;
                 const uint32_t sb = sa + S::A_BYTES;
                 int nk = BK / 16;
-                if (MODE == MODE_WGRAD && (kb == t.kblocks - 1 || kb == t.khalf - 1)) {
+                if ((kb == t.kblocks - 1 || kb == t.khalf - 1)) {
                     // K tail: the MMA reads rows [0, 16*nk) of the slot; rows
                     // [rem, 16*nk) lie past this group's load and are zeroed in
                     // both operands (one 128-byte line per K row per 64-wide chunk).
@@ -658,8 +694,9 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     __syncwarp();
                 }
                 if (lane == 0) {
+                    const uint64_t da = operand_desc(sa, 0, A_MN), db = operand_desc(sb, 0, B_MN);
                     for (int kk = 0; kk < nk; ++kk)
-                        mma_bf16(dtmem, operand_desc(sa, kk, A_MN), operand_desc(sb, kk, B_MN), IDESC,
+                        mma_bf16(dtmem, desc_step(da, kk, A_MN), desc_step(db, kk, B_MN), IDESC,
                                  (kb | kk) != 0 ? 1u : 0u);
                     mma_commit(bar_empty(stage));
                 }

@@ -17,8 +17,9 @@
 // KSPLIT the residual rows after them -- is loaded once and reused by all M/256
 // row tiles of the group; their A k-blocks stream through a ring.
 //
-// Roles, per CTA (320 threads):
-//   warp 0      TMA producer: its own A and B halves into its own shared memory.
+// Roles, per CTA (352 threads):
+//   warps 0, 10 TMA producers of A (0) and B (10): the CTA's own halves into its
+//               own shared memory.
 //               A k-blocks complete on the leader's `afull` (both CTAs' bytes).
 //               With two B buffers a B tile completes on this CTA's own `bfull`;
 //               with one (K > 128 rows) each k-block piece of a dense B tile
@@ -75,7 +76,6 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
 // Bounded wait with acquire at cluster scope (barriers the peer CTA arrives on).
 static __device__ __noinline__ bool wait_phase_cluster(uint32_t bar, uint32_t parity,
                                                        volatile int *abort_flag, int *status) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
     const unsigned long long t0 = global_ns();
     for (uint32_t i = 1;; ++i) {
         if (mbar_try_wait_cluster(bar, parity)) return true;
@@ -148,6 +148,8 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
+constexpr int PAIR_THREADS = THREADS + 32;  // wgrad_pair_kernel: + the B producer
+
 // Shared memory of the pair kernel, per CTA.  KB = one k-block (64 K rows) of
 // 128 columns = 16 KB, for A and B alike.  The B region holds one or two
 // resident B tiles (NKB k-blocks, twice with KSPLIT); what is left of a 224 KB
@@ -202,7 +204,7 @@ struct PairSchedule {
 // (In the memory-budgeted backward B comes from a compact buffer, where the
 // rows before an entry belong to its neighbour: the tail warp zeroes them.)
 template <bool KSPLIT, int NKB>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(PAIR_THREADS, 1)
 wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const __grid_constant__ CUtensorMap tmBlo, const __grid_constant__ CUtensorMap tmD,
                   Args args, const __grid_constant__ PairSchedule sched) {
@@ -298,16 +300,55 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     };
 
     if (warp == 0) {
-        // ------------------------------------------------------------ producer
+        // ------------------------------------------------------------ A producer
         if (lane == 0) {
-            int ub = 0, ka = 0;
+            int sl = 0, issued = 0;  // slot s has had copies s, s + AS, ...
+            uint32_t phase = 0;
             bool ok = true;
-            // uses of each B piece so far (their parity gives the phase)
-            int b_issued[BP] = {}, a_issued[AS] = {};
             for (int u = u_first; u < u_end && ok; u += u_step) {
                 int g, n_blk, L;
                 decode(u, g, n_blk, L);
                 if (u + u_step >= u_end) pdl_launch_dependents();  // this pair's last unit
+                const int nkb = (L + BK - 1) / BK;
+                const int r0 = L - nkb * BK;  // first row of k-block 0 (<= 0)
+                for (int m = 0; m < tiles_m && ok; ++m)
+                    for (int kb = 0; kb < nkb; ++kb, ++issued) {
+                        if (!wait_phase(bar_aempty(sl), phase ^ 1u, abort_flag, args.status)) {
+                            ok = false;
+                            break;
+                        }
+                        if (leader) mbar_expect_tx(bar_afull(sl), 2u * S::KB);  // both CTAs' halves
+                        tma_load_4d_pair(smem_u32(a_ring) + sl * S::KB, &tmA, mapa_shared(bar_afull(sl), 0),
+                                         0, r0 + kb * BK, m * 4 + (int)rank * 2, g);
+                        if (++sl == AS) {
+                            sl = 0;
+                            phase ^= 1u;
+                        }
+                    }
+            }
+            // let copies in flight land before the CTA exits; the leader's afull
+            // counts the peer's copies too, and the peer waits for the leader at
+            // the closing cluster barrier
+            if (*abort_flag && leader) {
+                const unsigned long long t0 = global_ns();
+                for (int i = 0; i < AS && i < issued; ++i)
+                    while (!mbar_try_wait(bar_afull(i), (uint32_t)(((issued - 1 - i) / AS) & 1)) &&
+                           global_ns() - t0 < 200000000ull) {
+                    }
+            }
+        }
+        __syncwarp();
+        give_up();
+    } else if (warp == THREADS / 32) {
+        // ------------------------------------------------------------ B producer
+        if (lane == 0) {
+            int ub = 0;
+            bool ok = true;
+            // per B piece: parity of its uses so far (which gives the phase), and whether it has been used
+            uint32_t b_par = 0, b_any = 0;
+            for (int u = u_first; u < u_end && ok; u += u_step) {
+                int g, n_blk, L;
+                decode(u, g, n_blk, L);
                 const int nkb = (L + BK - 1) / BK;
                 if (nkb == 0) continue;
                 const int r0 = L - nkb * BK;  // first row of k-block 0 (<= 0)
@@ -318,10 +359,11 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 // B piece pc = k-blocks [kb0, kb1) (and their residual), once its
                 // previous use has been released by the MMAs
                 auto load_b = [&](int pc, int kb0, int kb1) -> bool {
-                    int &nb = b_issued[bb * NPC + pc];
-                    if (!wait_phase(bar_bempty(bb, pc), (uint32_t)(nb & 1) ^ 1u, abort_flag, args.status))
+                    const uint32_t bit = 1u << (bb * NPC + pc);
+                    if (!wait_phase(bar_bempty(bb, pc), (b_par & bit) ? 0u : 1u, abort_flag, args.status))
                         return false;
-                    ++nb;
+                    b_par ^= bit;
+                    b_any |= bit;
                     const uint32_t fb = bar_bfull(bb, pc);
                     const uint32_t bytes = (KSPLIT ? 2u : 1u) * (uint32_t)(kb1 - kb0) * S::KB;
                     const bool on_leader = PIECES && !cmpb;
@@ -348,52 +390,28 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     return true;
                 };
                 // Two buffers: the whole tile at once (its buffer was freed a
-                // unit ago).  One: each piece just before the first row tile's
-                // A k-block that needs it.
+                // unit ago).  One: each piece as the last row tile before frees it.
                 if (!PIECES) ok = load_b(0, 0, nkb);
-                for (int m = 0; m < tiles_m && ok; ++m)
-                    for (int kb = 0; kb < nkb; ++kb, ++ka) {
-                        if (PIECES && m == 0 && !load_b(kb, kb, kb + 1)) {
-                            ok = false;
-                            break;
-                        }
-                        const int sl = ka % AS;
-                        if (!wait_phase(bar_aempty(sl), (uint32_t)((ka / AS) & 1) ^ 1u, abort_flag,
-                                        args.status)) {
-                            ok = false;
-                            break;
-                        }
-                        if (leader) mbar_expect_tx(bar_afull(sl), 2u * S::KB);  // both CTAs' halves
-                        tma_load_4d_pair(smem_u32(a_ring) + sl * S::KB, &tmA, mapa_shared(bar_afull(sl), 0),
-                                         0, r0 + kb * BK, m * 4 + (int)rank * 2, g);
-                        ++a_issued[sl];
-                    }
+                for (int kb = 0; PIECES && kb < nkb && ok; ++kb) ok = load_b(kb, kb, kb + 1);
             }
-            if (*abort_flag) {  // let copies in flight land before the CTA exits
+            // let copies in flight land before the CTA exits (dense B pieces, like
+            // A, complete on the leader's barriers)
+            if (*abort_flag && (leader || !PIECES || cmpb)) {
                 const unsigned long long t0 = global_ns();
-                // (dense B pieces, like A, complete on the leader's barriers)
-                if (leader || !PIECES || cmpb)
-                    for (int i = 0; i < BP; ++i)
-                        if (b_issued[i] > 0)
-                            while (!mbar_try_wait(bar_bfull(i / NPC, i % NPC), (uint32_t)((b_issued[i] - 1) & 1)) &&
-                                   global_ns() - t0 < 100000000ull) {
-                            }
-                // the leader's afull counts the peer's copies too; the peer waits
-                // for the leader at the closing cluster barrier
-                if (leader)
-                    for (int i = 0; i < AS; ++i)
-                        if (a_issued[i] > 0)
-                            while (!mbar_try_wait(bar_afull(i), (uint32_t)((a_issued[i] - 1) & 1)) &&
-                                   global_ns() - t0 < 200000000ull) {
-                            }
+                for (int i = 0; i < BP; ++i)
+                    if ((b_any >> i) & 1u)
+                        while (!mbar_try_wait(bar_bfull(i / NPC, i % NPC), (b_par >> i) & 1u ? 0u : 1u) &&
+                               global_ns() - t0 < 100000000ull) {
+                        }
             }
         }
         __syncwarp();
         give_up();
     } else if (warp == 1) {
         // ------------------------------------------------------------ B hand-over (+ MMA in the leader)
-        int ub = 0, ka = 0, it = 0;
-        int b_used[BP] = {};  // uses of each B piece so far (their parity gives the phase)
+        int ub = 0, sl = 0, it = 0;
+        uint32_t aph = 0;    // phase of A slot sl
+        uint32_t b_par = 0;  // per B piece, the parity of its uses so far: the phase
         bool ok = true;
         for (int u = u_first; u < u_end && ok; u += u_step) {
             int g, n_blk, L;
@@ -409,8 +427,8 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             // compact-B rows of k-block 0 that belong to a neighbour, hand it
             // to the leader; the leader waits until both CTAs have.
             auto hand_over = [&](int pc) -> bool {
-                const uint32_t ph = (uint32_t)(b_used[bb * NPC + pc] & 1);
-                ++b_used[bb * NPC + pc];
+                const uint32_t ph = (b_par >> (bb * NPC + pc)) & 1u;
+                b_par ^= 1u << (bb * NPC + pc);
                 if (!wait_phase(bar_bfull(bb, pc), ph, abort_flag, args.status)) return false;
                 if (cmpb && pc == 0 && z > 0) {
                     // compact B: rows [0, z) of k-block 0 (both parts) hold the
@@ -427,7 +445,8 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(mapa_shared(bar_bready(bb, pc), 0));
-                return !leader || wait_phase_cluster(bar_bready(bb, pc), ph, abort_flag, args.status);
+                return !leader || mbar_try_wait_cluster(bar_bready(bb, pc), ph) ||
+                       wait_phase_cluster(bar_bready(bb, pc), ph, abort_flag, args.status);
             };
             if (!PIECES || cmpb)
                 for (int pc = 0; pc < (PIECES ? nkb : 1) && ok; ++pc) ok = hand_over(pc);
@@ -440,17 +459,16 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     break;
                 }
                 tc_fence_after();
-                for (int kb = 0; kb < nkb; ++kb, ++ka) {
+                for (int kb = 0; kb < nkb; ++kb) {
                     if (PIECES && !cmpb && m == 0) {  // dense B piece kb: both halves landed
-                        const uint32_t ph = (uint32_t)(b_used[bb * NPC + kb] & 1);
-                        ++b_used[bb * NPC + kb];
+                        const uint32_t ph = (b_par >> (bb * NPC + kb)) & 1u;
+                        b_par ^= 1u << (bb * NPC + kb);
                         if (!wait_phase(bar_bfull(bb, kb), ph, abort_flag, args.status)) {
                             ok = false;
                             break;
                         }
                     }
-                    const int sl = ka % AS;
-                    if (!wait_phase(bar_afull(sl), (uint32_t)((ka / AS) & 1), abort_flag, args.status)) {
+                    if (!wait_phase(bar_afull(sl), aph, abort_flag, args.status)) {
                         ok = false;
                         break;
                     }
@@ -458,19 +476,22 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     if (lane == 0) {
                         const int k0 = kb == 0 ? skip : 0;
                         const uint32_t dtmem = tmem_base + (uint32_t)(acc * S::BN);
-                        const uint32_t a0 = smem_u32(a_ring) + sl * S::KB;
-#pragma unroll 1
+                        const uint64_t da = operand_desc(smem_u32(a_ring) + sl * S::KB, 0, true);
                         for (int part = 0; part < (KSPLIT ? 2 : 1); ++part) {
-                            const uint32_t b0 = smem_u32(bres) + (part * NKB + kb) * S::KB;
+                            const uint64_t db = operand_desc(smem_u32(bres) + (part * NKB + kb) * S::KB, 0, true);
                             for (int kk = k0; kk < BK / 16; ++kk)
-                                mma_pair_bf16(dtmem, operand_desc(a0, kk, true), operand_desc(b0, kk, true),
-                                              IDESC, (kb | part | (kk - k0)) != 0 ? 1u : 0u);
+                                mma_pair_bf16(dtmem, desc_step(da, kk, true), desc_step(db, kk, true), IDESC,
+                                              (kb | part | (kk - k0)) != 0 ? 1u : 0u);
                         }
                         mma_pair_commit_both(bar_aempty(sl));
                         // the last row tile's MMAs on a piece are its last use
                         if (PIECES && last_m) mma_pair_commit_both(bar_bempty(bb, kb));
                     }
                     __syncwarp();
+                    if (++sl == AS) {
+                        sl = 0;
+                        aph ^= 1u;
+                    }
                 }
                 if (!ok) break;
                 if (lane == 0) mma_pair_commit_both(bar_tfull(acc));
@@ -746,9 +767,7 @@ row_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
-            int issued[STAGES];
-#pragma unroll
-            for (int s = 0; s < STAGES; ++s) issued[s] = 0;
+            int issued = 0;
             bool ok = true;
             const bool cmpa = (args.compact & CMP_A) != 0;
             for (int u = cid; u < total && ok; u += ncl) {
@@ -789,7 +808,7 @@ row_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         tma_load_4d_pair(sb, &tmB, fb, 0, kb * BK, n_blk * (BN / 64) + (int)rank * (BNC / 64), gr);
                     else
                         tma_load_3d_pair(sb, &tmB, fb, kb * BK, n_blk * BN + (int)rank * BNC, gr);
-                    issued[stage]++;
+                    ++issued;
                     if (++stage == STAGES) {
                         stage = 0;
                         phase ^= 1u;
@@ -798,11 +817,10 @@ row_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             }
             if (*abort_flag && leader) {  // copies in flight (both CTAs') land before the pair exits
                 const unsigned long long t0 = global_ns();
-                for (int s = 0; s < STAGES; ++s)
-                    if (issued[s] > 0)
-                        while (!mbar_try_wait(bar_full(s), (uint32_t)((issued[s] - 1) & 1)) &&
-                               global_ns() - t0 < 200000000ull) {
-                        }
+                for (int s = 0; s < STAGES && s < issued; ++s)
+                    while (!mbar_try_wait(bar_full(s), (uint32_t)(((issued - 1 - s) / STAGES) & 1)) &&
+                           global_ns() - t0 < 200000000ull) {
+                    }
             }
         }
         __syncwarp();
@@ -987,7 +1005,7 @@ int launch_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap 
     if (clusters <= 0) return VMOE_OK;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * clusters));
-    cfg.blockDim = dim3(THREADS);
+    cfg.blockDim = dim3(PAIR_THREADS);
     cfg.dynamicSmemBytes = S::SMEM_BYTES;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];

@@ -27,7 +27,7 @@ int pair_clusters(const void *kern, size_t smem) {
         if (e.kern.load(std::memory_order_acquire) == kern) return e.n.load(std::memory_order_relaxed);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)num_sms());
-    cfg.blockDim = dim3(THREADS);
+    cfg.blockDim = dim3(PAIR_THREADS);  // the larger of the pair kernels: one CTA an SM either way
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
