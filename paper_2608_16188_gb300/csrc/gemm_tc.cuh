@@ -10,7 +10,6 @@
 //   warp 1      MMA issuer: one thread issues tcgen05.mma (M=128, N=BN,
 //               K=16, bf16 in, fp32 accumulate in TMEM), commits each slot
 //               back to `empty[s]` and each finished tile to `tmem_full[a]`.
-//               The whole warp zeroes the K-tail rows of weight-gradient tiles.
 //   warps 2-9 (2-17)
 //               epilogue: tcgen05.ld of the accumulator (one TMEM lane per
 //               thread = one output row; the warps of a lane quarter split the
@@ -206,6 +205,19 @@ __device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volati
                                            unsigned long long limit_ns = TIMEOUT_NS) {
     return mbar_try_wait(bar, parity) || wait_phase_slow(bar, parity, abort_flag, status, limit_ns);
 }
+// One lane of a converged warp, the same one every time.  The compiler takes
+// the branch as run by one thread, which a test of the lane index does not tell
+// it: a k-block of four 128 x 128 MMAs with its wait and commit then issues in
+// 310 cycles instead of 427 (of 128 x 64: 238 instead of 347).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void fence_barrier_init() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -370,6 +382,7 @@ __device__ __forceinline__ Tile decode_tile(const Args &a, const int *prefix, in
         t.m_blk = local / a.tiles_n;
         t.n_blk = local - t.m_blk * a.tiles_n;
         t.kblocks = a.K_fixed / BK;
+        t.khalf = t.kblocks;
         t.kvalid = a.K_fixed;
         int L = __ldg(a.load + t.gr);
         t.rows_valid = L < 0 ? 0 : (L > a.C ? a.C : L);
@@ -537,16 +550,18 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // ------------------------------------------------------------ producers: A (warp 0), B (the last warp)
         // One thread each: a copy's wait, expected bytes and issue take it a few
         // hundred cycles, as long as the MMAs of a k-block, so A and B have their own.
-        if (lane == 0) {
+        if (elect_one()) {
             const bool isA = warp == 0;
             int stage = 0;
             uint32_t phase = 0;
             int issued = 0;  // copies so far: slot s has had those of index s, s + STAGES, ...
             bool ok = true;
             const bool cmpa = (args.compact & CMP_A) != 0, cmpb = (args.compact & CMP_B) != 0;
+            Tile t = decode_tile<MODE>(args, prefix, blockIdx.x < total ? blockIdx.x : 0);
             for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
-                const Tile t = decode_tile<MODE>(args, prefix, u);
-                if (isA && u + (int)gridDim.x >= total) pdl_launch_dependents();  // this CTA's last tile
+                Tile tn = t;  // the next tile, looked up behind this one's first copy
+                const bool last = u + (int)gridDim.x >= total;
+                if (isA && last) pdl_launch_dependents();  // this CTA's last tile
                 // Row mode, A rows [0, rn): the tile's valid rows rounded up to 16.  The
                 // slot's rows past rn keep stale data, which only reaches output rows
                 // past rows_valid -- never stored.
@@ -554,6 +569,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 const int rn = MODE != MODE_ROW || rem_rows >= BM ? BM : ((rem_rows + 15) & ~15);
                 const int r0 = (cmpa ? t.crow : 0) + t.m_blk * BM, gz = cmpa ? 0 : t.gr;
                 const uint32_t bytes = isA ? (uint32_t)rn * (BK * 2) : S::B_BYTES;
+                // Weight gradients: the first K row of k-block 0 (<= 0, see below)
+                const int k0 = t.kvalid - t.khalf * BK;
                 for (int kb = 0; kb < t.kblocks; ++kb) {
                     if (!wait_phase(bar_empty(stage), phase ^ 1u, abort_flag, args.status)) {
                         ok = false;
@@ -586,26 +603,29 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                             tma_load_3d(sb, &tmB, fb, kb * BK, t.n_blk * BN, t.gr);
                         }
                     } else {
-                        // Weight gradients: K = the group's rows.  With ksplit the second
-                        // half of the k-blocks pairs the same A rows with B's residual
-                        // rows, which start at row C of the group.
-                        // (Tail-sized boxes for the last k-block, as in the resident-B
-                        // kernel, made this streaming kernel slower: full boxes here.)
+                        // K = the group's rows, in k-blocks that end at its last row: only
+                        // k-block 0 is partial, and its missing rows lie before row 0, where
+                        // the tensor maps read zeros (in a compact B they are a neighbour's,
+                        // and the MMA warp zeroes them).  With ksplit the second half of the
+                        // k-blocks pairs the same A rows with B's residual rows.
                         const int hi = (kb >= t.khalf) ? 1 : 0;
-                        const int ka = (kb - hi * t.khalf) * BK;
+                        const int ka = k0 + (kb - hi * t.khalf) * BK;
                         if (isA)
                             tma_load_4d(sa, &tmA, fb, 0, ka, t.m_blk * (BM / 64), t.gr);
                         else if (cmpb)  // residual rows follow the entry's load rows
                             tma_load_4d(sb, &tmB, fb, 0, t.crow + hi * t.kvalid + ka, t.n_blk * (BN / 64), 0);
                         else
-                            tma_load_4d(sb, &tmB, fb, 0, hi * args.C + ka, t.n_blk * (BN / 64), t.gr);
+                            tma_load_4d(sb, hi ? &tmD2 : &tmB, fb, 0, ka, t.n_blk * (BN / 64), t.gr);
                     }
+                    if (kb == 0 && !last) tn = decode_tile<MODE>(args, prefix, u + gridDim.x);
                     ++issued;
                     if (++stage == STAGES) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
+                if (t.kblocks == 0 && !last) tn = decode_tile<MODE>(args, prefix, u + gridDim.x);
+                t = tn;
             }
             if (*abort_flag) {  // let copies in flight land before the CTA exits
                 int dummy = 0;
@@ -623,94 +643,88 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         uint32_t phase = 0;
         int it = 0;
         bool ok = true;
-        for (int u = blockIdx.x; MODE == MODE_ROW && lane == 0 && u < total && ok; u += gridDim.x, ++it) {
-            const int acc = it & 1;
-            if (!wait_phase(bar_tempty(acc), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag, args.status)) break;
-            tc_fence_after();
-            const uint32_t dtmem = tmem_base + (uint32_t)(acc * BN);
-            for (int kb = 0; kb < args.K_fixed / BK; ++kb) {
-                if (!wait_phase(bar_full(stage), phase, abort_flag, args.status)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t sa = tiles_addr + stage * S::STAGE_BYTES;
-                const uint64_t da = operand_desc(sa, 0, A_MN), db = operand_desc(sa + S::A_BYTES, 0, B_MN);
+        const bool cmpb = MODE == MODE_WGRAD && (args.compact & CMP_B) != 0;
+        const bool one = elect_one();
+        // Waits for slot `stage` and issues its MMAs from 16-row step k0 on.
+        auto k_block = [&](uint32_t dtmem, int k0, bool accumulate) {
+            const uint32_t sa = tiles_addr + stage * S::STAGE_BYTES;
+            const uint64_t da = operand_desc(sa, 0, A_MN), db = operand_desc(sa + S::A_BYTES, 0, B_MN);
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk)
-                    mma_bf16(dtmem, desc_step(da, kk, A_MN), desc_step(db, kk, B_MN), IDESC, (kb | kk) != 0 ? 1u : 0u);
-                mma_commit(bar_empty(stage));
-                if (++stage == STAGES) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
+            for (int kk = 0; kk < BK / 16; ++kk)
+                if (MODE == MODE_ROW || kk >= k0)
+                    mma_bf16(dtmem, desc_step(da, kk, A_MN), desc_step(db, kk, B_MN), IDESC,
+                             accumulate || kk > k0 ? 1u : 0u);
+            mma_commit(bar_empty(stage));
+        };
+        auto next_stage = [&]() {
+            if (++stage == STAGES) {
+                stage = 0;
+                phase ^= 1u;
             }
-            if (ok) mma_commit(bar_tfull(acc));
-        }
-        for (int u = blockIdx.x; MODE == MODE_WGRAD && u < total && ok; u += gridDim.x, ++it) {
-            const Tile t = decode_tile<MODE>(args, prefix, u);
-            const int acc = it & 1;
-            const uint32_t aph = (uint32_t)((it >> 1) & 1);
-            if (!wait_phase(bar_tempty(acc), aph ^ 1u, abort_flag, args.status)) break;
-            tc_fence_after();
-            const uint32_t dtmem = tmem_base + (uint32_t)(acc * BN);
-            if (t.kblocks == 0) {
-                if (lane == 0) mbar_arrive(bar_tfull(acc));
-                __syncwarp();
-                continue;
-            }
-            for (int kb = 0; kb < t.kblocks; ++kb) {
-                if (!wait_phase(bar_full(stage), phase, abort_flag, args.status)) {
-                    ok = false;
-                    break;
+        };
+        if (!cmpb) {
+            for (int u = blockIdx.x; one && u < total && ok; u += gridDim.x, ++it) {
+                int kblocks = args.K_fixed / BK, khalf = 0, skip = 0;
+                if (MODE == MODE_WGRAD) {
+                    const Tile t = decode_tile<MODE>(args, prefix, u);
+                    kblocks = t.kblocks;
+                    khalf = t.khalf;
+                    skip = (t.khalf * BK - t.kvalid) >> 4;  // all-zero 16-row steps of k-block 0
                 }
+                const int acc = it & 1;
+                if (!wait_phase(bar_tempty(acc), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag, args.status)) break;
                 tc_fence_after();
-                const uint32_t sa = tiles_addr + stage * S::STAGE_BYTES;
-                const uint32_t sb = sa + S::A_BYTES;
-                int nk = BK / 16;
-                if ((kb == t.kblocks - 1 || kb == t.khalf - 1)) {
-                    // K tail: the MMA reads rows [0, 16*nk) of the slot; rows
-                    // [rem, 16*nk) lie past this group's load and are zeroed in
-                    // both operands (one 128-byte line per K row per 64-wide chunk).
-                    const int rem = t.kvalid - (kb - (kb >= t.khalf ? t.khalf : 0)) * BK;
-                    nk = (rem + 15) >> 4;
-                    const int z0 = rem, z1 = nk * 16;
-                    if (z0 < z1) {
-                        const int rows = z1 - z0;
-                        constexpr int CH = BM / 64 + BN / 64;
-                        const int units = CH * rows * 8;
-                        uint8_t *slot_ptr = smem + stage * S::STAGE_BYTES;
-                        for (int i = lane; i < units; i += 32) {
-                            int c = i / (rows * 8);
-                            int w = i - c * rows * 8;
-                            int r = z0 + (w >> 3);
-                            int q = w & 7;
-                            uint8_t *base = (c < BM / 64) ? slot_ptr + c * 8192
-                                                          : slot_ptr + S::A_BYTES + (c - BM / 64) * 8192;
-                            *reinterpret_cast<uint4 *>(base + r * 128 + q * 16) = make_uint4(0, 0, 0, 0);
+                for (int kb = 0; kb < kblocks; ++kb) {
+                    if (!wait_phase(bar_full(stage), phase, abort_flag, args.status)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    k_block(tmem_base + (uint32_t)(acc * BN), kb == 0 || kb == khalf ? skip : 0, kb > 0);
+                    next_stage();
+                }
+                if (!ok) break;
+                if (kblocks == 0) mbar_arrive(bar_tfull(acc));
+                else mma_commit(bar_tfull(acc));
+            }
+        } else {  // compact B: the warp zeroes the rows of k-block 0 (both parts) that belong to a neighbour
+            for (int u = blockIdx.x; u < total && ok; u += gridDim.x, ++it) {
+                const Tile t = decode_tile<MODE>(args, prefix, u);
+                const int z = t.khalf * BK - t.kvalid;
+                const int acc = it & 1;
+                if (!wait_phase(bar_tempty(acc), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag, args.status)) break;
+                tc_fence_after();
+                for (int kb = 0; kb < t.kblocks; ++kb) {
+                    if (!wait_phase(bar_full(stage), phase, abort_flag, args.status)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const bool first = kb == 0 || kb == t.khalf;
+                    if (first && z > 0) {
+                        uint8_t *tile = smem + stage * S::STAGE_BYTES + S::A_BYTES;
+                        for (int i = lane; i < (BN / 64) * z * 8; i += 32) {
+                            const int c = i / (z * 8), w = i - c * z * 8;
+                            *reinterpret_cast<uint4 *>(tile + c * (BK * 128) + (w >> 3) * 128 + (w & 7) * 16) =
+                                make_uint4(0, 0, 0, 0);
                         }
                         fence_proxy_async();
                     }
                     __syncwarp();
+                    if (one) k_block(tmem_base + (uint32_t)(acc * BN), first ? z >> 4 : 0, kb > 0);
+                    __syncwarp();
+                    next_stage();
                 }
-                if (lane == 0) {
-                    const uint64_t da = operand_desc(sa, 0, A_MN), db = operand_desc(sb, 0, B_MN);
-                    for (int kk = 0; kk < nk; ++kk)
-                        mma_bf16(dtmem, desc_step(da, kk, A_MN), desc_step(db, kk, B_MN), IDESC,
-                                 (kb | kk) != 0 ? 1u : 0u);
-                    mma_commit(bar_empty(stage));
+                if (!ok) break;
+                if (one) {
+                    if (t.kblocks == 0) mbar_arrive(bar_tfull(acc));
+                    else mma_commit(bar_tfull(acc));
                 }
                 __syncwarp();
-                if (++stage == STAGES) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
             }
-            if (!ok) break;
-            if (lane == 0) mma_commit(bar_tfull(acc));
-            __syncwarp();
         }
-        if (lane == 0) {  // all MMAs of this CTA complete before TMEM is freed
+        __syncwarp();
+        if (one) {  // all MMAs of this CTA complete before TMEM is freed
             mma_commit(bar_drain);
             const unsigned long long t0 = global_ns();
             while (!mbar_try_wait(bar_drain, 0) && global_ns() - t0 < 1000000000ull) {

@@ -301,7 +301,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
     if (warp == 0) {
         // ------------------------------------------------------------ A producer
-        if (lane == 0) {
+        if (elect_one()) {
             int sl = 0, issued = 0;  // slot s has had copies s, s + AS, ...
             uint32_t phase = 0;
             bool ok = true;
@@ -341,7 +341,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         give_up();
     } else if (warp == THREADS / 32) {
         // ------------------------------------------------------------ B producer
-        if (lane == 0) {
+        if (elect_one()) {
             int ub = 0;
             bool ok = true;
             // per B piece: parity of its uses so far (which gives the phase), and whether it has been used
@@ -411,6 +411,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         // ------------------------------------------------------------ B hand-over (+ MMA in the leader)
         int ub = 0, sl = 0, it = 0;
         uint32_t aph = 0;    // phase of A slot sl
+        const bool one = elect_one();
         uint32_t b_par = 0;  // per B piece, the parity of its uses so far: the phase
         bool ok = true;
         for (int u = u_first; u < u_end && ok; u += u_step) {
@@ -473,7 +474,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                         break;
                     }
                     tc_fence_after();
-                    if (lane == 0) {
+                    if (one) {
                         const int k0 = kb == 0 ? skip : 0;
                         const uint32_t dtmem = tmem_base + (uint32_t)(acc * S::BN);
                         const uint64_t da = operand_desc(smem_u32(a_ring) + sl * S::KB, 0, true);
@@ -494,14 +495,14 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     }
                 }
                 if (!ok) break;
-                if (lane == 0) mma_pair_commit_both(bar_tfull(acc));
+                if (one) mma_pair_commit_both(bar_tfull(acc));
                 __syncwarp();
             }
             if (!ok) break;
-            if (!PIECES && lane == 0) mma_pair_commit_both(bar_bempty(bb, 0));  // B may be replaced now
+            if (!PIECES && one) mma_pair_commit_both(bar_bempty(bb, 0));  // B may be replaced now
             __syncwarp();
         }
-        if (leader && lane == 0) {  // all MMAs of the pair complete before TMEM is freed
+        if (leader && one) {  // all MMAs of the pair complete before TMEM is freed
             mma_pair_commit_local(bar_drain);
             const unsigned long long t0 = global_ns();
             while (!mbar_try_wait(bar_drain, 0) && global_ns() - t0 < 1000000000ull) {
@@ -1209,7 +1210,13 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
                       : launch_pair<false, 4>(ma, mb, mblo, md, a, units, s, name, sched);
     }
     if (!make_map_chunked(&ma, act1, M, C, G, 64, BM / 64)) return VMOE_ERR_CUDA;
-    if (!make_map_chunked(&mb, act2, N, b_rows, b_outer, 64, BN / 64)) return VMOE_ERR_CUDA;
+    // exactly C rows a group, and a map of its own for the residual, so that rows before row 0 read zeros
+    CUtensorMap mblo = {};
+    if (cmpb ? !make_map_chunked(&mb, act2, N, b_rows, 1, 64, BN / 64)
+             : !make_map_chunked(&mb, act2, N, C, G, 64, BN / 64, ksplit ? 2 * (uint64_t)C * N : 0) ||
+                   (ksplit && !make_map_chunked(&mblo, act2 + (size_t)C * N, N, C, G, 64, BN / 64,
+                                                2 * (uint64_t)C * N)))
+        return VMOE_ERR_CUDA;
     a.tiles_n = N / BN;
     a.tiles_m = M / BM;
     // Resident B when every group fits one B tile (C <= 128) but is not tiny: with
@@ -1230,8 +1237,8 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
     }
     long long max_tiles = (long long)a.G * a.tiles_m * a.tiles_n;
     const TailMaps unused{};  // the streaming kernel loads full k-blocks
-    return wide ? launch<256, MODE_WGRAD, true, true, EPI_STORE>(ma, mb, md, md, unused, a, max_tiles, s, name)
-                : launch<128, MODE_WGRAD, true, true, EPI_STORE>(ma, mb, md, md, unused, a, max_tiles, s, name);
+    return wide ? launch<256, MODE_WGRAD, true, true, EPI_STORE>(ma, mb, md, mblo, unused, a, max_tiles, s, name)
+                : launch<128, MODE_WGRAD, true, true, EPI_STORE>(ma, mb, md, mblo, unused, a, max_tiles, s, name);
 }
 
 }  // namespace tc
