@@ -43,7 +43,7 @@ namespace tc {
 
 constexpr int BM = 128;  // rows of one MMA tile (TMEM lanes)
 constexpr int BK = 64;   // K per pipeline slot = one 128-byte swizzle row of bf16
-constexpr int THREADS = 320;  // resident-B and SM-pair kernels: warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
+constexpr int THREADS = 320;  // SM-pair row kernel: warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
 constexpr int EPI_WARP_BYTES = 32 * 80;  // 32 rows x (64 data + 16 pad) bytes
 
 // Row-mode epilogue of the one-SM grouped GEMM: the two-output epilogues
@@ -133,21 +133,13 @@ struct Args {
 };
 enum { CMP_A = 1, CMP_B = 2, CMP_D = 4 };
 
-// Partial-box tensor maps: a group's padding rows [load, C) are not read.
-// Row mode: a[0..2] = the A operand with 64-, 32- and 16-row boxes; a tile
-// whose valid rows end inside it loads rows [0, 16 ceil(rows / 16)) as at most
-// three boxes instead of one 128-row box.
-// Weight gradients, resident-B kernel: a[i], b[i] = the A and B operands with
-// boxes of 16 (i + 1) K rows, for a group's last k-block when its valid rows
-// end inside it.  Such a box lands chunk-major with a chunk stride of
-// (rows x 128) bytes, which the k-block's MMA descriptors take as their
-// leading byte offset.
+// Partial-box tensor maps: a group's padding rows [load, C) are not read.  Row
+// mode: a[0..2] = the A operand with 64-, 32- and 16-row boxes; a tile whose
+// valid rows end inside it loads rows [0, 16 ceil(rows / 16)) as at most three
+// boxes instead of one 128-row box.
 struct TailMaps {
-    CUtensorMap a[3], b[3];
+    CUtensorMap a[3];
 };
-// Rows loaded for a k-block with `rem` valid K rows (>= 1): all BK, or rem
-// rounded up to 16.
-__host__ __device__ __forceinline__ int tail_rows(int rem) { return rem >= 64 ? 64 : ((rem + 15) & ~15); }
 __device__ __forceinline__ int real_group(const Args &a, int i) { return a.glist ? __ldg(a.glist + i) : i; }
 
 // ---------------------------------------------------------------------------
@@ -232,12 +224,21 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
         "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
         : "memory");
 }
+// L2 policy of the weight-gradient stores: first to be evicted.  Nothing reads
+// a gradient again before the step ends, and its lines otherwise push the
+// activations out.  Measured at the 17-task step: dW1 522 -> 506 us, dW2 465 ->
+// 445 us; the attention experts' dW_qkv 375 -> 355 us.
+__device__ __forceinline__ uint64_t evict_first_policy() {
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    return policy;
+}
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, uint32_t src, int c0, int c1,
-                                             int c2) {
+                                             int c2, uint64_t policy) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
+        "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group.L2::cache_hint [%0, {%2, %3, %4}], [%1], %5;" ::"l"(
             reinterpret_cast<uint64_t>(map)),
-        "r"(src), "r"(c0), "r"(c1), "r"(c2)
+        "r"(src), "r"(c0), "r"(c1), "r"(c2), "l"(policy)
         : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
@@ -346,10 +347,6 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t tile, int kk, bool mn_
 __device__ __forceinline__ uint64_t desc_step(uint64_t d, int kk, bool mn_major) {
     return d + (uint64_t)(kk * ((mn_major ? 2048 : 32) >> 4));
 }
-// MN-major k-block of `rows` K rows: its MN chunks are rows x 128 bytes apart.
-__device__ __forceinline__ uint64_t operand_desc_mn(uint32_t tile, int kk, int rows) {
-    return sdesc_sw128(tile + kk * 2048, (uint32_t)rows * 128u, 1024);
-}
 
 // Instruction descriptor of tcgen05.mma kind::f16: D fp32 (bits 4-5 = 1),
 // A and B bf16 (bits 7-9, 10-12 = 1), A / B MN-major (bits 15 / 16),
@@ -442,7 +439,12 @@ __device__ __forceinline__ void epilogue_chunk(f32x2 (&v)[CH / 2], const uint4 *
     }
 }
 
-template <int BN, int MODE, bool A_MN, bool B_MN, int EPI>
+// EAGER: the producers and the MMA thread run as elected threads and look the
+// next tile up early.  The weight gradients of groups of at most 128 rows run
+// better without: they are bound by their stores, and copies issued faster only
+// get in their way (17-task step, dW2 477 us with, 445 without; attention dW_qkv
+// 355 / 326; with C 493, ViT-S, 29.3 / 31.0, and there the operands bound it).
+template <int BN, int MODE, bool A_MN, bool B_MN, int EPI, bool EAGER>
 __global__ void __launch_bounds__(Roles<MODE, EPI>::NT, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmD2,
@@ -550,7 +552,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // ------------------------------------------------------------ producers: A (warp 0), B (the last warp)
         // One thread each: a copy's wait, expected bytes and issue take it a few
         // hundred cycles, as long as the MMAs of a k-block, so A and B have their own.
-        if (elect_one()) {
+        if (EAGER ? elect_one() : lane == 0) {
             const bool isA = warp == 0;
             int stage = 0;
             uint32_t phase = 0;
@@ -617,7 +619,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         else
                             tma_load_4d(sb, hi ? &tmD2 : &tmB, fb, 0, ka, t.n_blk * (BN / 64), t.gr);
                     }
-                    if (kb == 0 && !last) tn = decode_tile<MODE>(args, prefix, u + gridDim.x);
+                    if (kb == (EAGER ? 0 : t.kblocks - 1) && !last) tn = decode_tile<MODE>(args, prefix, u + gridDim.x);
                     ++issued;
                     if (++stage == STAGES) {
                         stage = 0;
@@ -644,7 +646,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         int it = 0;
         bool ok = true;
         const bool cmpb = MODE == MODE_WGRAD && (args.compact & CMP_B) != 0;
-        const bool one = elect_one();
+        const bool one = EAGER ? elect_one() : lane == 0;
         // Waits for slot `stage` and issues its MMAs from 16-row step k0 on.
         auto k_block = [&](uint32_t dtmem, int k0, bool accumulate) {
             const uint32_t sa = tiles_addr + stage * S::STAGE_BYTES;
@@ -742,6 +744,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         const int half = ew >> 2;
         constexpr int COLS = BN / 2;
         uint8_t *stg = epi_base + ew * EPI_WARP_BYTES_TMA;
+        const uint64_t policy = evict_first_policy();
         int nstore = 0;
         int it = 0;
         for (int u = blockIdx.x; u < total; u += gridDim.x, ++it) {
@@ -786,7 +789,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) {
-                    tma_store_3d(&tmD, smem_u32(buf), colw + c * 64, row0, t.gr);
+                    tma_store_3d(&tmD, smem_u32(buf), colw + c * 64, row0, t.gr, policy);
                     bulk_commit();
                 }
                 ++nstore;
@@ -892,6 +895,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     }
                     epilogue_chunk<EPI, CH>(v, hcur, tanh_form, [&](const uint32_t(&w)[CH / 2], int out) {
                         stage(w);
+                        
                         store_rows(out == 0 ? args.D + gofs + c * CH : args.D2 + gofs2 + c * CH, nvalid);
                     });
                 }
@@ -905,357 +909,6 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             if (lane == 0) mbar_arrive(bar_tempty(acc));
             t = tn;
         }
-    }
-
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (warp == 0) tmem_dealloc(tmem_base, S::TMEM_COLS);
-}
-
-// ---------------------------------------------------------------------------
-// Weight gradients with the B operand resident ("B-stationary"), for groups of
-// at most 128 rows (C <= 128).
-//
-//   D[g][m-tile][n-tile] = A[g][K rows][m-tile]^T  B[g][K rows][n-tile]
-//
-// One work unit = (group g, column tile n, a run of up to MCH row tiles m).
-// The unit's B tile -- all K rows, and with KSPLIT the residual rows after
-// them -- is loaded once into a resident region and reused by every row tile
-// of the run, whose A tiles stream through a two-deep ring.  Against the
-// streaming kernel this cuts the L2 -> SM traffic of a 128 x 256 output tile
-// from (A + B) per tile to A per tile plus B / MCH.  With B_BUFS = 2 the next
-// unit's B tile loads while this unit's row tiles run (BN = 128 keeps two
-// resident tiles within shared memory).  Roles, TMEM double buffering, bounded
-// waits and the TMA-store epilogue are as in grouped_gemm_kernel.
-// Column tile and B buffering of the resident-B weight-gradient kernel: 256
-// columns with one resident B tile (default), or 128 columns with two.
-// Measured at the 17-task step: 0.580 ms against 0.800 ms -- twice the A
-// (L2 -> SM) traffic per output byte costs more than the hidden B loads save.
-#ifndef VMOE_BSTAT_BN
-#define VMOE_BSTAT_BN 256
-#endif
-constexpr int BSTAT_BN = VMOE_BSTAT_BN;
-constexpr int BSTAT_BUFS = BSTAT_BN == 128 ? 2 : 1;
-
-template <int BN, bool KSPLIT, int B_BUFS>
-struct BStatShape {
-    static constexpr int MCH = 6;                              // row tiles per unit
-    static constexpr uint32_t A_KB = BM * BK * 2;              // one A k-block (16 KB)
-    static constexpr uint32_t B_KB = BN * BK * 2;              // one B k-block
-    static constexpr uint32_t A_BUF = 2 * A_KB;                // up to 128 K rows
-    static constexpr uint32_t B_BYTES = (KSPLIT ? 4 : 2) * B_KB;
-    // A ring depth 2 (measured: a single A buffer, which would leave room for
-    // double-buffered staging with the split, made dW1 26% slower).
-    static constexpr int A_BUFS = 2;
-    static constexpr int STG_BUFS = KSPLIT ? 1 : 2;            // 32 x 64 staging tiles per warp
-    static constexpr uint32_t EPI_BYTES = 8 * STG_BUFS * 4096;
-    static constexpr uint32_t TMEM_COLS = 2 * BN;
-    static constexpr int NUM_BARS = 9 + 2 * B_BUFS;
-    static constexpr size_t SMEM_BYTES =
-        1024 + B_BUFS * B_BYTES + A_BUFS * A_BUF + EPI_BYTES + NUM_BARS * 8 + 16;
-};
-
-template <int BN, bool KSPLIT, int B_BUFS>
-__global__ void __launch_bounds__(THREADS, 1)
-wgrad_bstat_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ CUtensorMap tmD, const __grid_constant__ TailMaps tmT,
-                   Args args) {
-    using S = BStatShape<BN, KSPLIT, B_BUFS>;
-    constexpr uint32_t IDESC = idesc_bf16(BM, BN, true, true);
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t raw_addr = smem_u32(smem_raw);
-    uint8_t *smem = smem_raw + ((1024u - (raw_addr & 1023u)) & 1023u);
-    uint8_t *b_res = smem;  // B_BUFS x [hi kb0, hi kb1, lo kb0, lo kb1]
-    uint8_t *a_ring = b_res + B_BUFS * S::B_BYTES;          // 2 x [kb0, kb1]
-    uint8_t *epi_base = a_ring + S::A_BUFS * S::A_BUF;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(epi_base + S::EPI_BYTES);
-    int *misc = reinterpret_cast<int *>(bars + S::NUM_BARS);  // [0] tmem base, [1] abort
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    auto bar_afull = [&](int i) { return smem_u32(bars + 0 + i); };
-    auto bar_aempty = [&](int i) { return smem_u32(bars + 2 + i); };
-    auto bar_tfull = [&](int i) { return smem_u32(bars + 4 + i); };
-    auto bar_tempty = [&](int i) { return smem_u32(bars + 6 + i); };
-    const uint32_t bar_drain = smem_u32(bars + 8);
-    auto bar_bfull = [&](int i) { return smem_u32(bars + 9 + i); };
-    auto bar_bempty = [&](int i) { return smem_u32(bars + 9 + B_BUFS + i); };
-    volatile int *abort_flag = misc + 1;
-
-    if (tid == 0) {
-        for (int i = 0; i < B_BUFS; ++i) {
-            mbar_init(bar_bfull(i), 1);
-            mbar_init(bar_bempty(i), 1);
-        }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(bar_afull(i), 1);
-            mbar_init(bar_aempty(i), 1);
-            mbar_init(bar_tfull(i), 1);
-            mbar_init(bar_tempty(i), 8);
-        }
-        mbar_init(bar_drain, 1);
-        misc[1] = 0;
-        fence_barrier_init();
-        fence_proxy_async();
-        prefetch_map(&tmA);
-        prefetch_map(&tmB);
-        prefetch_map(&tmD);
-        for (int i = 0; i < 3; ++i) {
-            prefetch_map(&tmT.a[i]);
-            prefetch_map(&tmT.b[i]);
-        }
-    }
-    if (warp == 0) {
-        tmem_alloc(smem_u32(misc), S::TMEM_COLS);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    pdl_wait();  // the predecessor's outputs are complete from here on
-    const uint32_t tmem_base = (uint32_t)misc[0];
-    const int nch = (args.tiles_m + S::MCH - 1) / S::MCH;
-    const int total = args.G * args.tiles_n * nch;
-    // unit u -> entry (its real group g and compact row crow), column tile,
-    // first row tile and row-tile count
-    int crow = 0;
-    auto decode = [&](int u, int &g, int &n_blk, int &m0, int &mcnt, int &L) {
-        const int i = u / (args.tiles_n * nch);
-        const int r = u - i * args.tiles_n * nch;
-        g = real_group(args, i);
-        crow = args.crow ? __ldg(args.crow + i) : 0;
-        n_blk = r / nch;
-        m0 = (r - n_blk * nch) * S::MCH;
-        mcnt = min(S::MCH, args.tiles_m - m0);
-        L = __ldg(args.load + g);
-        L = L < 0 ? 0 : (L > args.C ? args.C : L);
-    };
-
-    if (warp == 0) {
-        // ------------------------------------------------------------ producer
-        if (lane == 0) {
-            int ub = 0;  // units with rows, in order: B buffer ub % B_BUFS
-            int ia = 0;
-            bool ok = true;
-            int b_issued[B_BUFS] = {}, a_issued[2] = {0, 0};
-            for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
-                int g, n_blk, m0, mcnt, L;
-                decode(u, g, n_blk, m0, mcnt, L);
-                if (u + (int)gridDim.x >= total) pdl_launch_dependents();  // this CTA's last unit
-                const int nkb = (L + BK - 1) / BK;
-                if (nkb == 0) continue;
-                const int bb = ub % B_BUFS;
-                if (!wait_phase(bar_bempty(bb), (uint32_t)((ub / B_BUFS) & 1) ^ 1u, abort_flag,
-                                args.status))
-                    break;
-                const uint32_t bdst = smem_u32(b_res) + bb * S::B_BYTES;
-                // the last k-block loads R = tail_rows(rem) rows (chunk stride R x 128)
-                const int Rl = tail_rows(L - (nkb - 1) * BK);
-                const uint32_t bbytes = (uint32_t)((nkb - 1) * BK + Rl) * (BN / 64) * 128u;
-                mbar_expect_tx(bar_bfull(bb), (KSPLIT ? 2u : 1u) * bbytes);
-                const bool cmpb = (args.compact & CMP_B) != 0;  // B rows from crow, residual after L
-                for (int kb = 0; kb < nkb; ++kb) {
-                    const CUtensorMap *mB = kb == nkb - 1 && Rl < BK ? &tmT.b[Rl / 16 - 1] : &tmB;
-                    tma_load_4d(bdst + kb * S::B_KB, mB, bar_bfull(bb), 0,
-                                (cmpb ? crow : 0) + kb * BK, n_blk * (BN / 64), cmpb ? 0 : g);
-                    if (KSPLIT)
-                        tma_load_4d(bdst + (2 + kb) * S::B_KB, mB, bar_bfull(bb), 0,
-                                    (cmpb ? crow + L : args.C) + kb * BK, n_blk * (BN / 64),
-                                    cmpb ? 0 : g);
-                }
-                ++b_issued[bb];
-                ++ub;
-                for (int m = m0; m < m0 + mcnt; ++m, ++ia) {
-                    const int ab = ia % S::A_BUFS;
-                    if (!wait_phase(bar_aempty(ab), (uint32_t)((ia / S::A_BUFS) & 1) ^ 1u, abort_flag,
-                                    args.status)) {
-                        ok = false;
-                        break;
-                    }
-                    mbar_expect_tx(bar_afull(ab), (uint32_t)((nkb - 1) * BK + Rl) * (BM / 64) * 128u);
-                    for (int kb = 0; kb < nkb; ++kb)
-                        tma_load_4d(smem_u32(a_ring) + ab * S::A_BUF + kb * S::A_KB,
-                                    kb == nkb - 1 && Rl < BK ? &tmT.a[Rl / 16 - 1] : &tmA,
-                                    bar_afull(ab), 0, kb * BK, m * (BM / 64), g);
-                    ++a_issued[ab];
-                }
-            }
-            if (*abort_flag) {  // let copies in flight land before the CTA exits
-                const unsigned long long t0 = global_ns();
-                for (int i = 0; i < B_BUFS; ++i)
-                    if (b_issued[i] > 0)
-                        while (!mbar_try_wait(bar_bfull(i), (uint32_t)((b_issued[i] - 1) & 1)) &&
-                               global_ns() - t0 < 100000000ull) {
-                        }
-                for (int i = 0; i < 2; ++i)
-                    if (a_issued[i] > 0)
-                        while (!mbar_try_wait(bar_afull(i), (uint32_t)((a_issued[i] - 1) & 1)) &&
-                               global_ns() - t0 < 200000000ull) {
-                        }
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer
-        int ub = 0;
-        int ia = 0, it = 0;
-        bool ok = true;
-        // rows [z0, z1) of every 64-wide chunk of the last k-block tile, whose
-        // chunks are z1 x 128 bytes apart (it holds z1 = tail_rows rows), are zeroed
-        auto zero_rows = [&](uint8_t *tile, int chunks, int z0, int z1) {
-            const int rows = z1 - z0;
-            const int units = chunks * rows * 8;
-            for (int i = lane; i < units; i += 32) {
-                const int c = i / (rows * 8);
-                const int w = i - c * rows * 8;
-                *reinterpret_cast<uint4 *>(tile + c * (z1 * 128) + (z0 + (w >> 3)) * 128 + (w & 7) * 16) =
-                    make_uint4(0, 0, 0, 0);
-            }
-        };
-        for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
-            int g, n_blk, m0, mcnt, L;
-            decode(u, g, n_blk, m0, mcnt, L);
-            const int nkb = (L + BK - 1) / BK;
-            const int rem = L - (nkb - 1) * BK;       // valid rows of the last k-block
-            const int nk_last = (rem + 15) >> 4;      // MMAs (K = 16) in the last k-block
-            const int bb = ub % B_BUFS;
-            uint8_t *bres = b_res + bb * S::B_BYTES;
-            if (nkb > 0) {
-                if (!wait_phase(bar_bfull(bb), (uint32_t)((ub / B_BUFS) & 1), abort_flag, args.status))
-                    break;
-                tc_fence_after();
-                if (rem < nk_last * 16) {  // K tail of the resident B: zero once per unit
-                    zero_rows(bres + (nkb - 1) * S::B_KB, BN / 64, rem, nk_last * 16);
-                    if (KSPLIT) zero_rows(bres + (1 + nkb) * S::B_KB, BN / 64, rem, nk_last * 16);
-                    fence_proxy_async();
-                }
-                __syncwarp();
-            }
-            for (int m = m0; m < m0 + mcnt; ++m, ++it) {
-                const int acc = it & 1;
-                if (!wait_phase(bar_tempty(acc), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag,
-                                args.status)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                if (nkb == 0) {
-                    if (lane == 0) mbar_arrive(bar_tfull(acc));
-                    __syncwarp();
-                    continue;
-                }
-                const int ab = ia % S::A_BUFS;
-                if (!wait_phase(bar_afull(ab), (uint32_t)((ia / S::A_BUFS) & 1), abort_flag, args.status)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                uint8_t *abuf = a_ring + ab * S::A_BUF;
-                if (rem < nk_last * 16) {
-                    zero_rows(abuf + (nkb - 1) * S::A_KB, BM / 64, rem, nk_last * 16);
-                    fence_proxy_async();
-                }
-                __syncwarp();
-                if (lane == 0) {
-                    const uint32_t dtmem = tmem_base + (uint32_t)(acc * BN);
-                    const uint32_t a0 = smem_u32(abuf), b0 = smem_u32(bres);
-                    for (int part = 0; part < (KSPLIT ? 2 : 1); ++part)
-                        for (int kb = 0; kb < nkb; ++kb) {
-                            const int nk = kb == nkb - 1 ? nk_last : BK / 16;
-                            const uint32_t at = a0 + kb * S::A_KB;
-                            const uint32_t bt = b0 + (part * 2 + kb) * S::B_KB;
-                            for (int kk = 0; kk < nk; ++kk)  // k-block of 16 nk rows (the last one: tail_rows)
-                                mma_bf16(dtmem, operand_desc_mn(at, kk, nk * 16), operand_desc_mn(bt, kk, nk * 16),
-                                         IDESC, (part | kb | kk) != 0 ? 1u : 0u);
-                        }
-                    mma_commit(bar_aempty(ab));
-                    mma_commit(bar_tfull(acc));
-                }
-                __syncwarp();
-                ++ia;
-            }
-            if (!ok) break;
-            if (nkb > 0) {
-                if (lane == 0) mma_commit(bar_bempty(bb));  // B may be replaced once these MMAs finish
-                __syncwarp();
-                ++ub;
-            }
-        }
-        if (lane == 0) {
-            mma_commit(bar_drain);
-            const unsigned long long t0 = global_ns();
-            while (!mbar_try_wait(bar_drain, 0) && global_ns() - t0 < 1000000000ull) {
-            }
-        }
-        __syncwarp();
-    } else {
-        // ------------------------------------------------------------ epilogue
-        const int ew = warp - 2;
-        const int q = warp & 3;
-        const int half = ew >> 2;
-        constexpr int COLS = BN / 2;
-        uint8_t *stg = epi_base + ew * S::STG_BUFS * 4096;
-        int nstore = 0, it = 0;
-        bool ok = true;
-        for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
-            int g, n_blk, m0, mcnt, L;
-            decode(u, g, n_blk, m0, mcnt, L);
-            for (int m = m0; m < m0 + mcnt; ++m, ++it) {
-                const int acc = it & 1;
-                if (!wait_phase(bar_tfull(acc), (uint32_t)((it >> 1) & 1), abort_flag, args.status)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const int row0 = m * BM + q * 32;
-                const int colw = n_blk * BN + half * COLS;
-                const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) +
-                                      (uint32_t)(acc * BN + half * COLS);
-                // all of this warp's accumulator columns with one wait, then
-                // 32 x 64 chunks through the staging tile(s) and TMA stores
-                uint32_t r[COLS / 32][32];
-                if (L > 0) {
-#pragma unroll
-                    for (int i = 0; i < COLS / 32; ++i) tmem_ld32(trow + i * 32, r[i]);
-                    tmem_ld_wait();
-                } else {
-#pragma unroll
-                    for (int i = 0; i < COLS / 32; ++i)
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) r[i][j] = 0u;
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_tempty(acc));
-#pragma unroll
-                for (int c = 0; c < COLS / 64; ++c) {
-                    uint8_t *buf = stg + (S::STG_BUFS == 2 ? (nstore & 1) * 4096 : 0);
-                    if (lane == 0 && nstore >= S::STG_BUFS) {
-                        if (S::STG_BUFS == 2) bulk_wait_read1();
-                        else bulk_wait_read0();
-                    }
-                    __syncwarp();
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const uint32_t *src = &r[2 * c + (j >> 2)][(j & 3) * 8];
-                        uint4 pk;
-                        pk.x = pack_bf16x2(__uint_as_float(src[0]), __uint_as_float(src[1]));
-                        pk.y = pack_bf16x2(__uint_as_float(src[2]), __uint_as_float(src[3]));
-                        pk.z = pack_bf16x2(__uint_as_float(src[4]), __uint_as_float(src[5]));
-                        pk.w = pack_bf16x2(__uint_as_float(src[6]), __uint_as_float(src[7]));
-                        *reinterpret_cast<uint4 *>(buf + lane * 128 + ((j ^ (lane & 7)) << 4)) = pk;
-                    }
-                    fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) {
-                        tma_store_3d(&tmD, smem_u32(buf), colw + c * 64, row0, g);
-                        bulk_commit();
-                    }
-                    ++nstore;
-                }
-            }
-        }
-        if (lane == 0) bulk_wait_all();
-        __syncwarp();
     }
 
     tc_fence_before();
@@ -1282,12 +935,12 @@ bool make_map_chunked(CUtensorMap *map, const void *base, uint64_t mn, uint64_t 
                       uint64_t outer, uint32_t box_rows, uint32_t box_chunks,
                       uint64_t outer_stride_elems = 0);
 
-template <int BN, int MODE, bool A_MN, bool B_MN, int EPI>
+template <int BN, int MODE, bool A_MN, bool B_MN, int EPI, bool EAGER = true>
 int launch(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &md,
            const CUtensorMap &md2, const TailMaps &mat, const Args &a, long long max_tiles,
            cudaStream_t s, const char *name) {
     using S = Shape<BN, MODE, EPI>;
-    auto kern = grouped_gemm_kernel<BN, MODE, A_MN, B_MN, EPI>;
+    auto kern = grouped_gemm_kernel<BN, MODE, A_MN, B_MN, EPI, EAGER>;
     static std::atomic<int> smem_limit[64];
     if (const int st = raise_smem_limit((const void *)kern, smem_limit, (int)S::SMEM_BYTES)) return st;
     if (max_tiles <= 0) return VMOE_OK;
@@ -1295,22 +948,6 @@ int launch(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &md,
     trace_before(s, name);
     const int st = launch_kernel(kern, dim3((unsigned)grid), dim3(S::NT), S::SMEM_BYTES, s, ma, mb,
                                  md, md2, mat, a);
-    trace_after(s);
-    return st;
-}
-
-template <int BN, bool KSPLIT, int B_BUFS>
-int launch_bstat(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &md, const TailMaps &mt,
-                 const Args &a, long long units, cudaStream_t s, const char *name) {
-    using S = BStatShape<BN, KSPLIT, B_BUFS>;
-    auto kern = wgrad_bstat_kernel<BN, KSPLIT, B_BUFS>;
-    static std::atomic<int> smem_limit[64];
-    if (const int st = raise_smem_limit((const void *)kern, smem_limit, (int)S::SMEM_BYTES)) return st;
-    if (units <= 0) return VMOE_OK;
-    long long grid = units < num_sms() ? units : num_sms();
-    trace_before(s, name);
-    const int st = launch_kernel(kern, dim3((unsigned)grid), dim3(THREADS), S::SMEM_BYTES, s, ma, mb,
-                                 md, mt, a);
     trace_after(s);
     return st;
 }

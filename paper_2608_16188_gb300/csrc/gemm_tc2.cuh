@@ -517,6 +517,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const int half = ew >> 2;
         constexpr int COLS = S::BN / 2;  // 128 columns per warp
         uint8_t *stg = epi_base + ew * S::STG_BUFS * 4096;
+        const uint64_t policy = evict_first_policy();
         int nstore = 0, it = 0;
         bool ok = true;
         for (int u = u_first; u < u_end && ok; u += u_step) {
@@ -569,7 +570,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) {
-                        tma_store_3d(&tmD, smem_u32(buf), colw + c * 64, row0, g);
+                        tma_store_3d(&tmD, smem_u32(buf), colw + c * 64, row0, g, policy);
                         bulk_commit();
                     }
                     ++nstore;
@@ -1140,15 +1141,16 @@ int row_gemm(const Dims &p, const __nv_bfloat16 *act, int K, const __nv_bfloat16
 // over each group's load[g] rows; both operands MN-major.
 // ksplit: act2 is [G, 2C, N] -- a bf16 part in rows [0, C) and its residual in
 // rows [C, 2C) -- and D = act1^T (hi + lo), summed over both halves.
-// Kernel choice (measured on GB300, ms per launch, one-SM kernel -> pair):
+// Kernel choice (measured on GB300, us per launch):
 //   M, N multiples of 256 and C <= 256: the SM-pair kernel above (resident B,
-//     double buffered where two B tiles fit) -- dW1 at the 17-task ViT-B step
-//     (C 124) 0.568 -> 0.539, at the 6-task one (C 247) 0.479 -> 0.387, at the
-//     Zipf-skewed one (C 25) 0.787 -> 0.724; dW2 0.298 -> 0.262 (C 247) and
-//     0.732 -> 0.722 (C 25) -- except dW2 with 32 < C <= 128, where the
-//     streaming kernel stays faster (0.477 against 0.512 at C 124);
-//   otherwise, 32 < C <= 128 with ksplit: the one-SM resident-B kernel;
-//   otherwise the streaming grouped GEMM (both halves in its K loop).
+//     double buffered where two B tiles fit), except dW2 with 32 < C <= 128,
+//     where the streaming kernel is faster (17-task ViT-B step, C 124: 445
+//     against 480);
+//   otherwise the streaming grouped GEMM (both halves in its K loop).  A one-SM
+//     kernel with a resident B tile used to take dW1 of M % 256 != 0 at 32 < C
+//     <= 128; since the producers are two threads it is slower (d 384, f 1536,
+//     C 124: 180 against 169 with 17 tasks of 32 experts, 33 against 26 with 4
+//     of 16).
 // VMOE_PAIR=0 in the environment turns the pair kernel off.
 inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __nv_bfloat16 *act2,
                       int N, const int32_t *load, __nv_bfloat16 *D, cudaStream_t s,
@@ -1158,19 +1160,7 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
     const bool wide = N % 256 == 0;
     const int BN = wide ? 256 : 128;
     const bool cmpb = (sl.compact & CMP_B) != 0;
-    // B: per-group slabs of C (with ksplit 2C) rows, or the compact buffer
-    const uint64_t b_rows = cmpb ? (uint64_t)sl.rows : (uint64_t)(ksplit ? 2 * C : C);
-    const uint64_t b_outer = cmpb ? 1 : (uint64_t)G;
     CUtensorMap ma, mb, md;
-    TailMaps mt;  // the last k-block's boxes of 16, 32 and 48 K rows
-    // a_chunks / b_chunks: the 64-column chunks of one A / B box
-    auto tail_maps = [&](int a_chunks, int b_chunks) {
-        for (int i = 0; i < 3; ++i)
-            if (!make_map_chunked(&mt.a[i], act1, M, C, G, 16 * (i + 1), a_chunks) ||
-                !make_map_chunked(&mt.b[i], act2, N, b_rows, b_outer, 16 * (i + 1), b_chunks))
-                return false;
-        return true;
-    };
     if (!make_map(&md, D, N, M, G, 32)) return VMOE_ERR_CUDA;  // 64 x 32 store boxes
     Args a = base_args(p, load);
     a.N = N;
@@ -1212,33 +1202,21 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
     if (!make_map_chunked(&ma, act1, M, C, G, 64, BM / 64)) return VMOE_ERR_CUDA;
     // exactly C rows a group, and a map of its own for the residual, so that rows before row 0 read zeros
     CUtensorMap mblo = {};
-    if (cmpb ? !make_map_chunked(&mb, act2, N, b_rows, 1, 64, BN / 64)
+    if (cmpb ? !make_map_chunked(&mb, act2, N, (uint64_t)sl.rows, 1, 64, BN / 64)
              : !make_map_chunked(&mb, act2, N, C, G, 64, BN / 64, ksplit ? 2 * (uint64_t)C * N : 0) ||
                    (ksplit && !make_map_chunked(&mblo, act2 + (size_t)C * N, N, C, G, 64, BN / 64,
                                                 2 * (uint64_t)C * N)))
         return VMOE_ERR_CUDA;
     a.tiles_n = N / BN;
     a.tiles_m = M / BM;
-    // Resident B when every group fits one B tile (C <= 128) but is not tiny: with
-    // C <= 32 a unit has almost no MMA work to hide its B reload behind, and the
-    // streaming kernel, which pipelines across tiles, is faster (measured at the
-    // Zipf-skewed workload, C = 25: 0.770 against 0.904 ms; at C = 124 the
-    // resident-B kernel wins, 0.566 against 0.749 ms).
-    constexpr int BSTAT_MIN_C = 32;
-    if (ksplit && N % BSTAT_BN == 0 && C <= 2 * BK && C > BSTAT_MIN_C) {
-        using SB = BStatShape<BSTAT_BN, true, BSTAT_BUFS>;
-        CUtensorMap mbs;
-        if (!make_map_chunked(&mbs, act2, N, b_rows, b_outer, 64, BSTAT_BN / 64)) return VMOE_ERR_CUDA;
-        if (!tail_maps(BM / 64, BSTAT_BN / 64)) return VMOE_ERR_CUDA;
-        a.tiles_n = N / BSTAT_BN;
-        const int nch = (a.tiles_m + SB::MCH - 1) / SB::MCH;
-        const long long units = (long long)a.G * a.tiles_n * nch;
-        return launch_bstat<BSTAT_BN, true, BSTAT_BUFS>(ma, mbs, md, mt, a, units, s, name);
-    }
     long long max_tiles = (long long)a.G * a.tiles_m * a.tiles_n;
     const TailMaps unused{};  // the streaming kernel loads full k-blocks
-    return wide ? launch<256, MODE_WGRAD, true, true, EPI_STORE>(ma, mb, md, mblo, unused, a, max_tiles, s, name)
-                : launch<128, MODE_WGRAD, true, true, EPI_STORE>(ma, mb, md, mblo, unused, a, max_tiles, s, name);
+    auto go = [&](auto kern_launch) { return kern_launch(ma, mb, md, mblo, unused, a, max_tiles, s, name); };
+    if (C <= 2 * BK && !ksplit)  // bound by their stores: see grouped_gemm_kernel's EAGER
+        return wide ? go(launch<256, MODE_WGRAD, true, true, EPI_STORE, false>)
+                    : go(launch<128, MODE_WGRAD, true, true, EPI_STORE, false>);
+    return wide ? go(launch<256, MODE_WGRAD, true, true, EPI_STORE>)
+                : go(launch<128, MODE_WGRAD, true, true, EPI_STORE>);
 }
 
 }  // namespace tc
