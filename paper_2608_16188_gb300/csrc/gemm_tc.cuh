@@ -241,6 +241,22 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, uint32_t sr
         "r"(src), "r"(c0), "r"(c1), "r"(c2), "l"(policy)
         : "memory");
 }
+// An empty group's weight gradient is zeros, one contiguous slab: its unit (or
+// tile) `part` of `parts` writes the slab's share by 4 KB copies of `zeros` (4 KB
+// of zeroed shared memory), `w` of `nw` warps taking every nw-th copy (called by
+// one thread).  slab: bytes, a multiple of 4096 * parts.  Against 32 x 64 boxes
+// staged and waited for one by one, dW1 and dW2 of the Zipf-skewed step, where
+// two groups in three are empty: ZEROS_MEASURED.
+__device__ __forceinline__ void store_zeros(uint8_t *slab_base, long long slab, int part, int parts, int w, int nw,
+                                            uint32_t zeros, uint64_t policy) {
+    const long long n = slab / parts / 4096;
+    uint8_t *dst = slab_base + (long long)part * n * 4096;
+    for (long long i = w; i < n; i += nw)
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], 4096, %2;" ::"l"(dst + i * 4096),
+                     "r"(zeros), "l"(policy)
+                     : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read1() {
     asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
@@ -354,6 +370,20 @@ __device__ __forceinline__ uint64_t desc_step(uint64_t d, int kk, bool mn_major)
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn, bool b_mn) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) |
            ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// Zeroes a warp's first 4 KB staging tile for store_zeros, once the copies that
+// read it are done (`zeroed`: it already holds zeros).
+__device__ __forceinline__ void zero_staging(uint8_t *stg, bool &zeroed) {
+    if (zeroed) return;
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) bulk_wait_read0();
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4 *>(stg + (i * 32 + lane) * 16) = make_uint4(0, 0, 0, 0);
+    fence_proxy_async();
+    __syncwarp();
+    zeroed = true;
 }
 
 struct Tile {
@@ -747,27 +777,35 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         const uint64_t policy = evict_first_policy();
         int nstore = 0;
         int it = 0;
+        bool zeroed = false;  // the first staging tile holds zeros that copies in flight read
         for (int u = blockIdx.x; u < total; u += gridDim.x, ++it) {
             const Tile t = decode_tile<MODE>(args, prefix, u);
             const int acc = it & 1;
             const uint32_t aph = (uint32_t)((it >> 1) & 1);
             if (!wait_phase(bar_tfull(acc), aph, abort_flag, args.status)) break;
             tc_fence_after();
+            if (t.kblocks == 0) {
+                zero_staging(stg, zeroed);
+                if (lane == 0) {
+                    mbar_arrive(bar_tempty(acc));
+                    const int parts = args.tiles_m * args.tiles_n;
+                    store_zeros(reinterpret_cast<uint8_t *>(args.D + (long long)t.gr * args.sD), args.sD * 2,
+                                t.m_blk * args.tiles_n + t.n_blk, parts, ew, 8, smem_u32(stg), policy);
+                }
+                continue;
+            }
+            if (zeroed) {
+                if (lane == 0) bulk_wait_read0();
+                zeroed = false;
+            }
             const int row0 = t.m_blk * BM + q * 32;
             const int colw = t.n_blk * BN + half * COLS;
             const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) +
                                   (uint32_t)(acc * BN + half * COLS);
             uint32_t r[COLS / 32][32];
-            if (t.kblocks > 0) {
 #pragma unroll
-                for (int i = 0; i < COLS / 32; ++i) tmem_ld32(trow + i * 32, r[i]);
-                tmem_ld_wait();
-            } else {
-#pragma unroll
-                for (int i = 0; i < COLS / 32; ++i)
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) r[i][j] = 0u;
-            }
+            for (int i = 0; i < COLS / 32; ++i) tmem_ld32(trow + i * 32, r[i]);
+            tmem_ld_wait();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_tempty(acc));  // the accumulator is in registers now

@@ -519,36 +519,40 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         uint8_t *stg = epi_base + ew * S::STG_BUFS * 4096;
         const uint64_t policy = evict_first_policy();
         int nstore = 0, it = 0;
-        bool ok = true;
+        bool ok = true, zeroed = false;  // zeroed: the first staging tile holds zeros that copies in flight read
         for (int u = u_first; u < u_end && ok; u += u_step) {
             int g, n_blk, L;
             decode(u, g, n_blk, L);
+            if (L == 0) {
+                zero_staging(stg, zeroed);
+                if (lane == 0)
+                    store_zeros(reinterpret_cast<uint8_t *>(args.D + (long long)g * args.sD), args.sD * 2, n_blk,
+                                args.tiles_n, (int)rank * 8 + ew, 16, smem_u32(stg), policy);
+                continue;
+            }
+            if (zeroed) {
+                if (lane == 0) bulk_wait_read0();
+                zeroed = false;
+            }
             for (int m = 0; m < tiles_m; ++m) {
                 const int row0 = m * S::MP + (int)rank * 128 + q * 32;
                 const int colw = n_blk * S::BN + half * COLS;
                 uint32_t r[COLS / 32][32];
-                if (L > 0) {
-                    const int acc = it & 1;
-                    if (!wait_phase(bar_tfull(acc), (uint32_t)((it >> 1) & 1), abort_flag, args.status)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) +
-                                          (uint32_t)(acc * S::BN + half * COLS);
-#pragma unroll
-                    for (int i = 0; i < COLS / 32; ++i) tmem_ld32(trow + i * 32, r[i]);
-                    tmem_ld_wait();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_remote(mapa_shared(bar_tempty(acc), 0));
-                    ++it;
-                } else {
-#pragma unroll
-                    for (int i = 0; i < COLS / 32; ++i)
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) r[i][j] = 0u;
+                const int acc = it & 1;
+                if (!wait_phase(bar_tfull(acc), (uint32_t)((it >> 1) & 1), abort_flag, args.status)) {
+                    ok = false;
+                    break;
                 }
+                tc_fence_after();
+                const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) +
+                                      (uint32_t)(acc * S::BN + half * COLS);
+#pragma unroll
+                for (int i = 0; i < COLS / 32; ++i) tmem_ld32(trow + i * 32, r[i]);
+                tmem_ld_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_remote(mapa_shared(bar_tempty(acc), 0));
+                ++it;
 #pragma unroll
                 for (int c = 0; c < COLS / 64; ++c) {
                     uint8_t *buf = stg + (S::STG_BUFS == 2 ? (nstore & 1) * 4096 : 0);
