@@ -21,7 +21,8 @@
 //               The accumulator is double buffered in TMEM
 //               (2 x BN columns), so tile i's epilogue overlaps tile i+1's
 //               main loop.
-// Tiles are distributed statically: CTA b takes tiles b, b + grid, ...  In
+// Tiles go to CTAs with a fixed stride (CTA b takes tiles b, b + grid, ...), the
+// weight gradients' larger ones by cluster launch control.  In
 // row mode (H = Xe W1 etc.) a group contributes ceil(load/128) x N/BN tiles,
 // counted from the device-resident loads by every CTA with a block scan, so
 // empty groups cost nothing and no host round trip is needed.  In weight-
@@ -35,6 +36,8 @@
 #pragma once
 
 #include <cuda.h>  // CUtensorMap and its enums (types only; the encoder is fetched at run time)
+
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -67,7 +70,8 @@ constexpr int ROW_CH = 32;
 template <int MODE, int EPI>
 struct Roles {
     static constexpr int EW = (MODE == 0 && EPI != EPI_STORE) ? 16 : 8;  // epilogue warps
-    static constexpr int NT = 96 + 32 * EW;  // threads: A producer, MMA, epilogue, B producer
+    // threads: A producer, MMA, epilogue, B producer; weight gradients: scheduler
+    static constexpr int NT = 96 + 32 * EW + (MODE == 1 ? 32 : 0);
     static constexpr int PITCH = 80;         // staging row pitch (bytes): 64 data + 16 pad
 };
 
@@ -226,8 +230,8 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
 }
 // L2 policy of the weight-gradient stores: first to be evicted.  Nothing reads
 // a gradient again before the step ends, and its lines otherwise push the
-// activations out.  Measured at the 17-task step: dW1 522 -> 506 us, dW2 465 ->
-// 445 us; the attention experts' dW_qkv 375 -> 355 us.
+// activations out.  Measured at the 17-task step (before dynamic tiles): dW1 522
+// -> 506 us, dW2 499 -> 477 us; the attention experts' dW_qkv 375 -> 355 us.
 __device__ __forceinline__ uint64_t evict_first_policy() {
     uint64_t policy;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
@@ -245,8 +249,8 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, uint32_t sr
 // tile) `part` of `parts` writes the slab's share by 4 KB copies of `zeros` (4 KB
 // of zeroed shared memory), `w` of `nw` warps taking every nw-th copy (called by
 // one thread).  slab: bytes, a multiple of 4096 * parts.  Against 32 x 64 boxes
-// staged and waited for one by one, dW1 and dW2 of the Zipf-skewed step, where
-// two groups in three are empty: ZEROS_MEASURED.
+// staged and waited for one by one, the Zipf-skewed step, where two groups in
+// three are empty, went from 2386 to 2353 us.
 __device__ __forceinline__ void store_zeros(uint8_t *slab_base, long long slab, int part, int parts, int w, int nw,
                                             uint32_t zeros, uint64_t policy) {
     const long long n = slab / parts / 4096;
@@ -273,6 +277,126 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map
         "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
         : "memory");
 }
+// ---------------------------------------------------------------------------
+// Dynamic tiles by cluster launch control: the grid has a CTA (or pair) per
+// tile, the ones that run take the next one not yet launched
+// (clusterlaunchcontrol.try_cancel) instead of a fixed stride.  The tiles in
+// work are then always the oldest ones, so the addresses being written stay
+// close together; with a fixed stride the SMs drift apart and DRAM loses
+// bandwidth to it: zeros to 4 GB by 4 KB bulk copies from one CTA an SM run
+// 6.8 TB/s with a stride and 7.8 TB/s this way.
+//
+// One thread a CTA asks (clc_scheduler), CLC_DEPTH answers ahead of the roles;
+// every role reads each answer (clc_take) and frees its slot.  In a pair the
+// leader asks and the answer goes to both CTAs.
+constexpr int CLC_DEPTH = 4;
+struct ClcQueue {
+    uint4 resp[CLC_DEPTH + 1];  // the last one: draining after an abort
+    uint64_t full[CLC_DEPTH], empty[CLC_DEPTH], drain;
+};
+template <bool PAIR>
+__device__ __forceinline__ void clc_try(uint32_t resp, uint32_t bar) {
+    if (PAIR)
+        asm volatile(
+            "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.multicast::cluster::all.b128 "
+            "[%0], [%1];" ::"r"(resp),
+            "r"(bar)
+            : "memory");
+    else
+        asm volatile(
+            "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(resp),
+            "r"(bar)
+            : "memory");
+}
+// Whether an answer holds a CTA, and its (a pair's first) blockIdx.x.
+__device__ __forceinline__ bool clc_query(uint32_t resp, uint32_t &x) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .b128 r;\n\t.reg .pred p;\n\t"
+        "ld.shared.b128 r, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+        "selp.u32 %1, 1, 0, p;\n\t"
+        "mov.u32 %0, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, r;\n\t}\n"
+        : "=r"(x), "=r"(ok)
+        : "r"(resp)
+        : "memory");
+    return ok != 0;
+}
+// consumers: arrivals that free a slot (a pair's leader counts both CTAs' roles)
+__device__ __forceinline__ void clc_init(ClcQueue &q, int consumers) {
+    for (int i = 0; i < CLC_DEPTH; ++i) {
+        mbar_init(smem_u32(q.full + i), 1);
+        mbar_init(smem_u32(q.empty + i), consumers);
+    }
+    mbar_init(smem_u32(&q.drain), 1);
+}
+// One thread a CTA.  `issue`: this CTA asks (a pair's peer only receives).
+// After an abort the CTAs not launched yet are taken and dropped, so that none
+// of them starts and runs into the same wait.
+template <bool PAIR>
+__device__ __forceinline__ void clc_scheduler(ClcQueue &q, bool issue, volatile int *abort_flag, int *status) {
+    uint32_t ph = 0, x;
+    int s = 0;
+    bool more = true, ok = true;
+    while (more) {
+        if (!wait_phase(smem_u32(q.empty + s), ph ^ 1u, abort_flag, status)) {
+            ok = false;
+            break;
+        }
+        fence_proxy_async();  // the roles' reads of the slot before it is written again
+        mbar_expect_tx(smem_u32(q.full + s), 16);
+        if (issue) clc_try<PAIR>(smem_u32(q.resp + s), smem_u32(q.full + s));
+        if (!wait_phase(smem_u32(q.full + s), ph, abort_flag, status)) {
+            ok = false;
+            const unsigned long long t0 = global_ns();  // the answer in flight lands before the CTA exits
+            while (!mbar_try_wait(smem_u32(q.full + s), ph) && global_ns() - t0 < 100000000ull) {
+            }
+            break;
+        }
+        more = clc_query(smem_u32(q.resp + s), x);
+        if (++s == CLC_DEPTH) {
+            s = 0;
+            ph ^= 1u;
+        }
+    }
+    pdl_launch_dependents();  // nothing is left to take
+    for (uint32_t n = 0; !ok && issue && n < (1u << 28); ++n) {
+        const unsigned long long t0 = global_ns();
+        fence_proxy_async();
+        mbar_expect_tx(smem_u32(&q.drain), 16);
+        clc_try<false>(smem_u32(q.resp + CLC_DEPTH), smem_u32(&q.drain));
+        bool got = false;
+        while (!got && global_ns() - t0 < 100000000ull) got = mbar_try_wait(smem_u32(&q.drain), n & 1u);
+        if (!got || !clc_query(smem_u32(q.resp + CLC_DEPTH), x)) break;
+    }
+}
+// A role's place in the queue.  WARP: the whole warp takes (lane 0 frees the
+// slot), else one thread.  leader_empty: in a pair's peer, the leader's `empty`
+// barriers (cluster address), which it frees too.
+struct ClcPos {
+    int s = 0;
+    uint32_t ph = 0;
+};
+template <bool WARP>
+__device__ __forceinline__ bool clc_take(ClcQueue &q, ClcPos &c, uint32_t &x, volatile int *abort_flag, int *status,
+                                         uint32_t leader_empty = 0) {
+    if (!wait_phase(smem_u32(q.full + c.s), c.ph, abort_flag, status)) return false;
+    const bool ok = clc_query(smem_u32(q.resp + c.s), x);
+    fence_proxy_async();
+    if (WARP) __syncwarp();
+    if (!WARP || (threadIdx.x & 31) == 0) {
+        mbar_arrive(smem_u32(q.empty + c.s));
+        if (leader_empty)
+            asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(leader_empty + 8u * (uint32_t)c.s) : "memory");
+    }
+    if (++c.s == CLC_DEPTH) {
+        c.s = 0;
+        c.ph ^= 1u;
+    }
+    return ok;
+}
+
 // Named barrier over `count` threads (ids 1..15; 0 is __syncthreads).
 __device__ __forceinline__ void named_bar(int id, int count) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
@@ -469,12 +593,9 @@ __device__ __forceinline__ void epilogue_chunk(f32x2 (&v)[CH / 2], const uint4 *
     }
 }
 
-// EAGER: the producers and the MMA thread run as elected threads and look the
-// next tile up early.  The weight gradients of groups of at most 128 rows run
-// better without: they are bound by their stores, and copies issued faster only
-// get in their way (17-task step, dW2 477 us with, 445 without; attention dW_qkv
-// 355 / 326; with C 493, ViT-S, 29.3 / 31.0, and there the operands bound it).
-template <int BN, int MODE, bool A_MN, bool B_MN, int EPI, bool EAGER>
+// CLC: tiles by cluster launch control (weight gradients only; the grid is the
+// tile count), else tiles blockIdx.x, blockIdx.x + gridDim.x, ...
+template <int BN, int MODE, bool A_MN, bool B_MN, int EPI, bool CLC>
 __global__ void __launch_bounds__(Roles<MODE, EPI>::NT, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmD2,
@@ -501,8 +622,25 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     auto bar_tempty = [&](int a) { return smem_u32(bars + 2 * STAGES + 2 + a); };
     const uint32_t bar_drain = smem_u32(bars + 2 * STAGES + 4);
     volatile int *abort_flag = misc + 1;
+    static_assert(!CLC || MODE == MODE_WGRAD, "a row-mode grid cannot be the tile count: the host does not know it");
+    __shared__ __align__(16) ClcQueue clc;
+    int total = 0;
+    // The tile after u, for a role of one thread or of a whole warp.
+    auto next_tile = [&](auto warp_wide, ClcPos &pos, int &u) -> bool {
+        if (!CLC) {
+            u += (int)gridDim.x;
+            return u < total;
+        }
+        uint32_t x;
+        if (!clc_take<decltype(warp_wide)::value>(clc, pos, x, abort_flag, args.status)) return false;
+        u = (int)x;
+        return true;
+    };
+    constexpr std::true_type WARP_WIDE{};
+    constexpr std::false_type ONE_THREAD{};
 
     if (tid == 0) {
+        if (CLC) clc_init(clc, Roles<MODE, EPI>::EW + 3);
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar_full(s), 2);  // the A and the B producer's arrivals
             mbar_init(bar_empty(s), 1);
@@ -527,7 +665,6 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     pdl_wait();  // the predecessor's outputs (loads, operands) are complete from here on
 
     // Tile count (and, in row mode, the per-group tile prefix).
-    int total;
     if (MODE == MODE_ROW) {
         const int G = args.G;
         const int per = (G + NT - 1) / NT;
@@ -582,18 +719,24 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // ------------------------------------------------------------ producers: A (warp 0), B (the last warp)
         // One thread each: a copy's wait, expected bytes and issue take it a few
         // hundred cycles, as long as the MMAs of a k-block, so A and B have their own.
-        if (EAGER ? elect_one() : lane == 0) {
+        if (elect_one()) {
             const bool isA = warp == 0;
             int stage = 0;
             uint32_t phase = 0;
             int issued = 0;  // copies so far: slot s has had those of index s, s + STAGES, ...
             bool ok = true;
             const bool cmpa = (args.compact & CMP_A) != 0, cmpb = (args.compact & CMP_B) != 0;
-            Tile t = decode_tile<MODE>(args, prefix, blockIdx.x < total ? blockIdx.x : 0);
-            for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
+            ClcPos pos;
+            int u = (int)blockIdx.x;
+            bool more = u < total;
+            Tile t = decode_tile<MODE>(args, prefix, more ? u : 0);
+            while (more && ok) {
                 Tile tn = t;  // the next tile, looked up behind this one's first copy
-                const bool last = u + (int)gridDim.x >= total;
-                if (isA && last) pdl_launch_dependents();  // this CTA's last tile
+                auto look_up = [&]() {
+                    more = next_tile(ONE_THREAD, pos, u);
+                    if (more) tn = decode_tile<MODE>(args, prefix, u);
+                };
+                if (!CLC && isA && u + (int)gridDim.x >= total) pdl_launch_dependents();  // this CTA's last tile
                 // Row mode, A rows [0, rn): the tile's valid rows rounded up to 16.  The
                 // slot's rows past rn keep stale data, which only reaches output rows
                 // past rows_valid -- never stored.
@@ -649,14 +792,14 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         else
                             tma_load_4d(sb, hi ? &tmD2 : &tmB, fb, 0, ka, t.n_blk * (BN / 64), t.gr);
                     }
-                    if (kb == (EAGER ? 0 : t.kblocks - 1) && !last) tn = decode_tile<MODE>(args, prefix, u + gridDim.x);
+                    if (kb == 0) look_up();
                     ++issued;
                     if (++stage == STAGES) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
-                if (t.kblocks == 0 && !last) tn = decode_tile<MODE>(args, prefix, u + gridDim.x);
+                if (t.kblocks == 0) look_up();
                 t = tn;
             }
             if (*abort_flag) {  // let copies in flight land before the CTA exits
@@ -676,7 +819,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         int it = 0;
         bool ok = true;
         const bool cmpb = MODE == MODE_WGRAD && (args.compact & CMP_B) != 0;
-        const bool one = EAGER ? elect_one() : lane == 0;
+        const bool one = elect_one();
         // Waits for slot `stage` and issues its MMAs from 16-row step k0 on.
         auto k_block = [&](uint32_t dtmem, int k0, bool accumulate) {
             const uint32_t sa = tiles_addr + stage * S::STAGE_BYTES;
@@ -694,11 +837,15 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 phase ^= 1u;
             }
         };
+        ClcPos pos;
+        int u = (int)blockIdx.x;
         if (!cmpb) {
-            for (int u = blockIdx.x; one && u < total && ok; u += gridDim.x, ++it) {
+            bool more = one && u < total;
+            Tile t;
+            if (MODE == MODE_WGRAD && more) t = decode_tile<MODE>(args, prefix, u);
+            for (; more && ok; ++it) {
                 int kblocks = args.K_fixed / BK, khalf = 0, skip = 0;
                 if (MODE == MODE_WGRAD) {
-                    const Tile t = decode_tile<MODE>(args, prefix, u);
                     kblocks = t.kblocks;
                     khalf = t.khalf;
                     skip = (t.khalf * BK - t.kvalid) >> 4;  // all-zero 16-row steps of k-block 0
@@ -718,9 +865,12 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (!ok) break;
                 if (kblocks == 0) mbar_arrive(bar_tfull(acc));
                 else mma_commit(bar_tfull(acc));
+                more = next_tile(ONE_THREAD, pos, u);
+                if (MODE == MODE_WGRAD && more) t = decode_tile<MODE>(args, prefix, u);
             }
         } else {  // compact B: the warp zeroes the rows of k-block 0 (both parts) that belong to a neighbour
-            for (int u = blockIdx.x; u < total && ok; u += gridDim.x, ++it) {
+            bool more = u < total;
+            for (; more && ok; more = next_tile(WARP_WIDE, pos, u), ++it) {
                 const Tile t = decode_tile<MODE>(args, prefix, u);
                 const int z = t.khalf * BK - t.kvalid;
                 const int acc = it & 1;
@@ -763,6 +913,10 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
         }
         __syncwarp();
+    } else if (MODE == MODE_WGRAD && warp == Roles<MODE, EPI>::EW + 3) {
+        // ------------------------------------------------------------ scheduler (idle without CLC)
+        if (CLC && elect_one()) clc_scheduler<false>(clc, true, abort_flag, args.status);
+        __syncwarp();
     } else if (MODE == MODE_WGRAD) {
         // ------------------------------------------------------------ epilogue (weight gradients)
         // Every tile is full.  Each warp reads all BN/2 accumulator columns of its
@@ -778,7 +932,10 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         int nstore = 0;
         int it = 0;
         bool zeroed = false;  // the first staging tile holds zeros that copies in flight read
-        for (int u = blockIdx.x; u < total; u += gridDim.x, ++it) {
+        ClcPos pos;
+        int u = (int)blockIdx.x;
+        bool more = u < total;
+        for (; more; more = next_tile(WARP_WIDE, pos, u), ++it) {
             const Tile t = decode_tile<MODE>(args, prefix, u);
             const int acc = it & 1;
             const uint32_t aph = (uint32_t)((it >> 1) & 1);
@@ -893,11 +1050,14 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
         };
         int it = 0;
-        Tile t = decode_tile<MODE>(args, prefix, blockIdx.x < total ? blockIdx.x : 0);
-        if (EPI == EPI_DGELU && blockIdx.x < total) load_h(t, jw, hcur);
-        for (int u = blockIdx.x; u < total; u += gridDim.x, ++it) {
-            const bool have_next = u + (int)gridDim.x < total;
-            const Tile tn = decode_tile<MODE>(args, prefix, have_next ? u + gridDim.x : u);
+        ClcPos pos;
+        int u = (int)blockIdx.x;
+        bool have = u < total;
+        Tile t = decode_tile<MODE>(args, prefix, have ? u : 0);
+        if (EPI == EPI_DGELU && have) load_h(t, jw, hcur);
+        for (; have; ++it) {
+            const bool have_next = next_tile(WARP_WIDE, pos, u);
+            const Tile tn = have_next ? decode_tile<MODE>(args, prefix, u) : t;
             const int acc = it & 1;
             const uint32_t aph = (uint32_t)((it >> 1) & 1);
             if (!wait_phase(bar_tfull(acc), aph, abort_flag, args.status)) break;
@@ -946,6 +1106,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_tempty(acc));
             t = tn;
+            have = have_next;
         }
     }
 
@@ -973,16 +1134,16 @@ bool make_map_chunked(CUtensorMap *map, const void *base, uint64_t mn, uint64_t 
                       uint64_t outer, uint32_t box_rows, uint32_t box_chunks,
                       uint64_t outer_stride_elems = 0);
 
-template <int BN, int MODE, bool A_MN, bool B_MN, int EPI, bool EAGER = true>
+template <int BN, int MODE, bool A_MN, bool B_MN, int EPI, bool CLC = false>
 int launch(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &md,
            const CUtensorMap &md2, const TailMaps &mat, const Args &a, long long max_tiles,
            cudaStream_t s, const char *name) {
     using S = Shape<BN, MODE, EPI>;
-    auto kern = grouped_gemm_kernel<BN, MODE, A_MN, B_MN, EPI, EAGER>;
+    auto kern = grouped_gemm_kernel<BN, MODE, A_MN, B_MN, EPI, CLC>;
     static std::atomic<int> smem_limit[64];
     if (const int st = raise_smem_limit((const void *)kern, smem_limit, (int)S::SMEM_BYTES)) return st;
     if (max_tiles <= 0) return VMOE_OK;
-    long long grid = max_tiles < num_sms() ? max_tiles : num_sms();
+    const long long grid = CLC || max_tiles < num_sms() ? max_tiles : num_sms();
     trace_before(s, name);
     const int st = launch_kernel(kern, dim3((unsigned)grid), dim3(S::NT), S::SMEM_BYTES, s, ma, mb,
                                  md, md2, mat, a);

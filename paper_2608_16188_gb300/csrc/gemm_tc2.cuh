@@ -17,7 +17,7 @@
 // KSPLIT the residual rows after them -- is loaded once and reused by all M/256
 // row tiles of the group; their A k-blocks stream through a ring.
 //
-// Roles, per CTA (352 threads):
+// Roles, per CTA (384 threads):
 //   warps 0, 10 TMA producers of A (0) and B (10): the CTA's own halves into its
 //               own shared memory.
 //               A k-blocks complete on the leader's `afull` (both CTAs' bytes).
@@ -31,6 +31,7 @@
 //               also issues the MMAs once both CTAs' operands are in and commits
 //               them with a multicast arrive on both CTAs' `aempty`, `bempty`
 //               (per piece with one B buffer) and `tfull`.
+//   warp 11     scheduler: takes the pair's next units by cluster launch control.
 //   warps 2-9   epilogue: tcgen05.ld of this CTA's 128 accumulator rows, arrive on
 //               the leader's `tempty` (count 16: 8 warps x 2 CTAs), bf16 packing
 //               and TMA bulk tensor stores from 128-byte-swizzled staging.
@@ -148,7 +149,8 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
-constexpr int PAIR_THREADS = THREADS + 32;  // wgrad_pair_kernel: + the B producer
+constexpr int PAIR_THREADS = THREADS + 64;  // wgrad_pair_kernel: + the B producer and the scheduler
+constexpr int PAIR_ROLES = 11;              // takers of a tile a CTA: A and B producers, hand-over / MMA warp, 8 epilogue warps
 
 // Shared memory of the pair kernel, per CTA.  KB = one k-block (64 K rows) of
 // 128 columns = 16 KB, for A and B alike.  The B region holds one or two
@@ -181,10 +183,11 @@ struct PairShape {
     static_assert(SMEM_BYTES <= 232448, "over the 227 KB shared-memory limit");
 };
 
-// Which units each SM pair works on.  By default (enabled = 0) pair c takes
-// units c, c + P, c + 2P, ... of P pairs -- a static round-robin over units
-// of nearly equal cost.  With enabled = 1 pair c takes the contiguous units
-// [first[c], first[c] + count[c]): the per-group pair shares of the
+// Which units each SM pair works on.  By default (enabled = 0) a pair takes the
+// next unit not taken yet (cluster launch control; dW1 at the 17-task step 508 ->
+// 484 us against a fixed stride, 703 -> 599 at the Zipf-skewed one, the attention
+// experts' dW_o at C 247 78 -> 66).  With enabled = 1 pair c takes the contiguous
+// units [first[c], first[c] + count[c]): the per-group pair shares of the
 // fill-clamp-refill allocation (Section 3.2.2), each group's units split
 // evenly over the pairs of its share (vmoe_plan_shares; the memory-budgeted
 // backward, whose loads are on the host).
@@ -245,7 +248,11 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     // the peer's abort flag, raised when this CTA gives up
     const uint32_t peer_abort = mapa_shared(smem_u32(misc + 1), rank ^ 1u);
 
+    __shared__ __align__(16) ClcQueue clc;
+    const uint32_t leader_empty = leader ? 0u : mapa_shared(smem_u32(clc.empty), 0);
+
     if (tid == 0) {
+        clc_init(clc, leader ? 2 * PAIR_ROLES : PAIR_ROLES);
         for (int i = 0; i < AS; ++i) {
             mbar_init(bar_afull(i), 1);
             mbar_init(bar_aempty(i), 1);
@@ -278,14 +285,22 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     tc_fence_after();
     pdl_wait();  // the predecessor's outputs are complete from here on
     const uint32_t tmem_base = (uint32_t)misc[0];
-    const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
+    const int cid = blockIdx.x >> 1;
     const int total = args.G * args.tiles_n;
     const int tiles_m = args.tiles_m;  // M / 256
     const bool cmpb = (args.compact & CMP_B) != 0;  // B rows from crow, residual after L
-    // this pair's units: u = u_first, u_first + u_step, ... < u_end
+    // this pair's units: the next one not taken yet, or a contiguous range with a share schedule
     const int u_first = sched.enabled ? sched.first[cid] : cid;
-    const int u_step = sched.enabled ? 1 : ncl;
     const int u_end = sched.enabled ? min(total, sched.first[cid] + sched.count[cid]) : total;
+    auto next_unit = [&](auto warp_wide, ClcPos &pos, int &u) -> bool {
+        if (sched.enabled) return ++u < u_end;
+        uint32_t x;
+        if (!clc_take<decltype(warp_wide)::value>(clc, pos, x, abort_flag, args.status, leader_empty)) return false;
+        u = (int)(x >> 1);
+        return true;
+    };
+    constexpr std::true_type WARP_WIDE{};
+    constexpr std::false_type ONE_THREAD{};
     int crow = 0;
     auto decode = [&](int u, int &g, int &n_blk, int &L) {
         const int i = u / args.tiles_n;
@@ -304,11 +319,13 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if (elect_one()) {
             int sl = 0, issued = 0;  // slot s has had copies s, s + AS, ...
             uint32_t phase = 0;
-            bool ok = true;
-            for (int u = u_first; u < u_end && ok; u += u_step) {
+            ClcPos pos;
+            int u = u_first;
+            bool ok = true, more = u < u_end;
+            while (more && ok) {
                 int g, n_blk, L;
                 decode(u, g, n_blk, L);
-                if (u + u_step >= u_end) pdl_launch_dependents();  // this pair's last unit
+                if (sched.enabled && u + 1 >= u_end) pdl_launch_dependents();  // this pair's last unit
                 const int nkb = (L + BK - 1) / BK;
                 const int r0 = L - nkb * BK;  // first row of k-block 0 (<= 0)
                 for (int m = 0; m < tiles_m && ok; ++m)
@@ -325,6 +342,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                             phase ^= 1u;
                         }
                     }
+                more = next_unit(ONE_THREAD, pos, u);
             }
             // let copies in flight land before the CTA exits; the leader's afull
             // counts the peer's copies too, and the peer waits for the leader at
@@ -346,7 +364,9 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             bool ok = true;
             // per B piece: parity of its uses so far (which gives the phase), and whether it has been used
             uint32_t b_par = 0, b_any = 0;
-            for (int u = u_first; u < u_end && ok; u += u_step) {
+            ClcPos pos;
+            int u = u_first;
+            for (bool more = u < u_end; more && ok; more = next_unit(ONE_THREAD, pos, u)) {
                 int g, n_blk, L;
                 decode(u, g, n_blk, L);
                 const int nkb = (L + BK - 1) / BK;
@@ -407,6 +427,11 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
         __syncwarp();
         give_up();
+    } else if (warp == THREADS / 32 + 1) {
+        // ------------------------------------------------------------ scheduler
+        if (!sched.enabled && elect_one()) clc_scheduler<true>(clc, leader, abort_flag, args.status);
+        __syncwarp();
+        give_up();
     } else if (warp == 1) {
         // ------------------------------------------------------------ B hand-over (+ MMA in the leader)
         int ub = 0, sl = 0, it = 0;
@@ -414,7 +439,9 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const bool one = elect_one();
         uint32_t b_par = 0;  // per B piece, the parity of its uses so far: the phase
         bool ok = true;
-        for (int u = u_first; u < u_end && ok; u += u_step) {
+        ClcPos pos;
+        int u = u_first;
+        for (bool more = u < u_end; more && ok; more = next_unit(WARP_WIDE, pos, u)) {
             int g, n_blk, L;
             decode(u, g, n_blk, L);
             const int nkb = (L + BK - 1) / BK;
@@ -520,7 +547,9 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const uint64_t policy = evict_first_policy();
         int nstore = 0, it = 0;
         bool ok = true, zeroed = false;  // zeroed: the first staging tile holds zeros that copies in flight read
-        for (int u = u_first; u < u_end && ok; u += u_step) {
+        ClcPos pos;
+        int u = u_first;
+        for (bool more = u < u_end; more && ok; more = next_unit(WARP_WIDE, pos, u)) {
             int g, n_blk, L;
             decode(u, g, n_blk, L);
             if (L == 0) {
@@ -995,12 +1024,12 @@ int launch_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap 
     static std::atomic<int> smem_limit[64];
     if (const int st = raise_smem_limit((const void *)kern, smem_limit, (int)S::SMEM_BYTES)) return st;
     if (units <= 0) return VMOE_OK;
-    const int ncl = pair_clusters((const void *)kern, S::SMEM_BYTES);
-    if (ncl <= 0) return VMOE_ERR_CUDA;
-    long long clusters = units < ncl ? units : ncl;
+    long long clusters = units;
     PairSchedule sc;
     sc.enabled = 0;
     if (sched && sched->enabled) {  // a share schedule names its own pairs
+        const int ncl = pair_clusters((const void *)kern, S::SMEM_BYTES);
+        if (ncl <= 0) return VMOE_ERR_CUDA;
         sc = *sched;
         int used = 0;
         for (int c = 0; c < MAX_PAIRS; ++c)
@@ -1148,8 +1177,8 @@ int row_gemm(const Dims &p, const __nv_bfloat16 *act, int K, const __nv_bfloat16
 // Kernel choice (measured on GB300, us per launch):
 //   M, N multiples of 256 and C <= 256: the SM-pair kernel above (resident B,
 //     double buffered where two B tiles fit), except dW2 with 32 < C <= 128,
-//     where the streaming kernel is faster (17-task ViT-B step, C 124: 445
-//     against 480);
+//     where the streaming kernel is faster (17-task ViT-B step, C 124, both with
+//     a fixed stride: 474 against 503);
 //   otherwise the streaming grouped GEMM (both halves in its K loop).  A one-SM
 //     kernel with a resident B tile used to take dW1 of M % 256 != 0 at 32 < C
 //     <= 128; since the producers are two threads it is slower (d 384, f 1536,
@@ -1216,9 +1245,12 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
     long long max_tiles = (long long)a.G * a.tiles_m * a.tiles_n;
     const TailMaps unused{};  // the streaming kernel loads full k-blocks
     auto go = [&](auto kern_launch) { return kern_launch(ma, mb, md, mblo, unused, a, max_tiles, s, name); };
-    if (C <= 2 * BK && !ksplit)  // bound by their stores: see grouped_gemm_kernel's EAGER
-        return wide ? go(launch<256, MODE_WGRAD, true, true, EPI_STORE, false>)
-                    : go(launch<128, MODE_WGRAD, true, true, EPI_STORE, false>);
+    // Dynamic tiles where the gradient is larger than L2 twice over, so that its
+    // stores run at DRAM's rate (17-task step, dW2 474 -> 424 us); a layer whose
+    // gradient stays in L2 has nothing to gain (ViT-S 37.2 us with a fixed stride,
+    // 39.5 with), nor have 128-wide tiles, bound by their operands (d 384: 139 both).
+    constexpr long long CLC_MIN_BYTES = 256LL << 20;
+    if (wide && max_tiles * BM * BN * 2 >= CLC_MIN_BYTES) return go(launch<256, MODE_WGRAD, true, true, EPI_STORE, true>);
     return wide ? go(launch<256, MODE_WGRAD, true, true, EPI_STORE>)
                 : go(launch<128, MODE_WGRAD, true, true, EPI_STORE>);
 }
