@@ -11,7 +11,7 @@ import copy
 
 import torch
 
-from . import (VMOE_BF16, vmoe_combine, vmoe_dispatch, vmoe_expert_bwd,
+from . import (VMOE_BF16, _stream, vmoe_combine, vmoe_dispatch, vmoe_expert_bwd,
                vmoe_expert_bwd_workspace_size, vmoe_expert_fwd, vmoe_problem_capacity, vmoe_route,
                vmoe_router_bwd)
 
@@ -66,7 +66,7 @@ class StepRunner:
         self.b = bufs if bufs is not None else Buffers(p, inputs["x"].device)
 
     def forward(self, stream=None):
-        p, i, b = self.p, self.inp, self.b
+        p, i, b, stream = self.p, self.inp, self.b, _stream(stream)
         vmoe_route(p, i["x"], i["w_router"], i.get("bias"), b.logits, b.idx, b.gate, b.slot,
                    b.load, stream)
         vmoe_dispatch(p, i["x"], None, b.idx, b.slot, b.load, b.xe, stream)
@@ -74,7 +74,7 @@ class StepRunner:
         vmoe_combine(p, b.ye, b.gate, b.idx, b.slot, b.y, stream)
 
     def backward(self, stream=None):
-        p, i, b = self.p, self.inp, self.b
+        p, i, b, stream = self.p, self.inp, self.b, _stream(stream)
         vmoe_dispatch(p, i["dy"], b.gate, b.idx, b.slot, b.load, b.dye, stream)
         vmoe_expert_bwd(p, b.xe, b.h, b.a, i["w1"], i["w2"], b.dye, b.load, b.dxe, b.dw1, b.dw2,
                         b.workspace, stream=stream)
@@ -88,6 +88,7 @@ class StepRunner:
                         b.dgate, b.dlogits, b.dw_router, b.dbias, b.dx, stream)
 
     def step(self, stream=None):
+        stream = _stream(stream)
         self.forward(stream)
         self.backward(stream)
 

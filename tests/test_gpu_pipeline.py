@@ -43,3 +43,20 @@ def test_pipeline_matches_in_order_steps():
         assert torch.equal(outs[i][0], ref.b.y.cpu()), i
         assert torch.equal(outs[i][1], ref.b.dx.cpu()), i
     assert vm.vmoe_device_status() == 0
+
+
+def test_calls_follow_the_current_stream():
+    """With no stream argument a call goes to torch's current stream: work queued there before it is seen, on the
+    default stream and on another one."""
+    import paper_2608_16188_gb300 as vm
+    p = vm.problem(1, 64, 256, 128, 4, 2, 4.0, "bf16", flags=vm.VMOE_LOGITS_IN)
+    for side in (None, torch.cuda.Stream()):
+        with torch.cuda.stream(side):
+            assert vm._stream(None) == torch.cuda.current_stream().cuda_stream
+            logits = torch.zeros(1, 64, 4, device="cuda")
+            out = [torch.empty(1, 64, 2, dtype=d, device="cuda") for d in (torch.int32, torch.float32, torch.int32)]
+            load = torch.empty(1, 4, dtype=torch.int32, device="cuda")
+            torch.cuda._sleep(2_000_000)
+            logits[..., 3] = 1.0
+            vm.vmoe_route(p, None, None, None, logits, *out, load)
+            assert load.tolist() == [[64, 0, 0, 64]]
