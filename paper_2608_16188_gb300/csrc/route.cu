@@ -17,10 +17,13 @@
 // per-warp expert counters in shared memory; a per-expert exclusive scan over
 // the warps then gives the global rank, which becomes the slot (or -1 once it
 // reaches C).  No atomics, so the result is deterministic.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "common.cuh"
 #include "topk.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace vmoe {
 namespace {
@@ -171,17 +174,12 @@ route_f32_kernel(Dims p, const float *__restrict__ x, const float *__restrict__ 
 // W_lo = bf16(W - W_hi - W_mid), together about 24 significant bits): every
 // partial product is exact in fp32 and the mma.sync m16n8k16 instructions
 // accumulate in fp32, so the logits keep fp32 accuracy at a small fraction of
-// the CUDA-core instruction count.  One CTA = 4 warps x 16 tokens of one task;
+// the CUDA-core instruction count.  One CTA = 4 groups of 16 tokens of one task;
 // d is swept in chunks of RM_KC staged in shared memory.  The weight split is
 // done while staging, two values per conversion, into [part][expert][k]
 // tiles, so that one ldmatrix.x4 gives the B fragments of two 8-expert blocks
 // (and one gives a warp's A fragment).
-constexpr int RM_TOK = 64;
-constexpr int RM_THREADS = 128;
-#ifndef VMOE_ROUTE_KC
-#define VMOE_ROUTE_KC 128
-#endif
-constexpr int RM_KC = VMOE_ROUTE_KC;  // d per staged chunk: 128 halves the chunk chain of 64
+constexpr int RM_KC = 128;        // d per staged chunk
 constexpr int RM_XP = RM_KC + 8;  // row pitch (bf16) of the x and weight tiles: conflict-free ldmatrix
 
 __device__ __forceinline__ void rm_ldsm_x4(uint32_t (&r)[4], const void *smem) {
@@ -191,39 +189,65 @@ __device__ __forceinline__ void rm_ldsm_x4(uint32_t (&r)[4], const void *smem) {
                  : "r"(a));
 }
 
-// NB blocks of 8 experts per pass (NB even).
-template <int NB>
-__global__ void __launch_bounds__(RM_THREADS, 3)
-route_mma_kernel(Dims p, const __nv_bfloat16 *__restrict__ x, const float *__restrict__ wr,
+// NB blocks of 8 experts per pass (NB even); 4 groups of 16 tokens and KS slices
+// of each chunk's k steps: 4 KS warps.  KS = 2 for more than 32 experts, whose
+// weights take 128 threads twice as long to stage (8 tasks of 1576 tokens, d 1024,
+// 64 experts: 49.5 -> 42 us; 17 tasks, d 768, 32 experts: 31.8 -> 43.4, so not there).
+//
+// `split`: that many CTAs (a cluster) share a token tile, each with a range of
+// the chunks; their partial logits are summed through distributed shared memory
+// in rank order and each finishes a share of the tokens.  A chunk is a chain of
+// a load from DRAM, the split of the weights and the MMAs, 2 us long; few
+// tokens leave nothing else to run behind it.  Measured on GB300: 4 tasks of 197
+// tokens, d 768, 32 experts 20.5 -> 16.4 us; 2 of 300, d 1024, 64 experts (with
+// KS = 2) 40.7 -> 12.4 us.
+template <int NB, int KS>
+struct RouteMma {
+    static constexpr int TG = 4, TOK = 16 * TG, NT = 32 * TG * KS, NP = 8 * NB;
+    static constexpr int PARTS = (KS - 1) * TOK * NP;  // floats, over the tiles after the last chunk
+    static constexpr size_t TILES = (size_t)TOK * RM_XP * 2 + (size_t)3 * NP * RM_XP * 2;
+    static constexpr size_t smem(int E) { return TILES + (size_t)TOK * (E + 1) * 4; }
+    static_assert((size_t)(PARTS + TOK * NP) * 4 <= TILES, "partial sums reuse the tiles");
+};
+
+template <int NB, int KS, bool SPLIT>
+__global__ void __launch_bounds__(RouteMma<NB, KS>::NT, KS == 1 ? 3 : 2)
+route_mma_kernel(Dims p, int nsplit, const __nv_bfloat16 *__restrict__ x, const float *__restrict__ wr,
                  const float *__restrict__ bias, float *__restrict__ logits,
                  int32_t *__restrict__ out_idx, float *__restrict__ out_gate) {
     static_assert(NB % 2 == 0, "B fragments are loaded two expert blocks at a time");
+    using S = RouteMma<NB, KS>;
+    constexpr int NP = S::NP, NT = S::NT, TOK = S::TOK, TG = S::TG;
     pdl_wait();
-    constexpr int NP = NB * 8;
     extern __shared__ __align__(16) uint8_t rm_smem[];
-    __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(rm_smem);  // [64][RM_XP]
-    __nv_bfloat16 *ws = xs + RM_TOK * RM_XP;                         // [3][NP][RM_XP]
-    float *lg = reinterpret_cast<float *>(ws + 3 * NP * RM_XP);      // [64][E+1]
-    const int t = blockIdx.y, n0 = blockIdx.x * RM_TOK;
+    __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(rm_smem);  // [TOK][RM_XP]
+    __nv_bfloat16 *ws = xs + TOK * RM_XP;                            // [3][NP][RM_XP]
+    float *part = reinterpret_cast<float *>(rm_smem);                // [KS - 1][TOK][NP]
+    float *red = part + S::PARTS;                                    // [TOK][NP]: this CTA's sums (split > 1)
+    const int split = SPLIT ? nsplit : 1, rank = SPLIT ? (int)(blockIdx.x % split) : 0;
+    const int t = blockIdx.y, n0 = (int)(SPLIT ? blockIdx.x / split : blockIdx.x) * TOK;
     const int E = p.E, d = p.d, N = p.N;
     const int ldl = E + 1;
+    float *lg = reinterpret_cast<float *>(rm_smem + S::TILES);  // [TOK][E+1]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tg = warp % TG, sl = warp / TG;
     const int g = lane >> 2, tq = lane & 3;
-    const int ntok = min(RM_TOK, N - n0);
+    const int ntok = min(TOK, N - n0);
     const __nv_bfloat16 *xt = x + ((long long)t * N + n0) * d;
     const float *wt = wr + (long long)t * d * E;
     // Per thread and chunk: XV x vectors (16 B each) and WI weight items, an
     // item being 8 consecutive k of one expert.  The next chunk's values are
     // loaded into registers before the current chunk's MMAs run, so global
     // latency overlaps the tensor-core work.
-    constexpr int XV = RM_TOK * (RM_KC / 8) / RM_THREADS;
-    constexpr int WI = (RM_KC / 8) * NP / RM_THREADS;
+    constexpr int XV = TOK * (RM_KC / 8) / NT;
+    constexpr int WI = (RM_KC / 8) * NP / NT;
+    static_assert(XV >= 1 && WI >= 1, "every thread stages a vector of each tile");
     uint4 xv[XV];
     float wv[WI][8];
     auto load_chunk = [&](int e0, int k0) {
 #pragma unroll
         for (int q = 0; q < XV; ++q) {
-            const int i = tid + q * RM_THREADS;
+            const int i = tid + q * NT;
             const int r = i / (RM_KC / 8), c = (i % (RM_KC / 8)) * 8;
             xv[q] = make_uint4(0, 0, 0, 0);
             if (r < ntok && k0 + c < d)
@@ -231,7 +255,7 @@ route_mma_kernel(Dims p, const __nv_bfloat16 *__restrict__ x, const float *__res
         }
 #pragma unroll
         for (int q = 0; q < WI; ++q) {  // consecutive threads: consecutive experts (coalesced)
-            const int i = tid + q * RM_THREADS;
+            const int i = tid + q * NT;
             const int n = i % NP, e = e0 + n, kk = k0 + (i / NP) * 8;
 #pragma unroll
             for (int r = 0; r < 8; ++r)
@@ -241,13 +265,13 @@ route_mma_kernel(Dims p, const __nv_bfloat16 *__restrict__ x, const float *__res
     auto stage_chunk = [&]() {
 #pragma unroll
         for (int q = 0; q < XV; ++q) {
-            const int i = tid + q * RM_THREADS;
+            const int i = tid + q * NT;
             const int r = i / (RM_KC / 8), c = (i % (RM_KC / 8)) * 8;
             *reinterpret_cast<uint4 *>(xs + r * RM_XP + c) = xv[q];
         }
 #pragma unroll
         for (int q = 0; q < WI; ++q) {
-            const int i = tid + q * RM_THREADS;
+            const int i = tid + q * NT;
             const int n = i % NP, c = (i / NP) * 8;
             uint32_t hi[4], mid[4], lo[4];
 #pragma unroll
@@ -267,24 +291,28 @@ route_mma_kernel(Dims p, const __nv_bfloat16 *__restrict__ x, const float *__res
             *reinterpret_cast<uint4 *>(ws + (2 * NP + n) * RM_XP + c) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         }
     };
-    // ldmatrix row addresses: A, rows warp*16 + (lane & 15), k offset 8 (lane >> 4);
+    // ldmatrix row addresses: A, rows tg*16 + (lane & 15), k offset 8 (lane >> 4);
     // B, expert (lane & 7) + 8 (lane >> 4) of a block pair, k offset 8 ((lane >> 3) & 1)
-    const __nv_bfloat16 *xa = xs + (warp * 16 + (lane & 15)) * RM_XP + (lane >> 4) * 8;
+    const __nv_bfloat16 *xa = xs + (tg * 16 + (lane & 15)) * RM_XP + (lane >> 4) * 8;
     const __nv_bfloat16 *wb = ws + ((lane & 7) + (lane >> 4) * 8) * RM_XP + ((lane >> 3) & 1) * 8;
+    const int chunks = (d + RM_KC - 1) / RM_KC;
+    const int k_beg = SPLIT ? chunks * rank / split * RM_KC : 0;
+    const int k_end = SPLIT ? min(d, chunks * (rank + 1) / split * RM_KC) : d;
     for (int e0 = 0; e0 < E; e0 += NP) {
         float acc[NB][4];
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[nb][i] = 0.0f;
-        load_chunk(e0, 0);
-        for (int k0 = 0; k0 < d; k0 += RM_KC) {
-            __syncthreads();  // the previous chunk's fragments have been read
+        load_chunk(e0, k_beg);  // a rank has at least one chunk
+        for (int k0 = k_beg; k0 < k_end; k0 += RM_KC) {
+            __syncthreads();  // the previous chunk's fragments (or the last pass's parts) have been read
             stage_chunk();
             __syncthreads();
-            if (k0 + RM_KC < d) load_chunk(e0, k0 + RM_KC);
+            if (k0 + RM_KC < k_end) load_chunk(e0, k0 + RM_KC);
 #pragma unroll
-            for (int ks = 0; ks < RM_KC; ks += 16) {
+            for (int kq = 0; kq < RM_KC / 16 / KS; ++kq) {
+                const int ks = (sl * (RM_KC / 16 / KS) + kq) * 16;
                 uint32_t a[4];
                 rm_ldsm_x4(a, xa + ks);
 #pragma unroll
@@ -300,37 +328,115 @@ route_mma_kernel(Dims p, const __nv_bfloat16 *__restrict__ x, const float *__res
                 }
             }
         }
+        // the slices' partial sums, in slice order
+        if (KS > 1 || SPLIT) __syncthreads();
+        if (KS > 1) {
+            if (sl > 0) {
 #pragma unroll
-        for (int nb = 0; nb < NB; ++nb)
+                for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int r = warp * 16 + g + (i >> 1) * 8;
-                const int e = e0 + nb * 8 + 2 * tq + (i & 1);
-                if (r < ntok && e < E) lg[r * ldl + e] = acc[nb][i] + (bias ? bias[(long long)t * E + e] : 0.0f);
+                    for (int i = 0; i < 4; i += 2)
+                        *reinterpret_cast<float2 *>(part + ((sl - 1) * TOK + tg * 16 + g + (i >> 1) * 8) * NP + nb * 8 +
+                                                    2 * tq) = make_float2(acc[nb][i], acc[nb][i + 1]);
             }
+            __syncthreads();
+        }
+        if (sl == 0) {
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = tg * 16 + g + (i >> 1) * 8;
+                    const int n = nb * 8 + 2 * tq + (i & 1), e = e0 + n;
+                    float v = acc[nb][i];
+#pragma unroll
+                    for (int q = 1; q < KS; ++q) v += part[((q - 1) * TOK + r) * NP + n];
+                    if (SPLIT)
+                        red[r * NP + n] = v;
+                    else if (r < ntok && e < E)
+                        lg[r * ldl + e] = v + (bias ? bias[(long long)t * E + e] : 0.0f);
+                }
+        }
+        if (SPLIT) {  // this rank's tokens: rank, rank + split, ...
+            cg::cluster_group cluster = cg::this_cluster();
+            cluster.sync();
+            const int mine = (ntok - rank + split - 1) / split;
+            for (int i = tid; i < mine * NP; i += NT) {
+                const int r = rank + i / NP * split, n = i % NP, e = e0 + n;
+                if (e >= E) continue;
+                float v = 0.0f;
+                for (int q = 0; q < split; ++q) v += cluster.map_shared_rank(red, q)[r * NP + n];
+                lg[r * ldl + e] = v + (bias ? bias[(long long)t * E + e] : 0.0f);
+            }
+            cluster.sync();  // the sums stay until every rank has read them
+        }
     }
     __syncthreads();
-    for (int i = tid; i < ntok * E; i += RM_THREADS) {
+    if (SPLIT) {
+        const int mine = (ntok - rank + split - 1) / split;
+        for (int i = tid; i < mine * E; i += NT) {
+            const int r = rank + i / E * split, e = i % E;
+            logits[((long long)t * N + n0 + r) * E + e] = lg[r * ldl + e];
+        }
+        // a warp takes a row in about 1000 cycles, a thread in about 60 E, all rows at once
+        if ((mine + NT / 32 - 1) / (NT / 32) * 16 <= E) {
+            for (int r = rank + warp * split; r < ntok; r += NT / 32 * split)
+                topk_row_warp(p, lg + r * ldl, (long long)t * N + n0 + r, out_idx, out_gate);
+        } else {
+            for (int i = tid; i < mine; i += NT) {
+                const int r = rank + i * split;
+                topk_row(p, lg + r * ldl, (long long)t * N + n0 + r, out_idx, out_gate);
+            }
+        }
+        return;
+    }
+    for (int i = tid; i < ntok * E; i += NT) {
         const int r = i / E, e = i - r * E;
         logits[((long long)t * N + n0 + r) * E + e] = lg[r * ldl + e];
     }
-    topk_rows(p, lg, ldl, ntok, t, n0, out_idx, out_gate, RM_THREADS);
+    topk_rows(p, lg, ldl, ntok, t, n0, out_idx, out_gate, NT);
 }
 
-template <int NB>
+template <int NB, int KS>
 int launch_mma_router(const Dims &p, const __nv_bfloat16 *x, const float *wr, const float *bias,
                       float *logits, int32_t *idx, float *gate, cudaStream_t s) {
-    constexpr int NP = NB * 8;
-    size_t smem = (size_t)RM_TOK * RM_XP * 2 + (size_t)3 * NP * RM_XP * 2 + (size_t)RM_TOK * (p.E + 1) * 4;
+    using S = RouteMma<NB, KS>;
+    const size_t smem = S::smem(p.E);
     if (smem > 227 * 1024) return VMOE_ERR_UNSUPPORTED;
-    static std::atomic<int> smem_limit[64];  // the size depends on E
-    if (const int st = raise_smem_limit((const void *)route_mma_kernel<NB>, smem_limit, (int)smem)) return st;
-    dim3 grid((p.N + RM_TOK - 1) / RM_TOK, p.T);
+    // as many CTAs a tile as its chunks allow, while every SM has at most one; three
+    // or fewer do not pay for the cluster (1 task of 197 tokens, d 384: 12.2 -> 13.1
+    // us; 3 of 971, d 640: 17.0 -> 18.6)
+    const long long tiles = (long long)((p.N + S::TOK - 1) / S::TOK) * p.T;
+    int split = (p.d + RM_KC - 1) / RM_KC;
+    if (split > 8) split = 8;
+    while (split > 1 && tiles * split > num_sms()) --split;
+    if (split < 4) split = 1;
+    auto kern = split > 1 ? route_mma_kernel<NB, KS, true> : route_mma_kernel<NB, KS, false>;
+    static std::atomic<int> smem_limit[2][64];  // the size depends on E
+    if (const int st = raise_smem_limit((const void *)kern, smem_limit[split > 1], (int)smem)) return st;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((p.N + S::TOK - 1) / S::TOK * split), p.T);
+    cfg.blockDim = dim3(S::NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (split > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = split;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
+    if (pdl_enabled()) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
     trace_before(s, "route_topk");
-    const int st = launch_kernel(route_mma_kernel<NB>, grid, dim3(RM_THREADS), smem, s, p, x, wr, bias,
-                                 logits, idx, gate);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p, split, x, wr, bias, logits, idx, gate);
     trace_after(s);
-    return st;
+    return e == cudaSuccess ? VMOE_OK : VMOE_ERR_CUDA;
 }
 
 // SMEM_IDX: the task's idx array and the temporary ranks live in shared memory
@@ -464,8 +570,8 @@ int launch_route(const Dims &p, const void *x, const float *w_router, const floa
         if (route_tc_enabled() && route_tc_width(p) > 0)
             st = launch_route_tc(p, xb, w_router, bias, logits, idx, gate, s);
         else
-            st = p.E <= 32 ? launch_mma_router<4>(p, xb, w_router, bias, logits, idx, gate, s)
-                           : launch_mma_router<8>(p, xb, w_router, bias, logits, idx, gate, s);
+            st = p.E <= 32 ? launch_mma_router<4, 1>(p, xb, w_router, bias, logits, idx, gate, s)
+                           : launch_mma_router<8, 2>(p, xb, w_router, bias, logits, idx, gate, s);
     } else if (x == nullptr) {
         st = launch_given(p, logits, idx, gate, s);
     } else {

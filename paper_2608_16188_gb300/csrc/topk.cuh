@@ -64,4 +64,66 @@ __device__ __forceinline__ void topk_row(const Dims &p, const float *row, long l
         }
 }
 
+// The same row by a whole warp, lane l holding the logits of experts l, l + 32,
+// ... (E <= 256): a few hundred cycles of shuffles instead of a thread's k + 2
+// passes over the row, where a CTA has few rows.
+__device__ __forceinline__ void topk_row_warp(const Dims &p, const float *row, long long tok,
+                                              int32_t *__restrict__ out_idx, float *__restrict__ out_gate) {
+    constexpr int M = 8;  // 256 / 32
+    const int E = p.E, lane = threadIdx.x & 31;
+    float v[M], mx = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        const int e = lane + 32 * i;
+        const float x = e < E ? row[e] : -INFINITY;
+        v[i] = isnan(x) ? -INFINITY : x;
+        mx = fmaxf(mx, v[i]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    float sum = 0.0f;
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+        if (lane + 32 * i < E) sum += expf(v[i] - mx);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    unsigned taken = 0;  // this lane's logits already picked
+    float mine = 0.0f, kept = 0.0f;
+    int my_e = 0;
+    for (int j = 0; j < p.k; ++j) {
+        // the largest logit left, the lowest expert among equals
+        float bv = -INFINITY;
+        int be = 1 << 30;
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            const int e = lane + 32 * i;
+            if (e < E && !((taken >> i) & 1u) && (be == 1 << 30 || v[i] > bv)) {
+                bv = v[i];
+                be = e;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+            const int oe = __shfl_xor_sync(0xffffffffu, be, o);
+            // a lane with nothing left carries be = 2^30, which loses to any expert at -inf
+            if (ov > bv || (ov == bv && oe < be)) {
+                bv = ov;
+                be = oe;
+            }
+        }
+        if ((be & 31) == lane) taken |= 1u << (be >> 5);
+        const float ev = expf(bv - mx);
+        kept += ev;
+        if (lane == j) {
+            mine = ev;
+            my_e = be;
+        }
+    }
+    if (lane < p.k) {
+        out_idx[tok * p.k + lane] = my_e;
+        out_gate[tok * p.k + lane] = (p.flags & VMOE_NO_RENORM) ? mine / sum : mine / kept;
+    }
+}
+
 }  // namespace vmoe
