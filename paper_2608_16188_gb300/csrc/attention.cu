@@ -23,7 +23,7 @@
 // The tiles arrive by cp.async; in the forward and the dQ kernel, one commit
 // group per block of 64 keys, so the work on block j overlaps the copies of the
 // blocks after it (dK/dV and the fused backward wait for all of theirs: their
-// operand scales span every row).  The dQ kernel of groups above 128 tokens
+// operand scales span every row).  The dQ kernel of groups above 256 tokens
 // keeps bf16 operands and takes dS as a bf16 value plus its bf16 residual, two
 // products.  In fp16, every query block's CTA would scale the whole of K and V
 // (measured at 8 tasks and C 248: 245 us with the residual, against 297 us
@@ -204,9 +204,10 @@ __device__ __forceinline__ void at_zero(float (&acc)[NT][4]) {
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
 }
 
-// Writes a warp's 16 x 64 accumulator (times `mul`) as bf16 to rows row0.. of
+// Writes a warp's 16 x 8 NTL accumulator (times `mul`) as bf16 to rows row0.. of
 // dst (row stride ld, column col), rows at or past `valid` skipped.
-__device__ __forceinline__ void at_store(const float (&acc)[8][4], float mul, __nv_bfloat16 *dst, int ld, int row0,
+template <int NTL>
+__device__ __forceinline__ void at_store(const float (&acc)[NTL][4], float mul, __nv_bfloat16 *dst, int ld, int row0,
                                          int valid, int col) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -214,7 +215,7 @@ __device__ __forceinline__ void at_store(const float (&acc)[8][4], float mul, __
         const int r = row0 + g + 8 * h;
         if (r >= valid) continue;
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
+        for (int nt = 0; nt < NTL; ++nt)
             *reinterpret_cast<uint32_t *>(dst + (long long)r * ld + col + nt * 8 + 2 * t) =
                 pack_bf16x2(acc[nt][2 * h] * mul, acc[nt][2 * h + 1] * mul);
     }
@@ -588,31 +589,40 @@ __global__ void __launch_bounds__(AT_THREADS, AT_MIN_CTAS_BWD) attn_bwd_dkv_kern
     at_store(dv, sc.dv, dst, ld, k0 + warp * 16, L, (2 * H + h) * AT_DK);
 }
 
-// ------------------------------------------------------------------ backward, groups of <= 128 tokens
-// One CTA of 8 warps per (head, group) with L <= 128: S, P, dP and dS are formed
-// once for all queries and keys instead of in both kernels above.  Warp w owns
-// queries [16 w, 16 w + 16).  Per block of 64 keys: S = Q K^T, dP = dO V^T,
-// P = exp(S / sqrt(dk) - lse), dS = P (dP - D) (zero for queries or keys past
-// L), dQ += dS K in registers; P and dS (fp16, as the MMAs round them) go to
-// shared memory, and warps 0-3 form dV = P^T dO and warps 4-7 dK = dS^T Q for
-// the block's 64 keys (16 a warp), summed over the queries in increasing order.
-constexpr int AF_THREADS = 256;
-constexpr int AF_ROWS = 128;
+// ------------------------------------------------------------------ backward, groups of <= 256 tokens
+// One CTA of ROWS / 16 warps per (head, group) with L <= ROWS (128 or 256): S, P,
+// dP and dS are formed once for all queries and keys instead of in both kernels
+// above.  Warp w owns queries [16 w, 16 w + 16).  Per block of 64 keys: S = Q K^T,
+// dP = dO V^T, P = exp(S / sqrt(dk) - lse), dS = P (dP - D) (zero for queries or
+// keys past L), dQ += dS K in registers; P and dS (fp16, as the MMAs round them)
+// go to shared memory, and half of the warps form dV = P^T dO and half dK = dS^T Q
+// for the block's 64 keys, summed over the queries in increasing order.  With 256
+// rows dQ takes dS as an fp16 value and its fp16 residual, as the dQ kernel of
+// larger groups takes it as two bf16 values.
+// Rows, keys and queries past the load rounded up to 32 (16 for the queries) are
+// neither loaded nor multiplied: loads vary from group to group.
+// Measured on GB300 (us): 17 tasks, 12 heads, C 124: 304 with every row of the
+// block, 270 trimmed to the load; 8 tasks, C 247 (256 rows, one CTA of 16 warps an
+// SM): 143 + 186 in the two kernels, 250 in this one.  What is left is a chain per
+// CTA -- copies, maxima, conversion, products -- with two CTAs an SM to overlap it
+// (a stream of its 482 MB at C 124 takes 71).
+constexpr int AF_MAX_ROWS = 256;
 
-// acc[8][4] (16 keys x 64) += A^T B: A = 16 key columns (from acol) of a shared
-// [query][key] tile, B = a shared [query][64] tile, over queries [0, nq) in
-// steps of 16 (A fragments by ldmatrix.trans: A's rows are the tile's columns);
-// fp16 operands.
-__device__ __forceinline__ void at_mma_tb(float (&acc)[8][4], const __nv_bfloat16 *atile, int acol,
-                                          const __nv_bfloat16 *btile, int nq) {
+// acc[4 NDP / 2 ...] += A^T B: A = 16 key columns (from acol) of a shared
+// [query][key] tile, B = columns [16 dp0, 16 (dp0 + NDP)) of a shared [query][64]
+// tile, over queries [0, nq) in steps of 16 (A fragments by ldmatrix.trans: A's
+// rows are the tile's columns); fp16 operands.
+template <int NDP>
+__device__ __forceinline__ void at_mma_tb(float (&acc)[2 * NDP][4], const __nv_bfloat16 *atile, int acol,
+                                          const __nv_bfloat16 *btile, int dp0, int nq) {
     const int lane = threadIdx.x & 31, m = lane >> 3;
     for (int q0 = 0; q0 < nq; q0 += 16) {
         uint32_t a[4];
         at_ldsm_x4_t(a, atile + (q0 + (lane & 7) + (lane >> 4) * 8) * AT_PITCH + acol + (m & 1) * 8);
 #pragma unroll
-        for (int dp = 0; dp < 4; ++dp) {
+        for (int dp = 0; dp < NDP; ++dp) {
             uint32_t b[4];
-            at_ldsm_x4_t(b, btile + (q0 + (m & 1) * 8 + (lane & 7)) * AT_PITCH + dp * 16 + (m >> 1) * 8);
+            at_ldsm_x4_t(b, btile + (q0 + (m & 1) * 8 + (lane & 7)) * AT_PITCH + (dp0 + dp) * 16 + (m >> 1) * 8);
             at_mma<true>(acc[2 * dp], a[0], a[1], a[2], a[3], b[0], b[1]);
             at_mma<true>(acc[2 * dp + 1], a[0], a[1], a[2], a[3], b[2], b[3]);
         }
@@ -632,69 +642,83 @@ __device__ __forceinline__ void at_put(__nv_bfloat16 *tile, int row0, int col0, 
                 at_pack<true>(v[nt][2 * h], v[nt][2 * h + 1]);
 }
 
-__global__ void __launch_bounds__(AF_THREADS, 2) attn_bwd_fused_kernel(AtArgs a) {
+template <int ROWS>
+__global__ void __launch_bounds__(2 * ROWS, ROWS == 128 ? 2 : 1) attn_bwd_fused_kernel(AtArgs a) {
+    constexpr int NT = 2 * ROWS, W = ROWS / 16;
     pdl_wait();
     const int h = blockIdx.y, g = blockIdx.z;
     const int L = clamp_load(a.load, g, a.C);
     if (L == 0) return;
-    const int Lp = (L + AT_BLK - 1) / AT_BLK * AT_BLK;  // 64 or 128
+    const int L32 = (L + 31) & ~31, L16 = (L + 15) & ~15;
     const int H = a.H, ld = 3 * H * AT_DK, ldo = H * AT_DK;
     extern __shared__ __align__(16) __nv_bfloat16 at_smem[];
-    __nv_bfloat16 *qs = at_smem, *ks = qs + AF_ROWS * AT_PITCH, *vs = ks + AF_ROWS * AT_PITCH;
-    __nv_bfloat16 *dos = vs + AF_ROWS * AT_PITCH;
-    __nv_bfloat16 *ps = dos + AF_ROWS * AT_PITCH, *dss = ps + AF_ROWS * AT_PITCH;  // one 64-key block
-    float *dsh = reinterpret_cast<float *>(dss + AF_ROWS * AT_PITCH), *lse_s = dsh + AF_ROWS;
-    uint32_t *red = reinterpret_cast<uint32_t *>(lse_s + AF_ROWS);  // [5][8] block maxima
+    __nv_bfloat16 *qs = at_smem, *ks = qs + ROWS * AT_PITCH, *vs = ks + ROWS * AT_PITCH;
+    __nv_bfloat16 *dos = vs + ROWS * AT_PITCH;
+    __nv_bfloat16 *ps = dos + ROWS * AT_PITCH, *dss = ps + ROWS * AT_PITCH;  // one 64-key block
+    float *dsh = reinterpret_cast<float *>(dss + ROWS * AT_PITCH), *lse_s = dsh + ROWS;
+    uint32_t *red = reinterpret_cast<uint32_t *>(lse_s + ROWS);  // [5][W] block maxima
     const __nv_bfloat16 *src = a.qkv + (long long)g * a.C * ld;
     const long long ob = (long long)g * a.C * ldo;
-    at_cp_rows_n<AF_THREADS>(ps, a.o + ob, ldo, 0, AF_ROWS, L, h * AT_DK);
-    at_cp_rows_n<AF_THREADS>(qs, src, ld, 0, AF_ROWS, L, h * AT_DK);
-    at_cp_rows_n<AF_THREADS>(dos, a.dout + ob, ldo, 0, AF_ROWS, L, h * AT_DK);
-    at_cp_rows_n<AF_THREADS>(ks, src, ld, 0, AF_ROWS, L, (H + h) * AT_DK);
-    at_cp_rows_n<AF_THREADS>(vs, src, ld, 0, AF_ROWS, L, (2 * H + h) * AT_DK);
+    at_cp_rows_n<NT>(ps, a.o + ob, ldo, 0, L32, L, h * AT_DK);
+    at_cp_rows_n<NT>(qs, src, ld, 0, L32, L, h * AT_DK);
+    at_cp_rows_n<NT>(dos, a.dout + ob, ldo, 0, L32, L, h * AT_DK);
+    at_cp_rows_n<NT>(ks, src, ld, 0, L32, L, (H + h) * AT_DK);
+    at_cp_rows_n<NT>(vs, src, ld, 0, L32, L, (2 * H + h) * AT_DK);
     at_cp_commit();
-    for (int i = threadIdx.x; i < AF_ROWS; i += AF_THREADS)
+    for (int i = threadIdx.x; i < L32; i += NT)
         lse_s[i] = i < L ? __ldg(a.lse + ((long long)g * H + h) * a.C + i) : 0.0f;
     at_cp_wait(0);
-    uint32_t mx[5];
+    uint32_t mx[5] = {0, 0, 0, 0, 0};
     {
+        // D: two threads per row, 32 columns each, summed in column order
         const int r = threadIdx.x >> 1, c0 = (threadIdx.x & 1) * 32;
         float acc = 0.0f;
-#pragma unroll 8
-        for (int c = 0; c < 32; ++c)
-            acc += __bfloat162float(dos[r * AT_PITCH + c0 + c]) * __bfloat162float(ps[r * AT_PITCH + c0 + c]);
+        if (r < L32) {
+#pragma unroll
+            for (int c = 0; c < 32; c += 8) {
+                float x[8], y[8];
+                bf16x8_to_f32(*reinterpret_cast<const uint4 *>(dos + r * AT_PITCH + c0 + c), x);
+                bf16x8_to_f32(*reinterpret_cast<const uint4 *>(ps + r * AT_PITCH + c0 + c), y);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) acc = fmaf(x[q], y[q], acc);
+            }
+        }
         acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-        if ((threadIdx.x & 1) == 0) dsh[r] = acc;
+        if ((threadIdx.x & 1) == 0 && r < L32) dsh[r] = acc;
         mx[4] = __float_as_uint(fabsf(acc));
     }
-    mx[0] = at_tile_absmax<AF_THREADS>(qs, Lp);
-    mx[1] = at_tile_absmax<AF_THREADS>(ks, Lp);
-    mx[2] = at_tile_absmax<AF_THREADS>(vs, Lp);
-    mx[3] = at_tile_absmax<AF_THREADS>(dos, Lp);
-    at_block_max<5, AF_THREADS / 32>(mx, red);
+    mx[0] = at_tile_absmax<NT>(qs, L32);
+    mx[1] = at_tile_absmax<NT>(ks, L32);
+    mx[2] = at_tile_absmax<NT>(vs, L32);
+    mx[3] = at_tile_absmax<NT>(dos, L32);
+    at_block_max<5, W>(mx, red);
     const AtScales sc = at_scales(mx, a.scale);
-    at_tile_to_f16<AF_THREADS>(qs, Lp, sc.q);
-    at_tile_to_f16<AF_THREADS>(ks, Lp, sc.k);
-    at_tile_to_f16<AF_THREADS>(vs, Lp, sc.v);
-    at_tile_to_f16<AF_THREADS>(dos, Lp, sc.dO);
+    at_tile_to_f16<NT>(qs, L32, sc.q);
+    at_tile_to_f16<NT>(ks, L32, sc.k);
+    at_tile_to_f16<NT>(vs, L32, sc.v);
+    at_tile_to_f16<NT>(dos, L32, sc.dO);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & 3, g8 = lane >> 2;
     const int row0 = warp * 16;
-    float lse[2], dd[2];
+    const bool active = row0 < L;  // this warp has queries
+    float lse[2] = {0.0f, 0.0f}, dd[2] = {0.0f, 0.0f};
     bool rv[2];
 #pragma unroll
     for (int h2 = 0; h2 < 2; ++h2) {
         const int r = row0 + g8 + 8 * h2;
         rv[h2] = r < L;
-        lse[h2] = lse_s[r];
-        dd[h2] = dsh[r] * sc.d;
+        if (active) {
+            lse[h2] = lse_s[r];
+            dd[h2] = dsh[r] * sc.d;
+        }
     }
     float dq[8][4];
     at_zero(dq);
-    for (int kb = 0; kb < Lp; kb += AT_BLK) {
+    __nv_bfloat16 *dst = a.dqkv + (long long)g * a.C * ld;
+    for (int kb = 0; kb < L; kb += AT_BLK) {
         // in two halves of 32 keys, which holds S and dP in half the registers
 #pragma unroll 1
-        for (int k32 = 0; k32 < AT_BLK; k32 += 32) {
+        for (int k32 = 0; active && k32 < AT_BLK && kb + k32 < L; k32 += 32) {
             uint32_t fa[4][4];
             float s[4][4], dp[4][4];
             at_zero(s);
@@ -716,23 +740,35 @@ __global__ void __launch_bounds__(AF_THREADS, 2) attn_bwd_fused_kernel(AtArgs a)
             at_mma_pb<true, 4>(dq, dp, ks, kb + k32);
             at_put<4>(ps, row0, k32, s);
             at_put<4>(dss, row0, k32, dp);
+            if (ROWS > 128) {
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) dp[nt][j] -= __half2float(__float2half_rn(dp[nt][j]));
+                at_mma_pb<true, 4>(dq, dp, ks, kb + k32);
+            }
         }
         __syncthreads();
         {
-            float acc[8][4];
-            at_zero(acc);
-            const int key0 = (warp & 3) * 16;  // the warp's 16 keys of the block
-            if (warp < 4) {
-                at_mma_tb(acc, ps, key0, dos, Lp);   // dV = P^T dO
-                at_store(acc, sc.dv, a.dqkv + (long long)g * a.C * ld, ld, kb + key0, L, (2 * H + h) * AT_DK);
-            } else {
-                at_mma_tb(acc, dss, key0, qs, Lp);   // dK = dS^T Q / sqrt(dk)
-                at_store(acc, sc.dk, a.dqkv + (long long)g * a.C * ld, ld, kb + key0, L, (H + h) * AT_DK);
+            // half of the warps dV, half dK; each 16 of the 64 keys and, with 16
+            // warps, half of the 64 columns
+            constexpr int NDP = ROWS == 128 ? 4 : 2;
+            const int w = warp % (W / 2), key0 = (w & 3) * 16, dp0 = (w >> 2) * NDP;
+            if (kb + key0 < L) {
+                float acc[2 * NDP][4];
+                at_zero(acc);
+                if (warp < W / 2) {
+                    at_mma_tb<NDP>(acc, ps, key0, dos, dp0, L16);   // dV = P^T dO
+                    at_store(acc, sc.dv, dst, ld, kb + key0, L, (2 * H + h) * AT_DK + dp0 * 16);
+                } else {
+                    at_mma_tb<NDP>(acc, dss, key0, qs, dp0, L16);   // dK = dS^T Q / sqrt(dk)
+                    at_store(acc, sc.dk, dst, ld, kb + key0, L, (H + h) * AT_DK + dp0 * 16);
+                }
             }
         }
         __syncthreads();  // P and dS of this block are read; the next block rewrites them
     }
-    at_store(dq, sc.dq, a.dqkv + (long long)g * a.C * ld, ld, row0, L, h * AT_DK);
+    if (active) at_store(dq, sc.dq, dst, ld, row0, L, h * AT_DK);
 }
 
 size_t at_smem_fwd(int C) {
@@ -743,9 +779,10 @@ size_t at_smem_dq(int C) {
     const int Cp = (C + AT_BLK - 1) / AT_BLK * AT_BLK;
     return (size_t)(3 * AT_BLK + 2 * Cp) * AT_PITCH * 2 + AT_BLK * 4;
 }
-size_t at_smem_fused() {
-    return (size_t)6 * AF_ROWS * AT_PITCH * 2 + 2 * (size_t)AF_ROWS * 4 + 5 * (AF_THREADS / 32) * 4;
+constexpr size_t at_smem_fused(int rows) {
+    return (size_t)6 * rows * AT_PITCH * 2 + 2 * (size_t)rows * 4 + 5 * (rows / 16) * 4;
 }
+static_assert(at_smem_fused(AF_MAX_ROWS) <= 227 * 1024, "over the shared-memory limit");
 size_t at_smem_dkv(int C) {
     const int Cp = (C + AT_BLK - 1) / AT_BLK * AT_BLK;
     return (size_t)(2 * AT_BLK + 2 * Cp) * AT_PITCH * 2 + 2 * (size_t)Cp * 4 + 5 * (AT_THREADS / 32) * 4;
@@ -801,16 +838,17 @@ int launch_attn_core_bwd(int G, int C, int H, const int32_t *load, const __nv_bf
     a.dsum = dsum;
     a.dqkv = dqkv;
     a.scale = 1.0f / sqrtf((float)AT_DK);
-    if (C <= AF_ROWS) {  // every group fits one CTA: S, P, dP and dS formed once
-        static std::atomic<int> lim_f[64], carve_f[64];
-        const size_t smem = at_smem_fused();
-        if (const int st = raise_smem_limit((const void *)attn_bwd_fused_kernel, lim_f, (int)smem)) return st;
+    if (C <= AF_MAX_ROWS) {  // every group fits one CTA: S, P, dP and dS formed once
+        static std::atomic<int> lim_f[2][64], carve_f[2][64];
+        const int rows = C <= 128 ? 128 : AF_MAX_ROWS, v = rows > 128;
+        auto kern = v ? attn_bwd_fused_kernel<AF_MAX_ROWS> : attn_bwd_fused_kernel<128>;
+        const size_t smem = at_smem_fused(rows);
+        if (const int st = raise_smem_limit((const void *)kern, lim_f[v], (int)smem)) return st;
         int dev = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && !carve_f[dev].exchange(1))
-            cudaFuncSetAttribute((const void *)attn_bwd_fused_kernel,
-                                 cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && !carve_f[v][dev].exchange(1))
+            cudaFuncSetAttribute((const void *)kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         trace_before(s, "attn_bwd");
-        const int st = launch_kernel(attn_bwd_fused_kernel, dim3(1, H, G), dim3(AF_THREADS), smem, s, a);
+        const int st = launch_kernel(kern, dim3(1, H, G), dim3(2 * rows), smem, s, a);
         trace_after(s);
         return st;
     }
