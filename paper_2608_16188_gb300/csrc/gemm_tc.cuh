@@ -21,8 +21,7 @@
 //               The accumulator is double buffered in TMEM
 //               (2 x BN columns), so tile i's epilogue overlaps tile i+1's
 //               main loop.
-// Tiles go to CTAs with a fixed stride (CTA b takes tiles b, b + grid, ...), the
-// weight gradients' larger ones by cluster launch control.  In
+// Tiles are distributed statically: CTA b takes tiles b, b + grid, ...  In
 // row mode (H = Xe W1 etc.) a group contributes ceil(load/128) x N/BN tiles,
 // counted from the device-resident loads by every CTA with a block scan, so
 // empty groups cost nothing and no host round trip is needed.  In weight-
@@ -70,8 +69,7 @@ constexpr int ROW_CH = 32;
 template <int MODE, int EPI>
 struct Roles {
     static constexpr int EW = (MODE == 0 && EPI != EPI_STORE) ? 16 : 8;  // epilogue warps
-    // threads: A producer, MMA, epilogue, B producer; weight gradients: scheduler
-    static constexpr int NT = 96 + 32 * EW + (MODE == 1 ? 32 : 0);
+    static constexpr int NT = 96 + 32 * EW;  // threads: A producer, MMA, epilogue, B producer
     static constexpr int PITCH = 80;         // staging row pitch (bytes): 64 data + 16 pad
 };
 
@@ -123,7 +121,7 @@ struct Args {
     long long sD;              // group stride of D / D2 (elements)
     long long sAux;            // group stride of aux (elements)
     int ldd;                   // row stride of D / D2 / aux (elements)
-    int ksplit;                // weight-gradient mode: B holds [hi rows; lo rows] (K doubled)
+    int ksplit;                // weight-gradient mode, 0 or 1: B holds [hi rows; lo rows] (K doubled)
     int gelu_tanh;
     int *status;
     // Slices (the memory-budgeted backward): the launch covers G entries, entry i
@@ -246,17 +244,17 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, uint32_t sr
         : "memory");
 }
 // An empty group's weight gradient is zeros, one contiguous slab: its unit (or
-// tile) `part` of `parts` writes the slab's share by 4 KB copies of `zeros` (4 KB
-// of zeroed shared memory), `w` of `nw` warps taking every nw-th copy (called by
-// one thread).  slab: bytes, a multiple of 4096 * parts.  Against 32 x 64 boxes
-// staged and waited for one by one, the Zipf-skewed step, where two groups in
+// tile) `part` of `parts` writes its share of the slab's 4 KB pieces by copies of
+// `zeros` (4 KB of zeroed shared memory), `w` of `nw` warps taking every nw-th
+// piece (called by one thread).  slab: bytes, a multiple of 4096.  Against 32 x 64
+// boxes staged and waited for one by one, the Zipf-skewed step, where two groups in
 // three are empty, went from 2386 to 2353 us.
 __device__ __forceinline__ void store_zeros(uint8_t *slab_base, long long slab, int part, int parts, int w, int nw,
                                             uint32_t zeros, uint64_t policy) {
-    const long long n = slab / parts / 4096;
-    uint8_t *dst = slab_base + (long long)part * n * 4096;
-    for (long long i = w; i < n; i += nw)
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], 4096, %2;" ::"l"(dst + i * 4096),
+    const long long pieces = slab / 4096, end = pieces * (part + 1) / parts;
+    for (long long i = pieces * part / parts + w; i < end; i += nw)
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], 4096, %2;" ::"l"(
+                         slab_base + i * 4096),
                      "r"(zeros), "l"(policy)
                      : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -278,8 +276,8 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 // ---------------------------------------------------------------------------
-// Dynamic tiles by cluster launch control: the grid has a CTA (or pair) per
-// tile, the ones that run take the next one not yet launched
+// Dynamic tiles by cluster launch control (the SM-pair weight gradients): the grid
+// has a CTA pair per tile, the ones that run take the next one not yet launched
 // (clusterlaunchcontrol.try_cancel) instead of a fixed stride.  The tiles in
 // work are then always the oldest ones, so the addresses being written stay
 // close together; with a fixed stride the SMs drift apart and DRAM loses
@@ -510,6 +508,43 @@ __device__ __forceinline__ void zero_staging(uint8_t *stg, bool &zeroed) {
     zeroed = true;
 }
 
+// A warp's 32 rows x 64 CHUNKS columns of fp32 accumulators as bf16, 64 columns
+// at a time through its 128-byte-swizzled staging tile(s) (BUFS of 4 KB) and TMA
+// bulk tensor stores; only the first `valid` chunks.
+template <int CHUNKS, int BUFS>
+__device__ __forceinline__ void store_columns(const CUtensorMap &map, const uint32_t (&r)[2 * CHUNKS][32], uint8_t *stg,
+                                              int &nstore, int col, int row, int g, uint64_t policy,
+                                              int valid = CHUNKS) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int c = 0; c < CHUNKS; ++c) {
+        if (c >= valid) break;
+        uint8_t *buf = stg + (BUFS == 2 ? (nstore & 1) * 4096 : 0);
+        if (lane == 0 && nstore >= BUFS) {  // the store that used buf has read it
+            if (BUFS == 2) bulk_wait_read1();
+            else bulk_wait_read0();
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t *src = &r[2 * c + (j >> 2)][(j & 3) * 8];
+            uint4 pk;
+            pk.x = pack_bf16x2(__uint_as_float(src[0]), __uint_as_float(src[1]));
+            pk.y = pack_bf16x2(__uint_as_float(src[2]), __uint_as_float(src[3]));
+            pk.z = pack_bf16x2(__uint_as_float(src[4]), __uint_as_float(src[5]));
+            pk.w = pack_bf16x2(__uint_as_float(src[6]), __uint_as_float(src[7]));
+            *reinterpret_cast<uint4 *>(buf + lane * 128 + ((j ^ (lane & 7)) << 4)) = pk;
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+            tma_store_3d(&map, smem_u32(buf), col + c * 64, row, g, policy);
+            bulk_commit();
+        }
+        ++nstore;
+    }
+}
+
 struct Tile {
     int g, m_blk, n_blk, kblocks, kvalid, rows_valid;
     int khalf;  // weight-gradient mode: k-blocks per half (kblocks = 2 * khalf with ksplit)
@@ -593,9 +628,7 @@ __device__ __forceinline__ void epilogue_chunk(f32x2 (&v)[CH / 2], const uint4 *
     }
 }
 
-// CLC: tiles by cluster launch control (weight gradients only; the grid is the
-// tile count), else tiles blockIdx.x, blockIdx.x + gridDim.x, ...
-template <int BN, int MODE, bool A_MN, bool B_MN, int EPI, bool CLC>
+template <int BN, int MODE, bool A_MN, bool B_MN, int EPI>
 __global__ void __launch_bounds__(Roles<MODE, EPI>::NT, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmD2,
@@ -622,25 +655,9 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     auto bar_tempty = [&](int a) { return smem_u32(bars + 2 * STAGES + 2 + a); };
     const uint32_t bar_drain = smem_u32(bars + 2 * STAGES + 4);
     volatile int *abort_flag = misc + 1;
-    static_assert(!CLC || MODE == MODE_WGRAD, "a row-mode grid cannot be the tile count: the host does not know it");
-    __shared__ __align__(16) ClcQueue clc;
     int total = 0;
-    // The tile after u, for a role of one thread or of a whole warp.
-    auto next_tile = [&](auto warp_wide, ClcPos &pos, int &u) -> bool {
-        if (!CLC) {
-            u += (int)gridDim.x;
-            return u < total;
-        }
-        uint32_t x;
-        if (!clc_take<decltype(warp_wide)::value>(clc, pos, x, abort_flag, args.status)) return false;
-        u = (int)x;
-        return true;
-    };
-    constexpr std::true_type WARP_WIDE{};
-    constexpr std::false_type ONE_THREAD{};
 
     if (tid == 0) {
-        if (CLC) clc_init(clc, Roles<MODE, EPI>::EW + 3);
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar_full(s), 2);  // the A and the B producer's arrivals
             mbar_init(bar_empty(s), 1);
@@ -726,17 +743,11 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             int issued = 0;  // copies so far: slot s has had those of index s, s + STAGES, ...
             bool ok = true;
             const bool cmpa = (args.compact & CMP_A) != 0, cmpb = (args.compact & CMP_B) != 0;
-            ClcPos pos;
-            int u = (int)blockIdx.x;
-            bool more = u < total;
-            Tile t = decode_tile<MODE>(args, prefix, more ? u : 0);
-            while (more && ok) {
+            Tile t = decode_tile<MODE>(args, prefix, blockIdx.x < total ? blockIdx.x : 0);
+            for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
                 Tile tn = t;  // the next tile, looked up behind this one's first copy
-                auto look_up = [&]() {
-                    more = next_tile(ONE_THREAD, pos, u);
-                    if (more) tn = decode_tile<MODE>(args, prefix, u);
-                };
-                if (!CLC && isA && u + (int)gridDim.x >= total) pdl_launch_dependents();  // this CTA's last tile
+                const bool last = u + (int)gridDim.x >= total;
+                if (isA && last) pdl_launch_dependents();  // this CTA's last tile
                 // Row mode, A rows [0, rn): the tile's valid rows rounded up to 16.  The
                 // slot's rows past rn keep stale data, which only reaches output rows
                 // past rows_valid -- never stored.
@@ -781,10 +792,11 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         // K = the group's rows, in k-blocks that end at its last row: only
                         // k-block 0 is partial, and its missing rows lie before row 0, where
                         // the tensor maps read zeros (in a compact B they are a neighbour's,
-                        // and the MMA warp zeroes them).  With ksplit the second half of the
-                        // k-blocks pairs the same A rows with B's residual rows.
-                        const int hi = (kb >= t.khalf) ? 1 : 0;
-                        const int ka = k0 + (kb - hi * t.khalf) * BK;
+                        // and the MMA warp zeroes them).  With ksplit every other k-block
+                        // pairs the same A rows with B's residual rows: the order of sums of
+                        // the SM-pair kernels.
+                        const int hi = args.ksplit ? kb & 1 : 0;
+                        const int ka = k0 + (kb >> args.ksplit) * BK;
                         if (isA)
                             tma_load_4d(sa, &tmA, fb, 0, ka, t.m_blk * (BM / 64), t.gr);
                         else if (cmpb)  // residual rows follow the entry's load rows
@@ -792,14 +804,14 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         else
                             tma_load_4d(sb, hi ? &tmD2 : &tmB, fb, 0, ka, t.n_blk * (BN / 64), t.gr);
                     }
-                    if (kb == 0) look_up();
+                    if (kb == 0 && !last) tn = decode_tile<MODE>(args, prefix, u + gridDim.x);
                     ++issued;
                     if (++stage == STAGES) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
-                if (t.kblocks == 0) look_up();
+                if (t.kblocks == 0 && !last) tn = decode_tile<MODE>(args, prefix, u + gridDim.x);
                 t = tn;
             }
             if (*abort_flag) {  // let copies in flight land before the CTA exits
@@ -837,17 +849,12 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 phase ^= 1u;
             }
         };
-        ClcPos pos;
-        int u = (int)blockIdx.x;
         if (!cmpb) {
-            bool more = one && u < total;
-            Tile t;
-            if (MODE == MODE_WGRAD && more) t = decode_tile<MODE>(args, prefix, u);
-            for (; more && ok; ++it) {
-                int kblocks = args.K_fixed / BK, khalf = 0, skip = 0;
+            for (int u = blockIdx.x; one && u < total && ok; u += gridDim.x, ++it) {
+                int kblocks = args.K_fixed / BK, skip = 0;
                 if (MODE == MODE_WGRAD) {
+                    const Tile t = decode_tile<MODE>(args, prefix, u);
                     kblocks = t.kblocks;
-                    khalf = t.khalf;
                     skip = (t.khalf * BK - t.kvalid) >> 4;  // all-zero 16-row steps of k-block 0
                 }
                 const int acc = it & 1;
@@ -859,18 +866,15 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         break;
                     }
                     tc_fence_after();
-                    k_block(tmem_base + (uint32_t)(acc * BN), kb == 0 || kb == khalf ? skip : 0, kb > 0);
+                    k_block(tmem_base + (uint32_t)(acc * BN), (kb >> args.ksplit) == 0 ? skip : 0, kb > 0);
                     next_stage();
                 }
                 if (!ok) break;
                 if (kblocks == 0) mbar_arrive(bar_tfull(acc));
                 else mma_commit(bar_tfull(acc));
-                more = next_tile(ONE_THREAD, pos, u);
-                if (MODE == MODE_WGRAD && more) t = decode_tile<MODE>(args, prefix, u);
             }
         } else {  // compact B: the warp zeroes the rows of k-block 0 (both parts) that belong to a neighbour
-            bool more = u < total;
-            for (; more && ok; more = next_tile(WARP_WIDE, pos, u), ++it) {
+            for (int u = blockIdx.x; u < total && ok; u += gridDim.x, ++it) {
                 const Tile t = decode_tile<MODE>(args, prefix, u);
                 const int z = t.khalf * BK - t.kvalid;
                 const int acc = it & 1;
@@ -882,7 +886,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         break;
                     }
                     tc_fence_after();
-                    const bool first = kb == 0 || kb == t.khalf;
+                    const bool first = (kb >> args.ksplit) == 0;
                     if (first && z > 0) {
                         uint8_t *tile = smem + stage * S::STAGE_BYTES + S::A_BYTES;
                         for (int i = lane; i < (BN / 64) * z * 8; i += 32) {
@@ -913,10 +917,6 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
         }
         __syncwarp();
-    } else if (MODE == MODE_WGRAD && warp == Roles<MODE, EPI>::EW + 3) {
-        // ------------------------------------------------------------ scheduler (idle without CLC)
-        if (CLC && elect_one()) clc_scheduler<false>(clc, true, abort_flag, args.status);
-        __syncwarp();
     } else if (MODE == MODE_WGRAD) {
         // ------------------------------------------------------------ epilogue (weight gradients)
         // Every tile is full.  Each warp reads all BN/2 accumulator columns of its
@@ -932,10 +932,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         int nstore = 0;
         int it = 0;
         bool zeroed = false;  // the first staging tile holds zeros that copies in flight read
-        ClcPos pos;
-        int u = (int)blockIdx.x;
-        bool more = u < total;
-        for (; more; more = next_tile(WARP_WIDE, pos, u), ++it) {
+        for (int u = blockIdx.x; u < total; u += gridDim.x, ++it) {
             const Tile t = decode_tile<MODE>(args, prefix, u);
             const int acc = it & 1;
             const uint32_t aph = (uint32_t)((it >> 1) & 1);
@@ -966,29 +963,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_tempty(acc));  // the accumulator is in registers now
-#pragma unroll
-            for (int c = 0; c < COLS / 64; ++c) {
-                uint8_t *buf = stg + (nstore & 1) * 4096;
-                if (lane == 0 && nstore >= 2) bulk_wait_read1();  // the store that used buf has read it
-                __syncwarp();
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const uint32_t *src = &r[2 * c + (j >> 2)][(j & 3) * 8];
-                    uint4 pk;
-                    pk.x = pack_bf16x2(__uint_as_float(src[0]), __uint_as_float(src[1]));
-                    pk.y = pack_bf16x2(__uint_as_float(src[2]), __uint_as_float(src[3]));
-                    pk.z = pack_bf16x2(__uint_as_float(src[4]), __uint_as_float(src[5]));
-                    pk.w = pack_bf16x2(__uint_as_float(src[6]), __uint_as_float(src[7]));
-                    *reinterpret_cast<uint4 *>(buf + lane * 128 + ((j ^ (lane & 7)) << 4)) = pk;
-                }
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) {
-                    tma_store_3d(&tmD, smem_u32(buf), colw + c * 64, row0, t.gr, policy);
-                    bulk_commit();
-                }
-                ++nstore;
-            }
+            store_columns<COLS / 64, 2>(tmD, r, stg, nstore, colw, row0, t.gr, policy);
         }
         if (lane == 0) bulk_wait_all();
         __syncwarp();
@@ -1050,14 +1025,11 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
         };
         int it = 0;
-        ClcPos pos;
-        int u = (int)blockIdx.x;
-        bool have = u < total;
-        Tile t = decode_tile<MODE>(args, prefix, have ? u : 0);
-        if (EPI == EPI_DGELU && have) load_h(t, jw, hcur);
-        for (; have; ++it) {
-            const bool have_next = next_tile(WARP_WIDE, pos, u);
-            const Tile tn = have_next ? decode_tile<MODE>(args, prefix, u) : t;
+        Tile t = decode_tile<MODE>(args, prefix, blockIdx.x < total ? blockIdx.x : 0);
+        if (EPI == EPI_DGELU && blockIdx.x < total) load_h(t, jw, hcur);
+        for (int u = blockIdx.x; u < total; u += gridDim.x, ++it) {
+            const bool have_next = u + (int)gridDim.x < total;
+            const Tile tn = decode_tile<MODE>(args, prefix, have_next ? u + gridDim.x : u);
             const int acc = it & 1;
             const uint32_t aph = (uint32_t)((it >> 1) & 1);
             if (!wait_phase(bar_tfull(acc), aph, abort_flag, args.status)) break;
@@ -1106,7 +1078,6 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_tempty(acc));
             t = tn;
-            have = have_next;
         }
     }
 
@@ -1134,16 +1105,16 @@ bool make_map_chunked(CUtensorMap *map, const void *base, uint64_t mn, uint64_t 
                       uint64_t outer, uint32_t box_rows, uint32_t box_chunks,
                       uint64_t outer_stride_elems = 0);
 
-template <int BN, int MODE, bool A_MN, bool B_MN, int EPI, bool CLC = false>
+template <int BN, int MODE, bool A_MN, bool B_MN, int EPI>
 int launch(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &md,
            const CUtensorMap &md2, const TailMaps &mat, const Args &a, long long max_tiles,
            cudaStream_t s, const char *name) {
     using S = Shape<BN, MODE, EPI>;
-    auto kern = grouped_gemm_kernel<BN, MODE, A_MN, B_MN, EPI, CLC>;
+    auto kern = grouped_gemm_kernel<BN, MODE, A_MN, B_MN, EPI>;
     static std::atomic<int> smem_limit[64];
     if (const int st = raise_smem_limit((const void *)kern, smem_limit, (int)S::SMEM_BYTES)) return st;
     if (max_tiles <= 0) return VMOE_OK;
-    const long long grid = CLC || max_tiles < num_sms() ? max_tiles : num_sms();
+    const long long grid = max_tiles < num_sms() ? max_tiles : num_sms();
     trace_before(s, name);
     const int st = launch_kernel(kern, dim3((unsigned)grid), dim3(S::NT), S::SMEM_BYTES, s, ma, mb,
                                  md, md2, mat, a);

@@ -582,32 +582,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 __syncwarp();
                 if (lane == 0) mbar_arrive_remote(mapa_shared(bar_tempty(acc), 0));
                 ++it;
-#pragma unroll
-                for (int c = 0; c < COLS / 64; ++c) {
-                    uint8_t *buf = stg + (S::STG_BUFS == 2 ? (nstore & 1) * 4096 : 0);
-                    if (lane == 0 && nstore >= S::STG_BUFS) {
-                        if (S::STG_BUFS == 2) bulk_wait_read1();
-                        else bulk_wait_read0();
-                    }
-                    __syncwarp();
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const uint32_t *src = &r[2 * c + (j >> 2)][(j & 3) * 8];
-                        uint4 pk;
-                        pk.x = pack_bf16x2(__uint_as_float(src[0]), __uint_as_float(src[1]));
-                        pk.y = pack_bf16x2(__uint_as_float(src[2]), __uint_as_float(src[3]));
-                        pk.z = pack_bf16x2(__uint_as_float(src[4]), __uint_as_float(src[5]));
-                        pk.w = pack_bf16x2(__uint_as_float(src[6]), __uint_as_float(src[7]));
-                        *reinterpret_cast<uint4 *>(buf + lane * 128 + ((j ^ (lane & 7)) << 4)) = pk;
-                    }
-                    fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) {
-                        tma_store_3d(&tmD, smem_u32(buf), colw + c * 64, row0, g, policy);
-                        bulk_commit();
-                    }
-                    ++nstore;
-                }
+                store_columns<COLS / 64, S::STG_BUFS>(tmD, r, stg, nstore, colw, row0, g, policy);
             }
         }
         if (lane == 0) bulk_wait_all();
@@ -619,6 +594,261 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     cluster_sync_all();  // no MMA, copy or remote arrive of either CTA is still in flight
     tc_fence_after();
     if (warp == 0) tmem_dealloc_pair(tmem_base, S::TMEM_COLS);
+}
+
+// ---------------------------------------------------------------------------
+// The same tiles with nothing resident, for groups of more than 256 rows and for
+// M or N that is not a multiple of 256 (both of 128): a unit is one 256 x 256
+// tile; its k-blocks (A, B and, with KSPLIT, B's residual) stream through one
+// ring.  Against the one-SM streaming kernel's tiles of 128 columns (its only
+// ones when N % 256 != 0) a CTA loads 48 KB instead of 128 KB per 128 x 256
+// outputs and 64 rows of value and residual, which is what bounds those shapes:
+// their operands stay in L2.  Tiles at the edge load zeros for the columns past
+// M or N and skip their stores.
+// Measured on GB300 (us, one-SM streaming kernel -> this one): ViT-S, 32 groups of
+// about 394 rows, dW1 37.8 -> 34.2, dW2 29.9 -> 27.3; d 640, f 1664, 36 groups of
+// about 240, 49.7 -> 34.4 and 34.5 -> 29.6; d 384, f 1536, 544 groups of about 72,
+// 168 -> 145 and 140 -> 124; d 896, f 3584, 32 groups of about 150, 79 -> 61 and 66
+// -> 50; the 17-task step's dW2, whose stores bound it (2.57 GB: 380 at DRAM's
+// rate), 424 -> 422.
+template <bool KSPLIT>
+struct PairStreamShape {
+    static constexpr uint32_t KB = 64 * 128 * 2;  // one k-block of one operand half
+    static constexpr uint32_t STAGE = (KSPLIT ? 3u : 2u) * KB;
+    static constexpr int STG_BUFS = KSPLIT ? 1 : 2;
+    static constexpr int STAGES = KSPLIT ? 4 : 5;
+    static constexpr uint32_t EPI_BYTES = 8u * STG_BUFS * 4096u;
+    static constexpr int NUM_BARS = 2 * STAGES + 5;
+    static constexpr size_t SMEM_BYTES = 1024 + (size_t)STAGES * STAGE + EPI_BYTES + NUM_BARS * 8 + 16;
+    static_assert(SMEM_BYTES + sizeof(ClcQueue) <= 232448, "over the 227 KB shared-memory limit");
+};
+
+template <bool KSPLIT>
+__global__ void __launch_bounds__(PAIR_THREADS, 1)
+wgrad_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                         const __grid_constant__ CUtensorMap tmBlo, const __grid_constant__ CUtensorMap tmD, Args args) {
+    using S = PairStreamShape<KSPLIT>;
+    constexpr int STAGES = S::STAGES;
+    constexpr uint32_t IDESC = idesc_bf16(256, 256, true, true);
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw_addr = smem_u32(smem_raw);
+    uint8_t *smem = smem_raw + ((1024u - (raw_addr & 1023u)) & 1023u);
+    const uint32_t ring = smem_u32(smem);  // STAGES x [A, B, residual of B]
+    uint8_t *epi_base = smem + STAGES * S::STAGE;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(epi_base + S::EPI_BYTES);
+    int *misc = reinterpret_cast<int *>(bars + S::NUM_BARS);  // [0] tmem base, [1] abort
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t rank = cluster_ctarank();
+    const bool leader = rank == 0;
+    auto bar = [&](int i) { return smem_u32(bars + i); };
+    auto bar_full = [&](int i) { return bar(i); };  // the leader's: both CTAs' bytes of the slot
+    auto bar_empty = [&](int i) { return bar(STAGES + i); };
+    auto bar_tfull = [&](int i) { return bar(2 * STAGES + i); };
+    auto bar_tempty = [&](int i) { return bar(2 * STAGES + 2 + i); };
+    const uint32_t bar_drain = bar(2 * STAGES + 4);
+    volatile int *abort_flag = misc + 1;
+    const uint32_t peer_abort = mapa_shared(smem_u32(misc + 1), rank ^ 1u);
+    __shared__ __align__(16) ClcQueue clc;
+    const uint32_t leader_empty = leader ? 0u : mapa_shared(smem_u32(clc.empty), 0);
+
+    if (tid == 0) {
+        clc_init(clc, leader ? 2 * PAIR_ROLES : PAIR_ROLES);
+        for (int i = 0; i < STAGES; ++i) {
+            mbar_init(bar_full(i), 2);  // the leader's A and B producers
+            mbar_init(bar_empty(i), 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bar_tfull(i), 1);
+            mbar_init(bar_tempty(i), 16);
+        }
+        mbar_init(bar_drain, 1);
+        misc[1] = 0;
+        fence_barrier_init();
+        fence_proxy_async();
+        prefetch_map(&tmA);
+        prefetch_map(&tmB);
+        if (KSPLIT) prefetch_map(&tmBlo);
+        prefetch_map(&tmD);
+    }
+    if (warp == 0) {
+        tmem_alloc_pair(smem_u32(misc), 512);
+        tmem_relinquish_pair();
+    }
+    tc_fence_before();
+    cluster_sync_all();  // barriers initialised and TMEM allocated in both CTAs
+    tc_fence_after();
+    pdl_wait();  // the predecessor's outputs are complete from here on
+    const uint32_t tmem_base = (uint32_t)misc[0];
+    const int tpg = args.tiles_m * args.tiles_n;  // tiles a group
+    struct Unit {
+        int g, m, n, L, nkb;
+    };
+    auto decode = [&](int u) {
+        Unit t;
+        t.g = u / tpg;
+        const int local = u - t.g * tpg;
+        t.m = local / args.tiles_n;
+        t.n = local - t.m * args.tiles_n;
+        t.L = __ldg(args.load + t.g);
+        t.L = t.L < 0 ? 0 : (t.L > args.C ? args.C : t.L);
+        t.nkb = (t.L + BK - 1) / BK;
+        return t;
+    };
+    auto next_unit = [&](auto warp_wide, ClcPos &pos, int &u) -> bool {
+        uint32_t x;
+        if (!clc_take<decltype(warp_wide)::value>(clc, pos, x, abort_flag, args.status, leader_empty)) return false;
+        u = (int)(x >> 1);
+        return true;
+    };
+    constexpr std::true_type WARP_WIDE{};
+    constexpr std::false_type ONE_THREAD{};
+    auto give_up = [&]() {
+        if (*abort_flag && lane == 0) st_cluster_u32(peer_abort, 1u);
+    };
+    ClcPos pos;
+    int u = (int)(blockIdx.x >> 1);
+    bool more = true;
+
+    if (warp == 0 || warp == THREADS / 32) {
+        // ------------------------------------------------------------ producers: A (warp 0), B (warp 10)
+        if (elect_one()) {
+            const bool isA = warp == 0;
+            int s = 0, issued = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            while (more && ok) {
+                const Unit t = decode(u);
+                const int k0 = t.L - t.nkb * BK;  // first row of k-block 0 (<= 0)
+                const int chunk = (isA ? t.m : t.n) * 4 + (int)rank * 2;
+                for (int kb = 0; kb < t.nkb; ++kb) {
+                    if (!wait_phase(bar_empty(s), phase ^ 1u, abort_flag, args.status)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t dst = ring + s * S::STAGE + (isA ? 0 : S::KB), fb = mapa_shared(bar_full(s), 0);
+                    if (leader) mbar_expect_tx(bar_full(s), (isA || !KSPLIT ? 2u : 4u) * S::KB);  // both CTAs' halves
+                    tma_load_4d_pair(dst, isA ? &tmA : &tmB, fb, 0, k0 + kb * BK, chunk, t.g);
+                    if (KSPLIT && !isA) tma_load_4d_pair(dst + S::KB, &tmBlo, fb, 0, k0 + kb * BK, chunk, t.g);
+                    ++issued;
+                    if (++s == STAGES) {
+                        s = 0;
+                        phase ^= 1u;
+                    }
+                }
+                more = next_unit(ONE_THREAD, pos, u);
+            }
+            if (*abort_flag && leader) {  // copies in flight (both CTAs') land before the pair exits
+                const unsigned long long t0 = global_ns();
+                for (int i = 0; i < STAGES && i < issued; ++i)
+                    while (!mbar_try_wait(bar_full(i), (uint32_t)(((issued - 1 - i) / STAGES) & 1)) &&
+                           global_ns() - t0 < 200000000ull) {
+                    }
+            }
+        }
+        __syncwarp();
+        give_up();
+    } else if (warp == THREADS / 32 + 1) {
+        // ------------------------------------------------------------ scheduler
+        if (elect_one()) clc_scheduler<true>(clc, leader, abort_flag, args.status);
+        __syncwarp();
+        give_up();
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA issuer (the leader's; the peer's only takes units)
+        if (elect_one()) {
+            int s = 0, it = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            while (more && ok) {
+                const Unit t = decode(u);
+                if (leader && t.nkb > 0) {
+                    const int skip = (t.nkb * BK - t.L) >> 4;  // all-zero 16-row steps of k-block 0
+                    const int acc = it & 1;
+                    const uint32_t dtmem = tmem_base + (uint32_t)(acc * 256);
+                    if (!wait_phase(bar_tempty(acc), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag, args.status)) break;
+                    tc_fence_after();
+                    for (int kb = 0; kb < t.nkb; ++kb) {
+                        if (!wait_phase(bar_full(s), phase, abort_flag, args.status)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const int kk0 = kb == 0 ? skip : 0;
+                        const uint64_t da = operand_desc(ring + s * S::STAGE, 0, true);
+#pragma unroll
+                        for (int part = 0; part < (KSPLIT ? 2 : 1); ++part) {
+                            const uint64_t db = operand_desc(ring + s * S::STAGE + (1 + part) * S::KB, 0, true);
+#pragma unroll
+                            for (int kk = 0; kk < BK / 16; ++kk)
+                                if (kk >= kk0)
+                                    mma_pair_bf16(dtmem, desc_step(da, kk, true), desc_step(db, kk, true), IDESC,
+                                                  (kb | part | (kk - kk0)) != 0 ? 1u : 0u);
+                        }
+                        mma_pair_commit_both(bar_empty(s));
+                        if (++s == STAGES) {
+                            s = 0;
+                            phase ^= 1u;
+                        }
+                    }
+                    if (!ok) break;
+                    mma_pair_commit_both(bar_tfull(acc));
+                    ++it;
+                }
+                more = next_unit(ONE_THREAD, pos, u);
+            }
+            if (leader) {  // all MMAs of the pair complete before TMEM is freed
+                mma_pair_commit_local(bar_drain);
+                const unsigned long long t0 = global_ns();
+                while (!mbar_try_wait(bar_drain, 0) && global_ns() - t0 < 1000000000ull) {
+                }
+            }
+        }
+        __syncwarp();
+        give_up();
+    } else {
+        // ------------------------------------------------------------ epilogue
+        const int ew = warp - 2, q = warp & 3, half = ew >> 2;
+        uint8_t *stg = epi_base + ew * S::STG_BUFS * 4096;
+        const uint64_t policy = evict_first_policy();
+        int nstore = 0, it = 0;
+        bool zeroed = false;  // the first staging tile holds zeros that copies in flight read
+        for (; more; more = next_unit(WARP_WIDE, pos, u)) {
+            const Unit t = decode(u);
+            if (t.L == 0) {
+                zero_staging(stg, zeroed);
+                if (lane == 0)
+                    store_zeros(reinterpret_cast<uint8_t *>(args.D + (long long)t.g * args.sD), args.sD * 2,
+                                t.m * args.tiles_n + t.n, tpg, (int)rank * 8 + ew, 16, smem_u32(stg), policy);
+                continue;
+            }
+            if (zeroed) {
+                if (lane == 0) bulk_wait_read0();
+                zeroed = false;
+            }
+            const int acc = it & 1;
+            if (!wait_phase(bar_tfull(acc), (uint32_t)((it >> 1) & 1), abort_flag, args.status)) break;
+            tc_fence_after();
+            uint32_t r[4][32];
+            const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * 256 + half * 128);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) tmem_ld32(trow + i * 32, r[i]);
+            tmem_ld_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(mapa_shared(bar_tempty(acc), 0));
+            ++it;
+            const int row0 = t.m * 256 + (int)rank * 128 + q * 32, col = t.n * 256 + half * 128;
+            if (row0 < args.M_fixed && col < args.N)  // M and N are multiples of 128: all of it or none
+                store_columns<2, S::STG_BUFS>(tmD, r, stg, nstore, col, row0, t.g, policy);
+        }
+        if (lane == 0) bulk_wait_all();
+        __syncwarp();
+        give_up();
+    }
+
+    tc_fence_before();
+    cluster_sync_all();  // no MMA, copy or remote arrive of either CTA is still in flight
+    tc_fence_after();
+    if (warp == 0) tmem_dealloc_pair(tmem_base, 512);
 }
 
 // ---------------------------------------------------------------------------
@@ -1059,6 +1289,33 @@ int launch_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap 
 }
 
 
+template <bool KSPLIT>
+int launch_pair_stream(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mblo, const CUtensorMap &md,
+                       const Args &a, long long units, cudaStream_t s, const char *name) {
+    using S = PairStreamShape<KSPLIT>;
+    auto kern = wgrad_pair_stream_kernel<KSPLIT>;
+    static std::atomic<int> smem_limit[64];
+    if (const int st = raise_smem_limit((const void *)kern, smem_limit, (int)S::SMEM_BYTES)) return st;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * units));
+    cfg.blockDim = dim3(PAIR_THREADS);
+    cfg.dynamicSmemBytes = S::SMEM_BYTES;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl_enabled() ? 2 : 1;
+    trace_before(s, name);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, ma, mb, mblo, md, a);
+    trace_after(s);
+    return e == cudaSuccess ? VMOE_OK : VMOE_ERR_CUDA;
+}
+
 template <int BN, bool B_MN, int EPI>
 int launch_row_pair(const CUtensorMap &ma, const CUtensorMap &mb, const TailMaps &mat, const Args &a,
                     long long max_tiles, cudaStream_t s, const char *name) {
@@ -1174,17 +1431,16 @@ int row_gemm(const Dims &p, const __nv_bfloat16 *act, int K, const __nv_bfloat16
 // over each group's load[g] rows; both operands MN-major.
 // ksplit: act2 is [G, 2C, N] -- a bf16 part in rows [0, C) and its residual in
 // rows [C, 2C) -- and D = act1^T (hi + lo), summed over both halves.
-// Kernel choice (measured on GB300, us per launch):
-//   M, N multiples of 256 and C <= 256: the SM-pair kernel above (resident B,
-//     double buffered where two B tiles fit), except dW2 with 32 < C <= 128,
-//     where the streaming kernel is faster (17-task ViT-B step, C 124, both with
-//     a fixed stride: 474 against 503);
-//   otherwise the streaming grouped GEMM (both halves in its K loop).  A one-SM
-//     kernel with a resident B tile used to take dW1 of M % 256 != 0 at 32 < C
-//     <= 128; since the producers are two threads it is slower (d 384, f 1536,
-//     C 124: 180 against 169 with 17 tasks of 32 experts, 33 against 26 with 4
-//     of 16).
-// VMOE_PAIR=0 in the environment turns the pair kernel off.
+// Kernel choice:
+//   M, N multiples of 256 and C <= 256: the SM-pair kernel with a resident B tile
+//     (double buffered where two fit), except dW2 with 32 < C <= 128, whose short
+//     tiles gain nothing from it (17-task ViT-B step, C 124, both with a fixed
+//     stride: 503 us against 474 streamed);
+//   otherwise M, N >= 256: the SM-pair streaming kernel;
+//   otherwise (M or N 128; the sliced backward's compact B at the shapes of the
+//     second line): the one-SM streaming grouped GEMM.
+// All sum a group's rows in the same order, k-block by k-block, value then residual.
+// VMOE_PAIR=0 in the environment turns the pair kernels off.
 inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __nv_bfloat16 *act2,
                       int N, const int32_t *load, __nv_bfloat16 *D, cudaStream_t s,
                       const char *name, bool ksplit = false, const Slice &sl = Slice(),
@@ -1209,7 +1465,9 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
         a.compact = sl.compact;
     }
     const bool pair_pays = ksplit || C <= 32 || C > 2 * BK;
-    if (pair_enabled() && pair_pays && M % 256 == 0 && N % 256 == 0 && C <= 4 * BK) {
+    const bool resident = pair_pays && M % 256 == 0 && N % 256 == 0 && C <= 4 * BK;
+    const bool stream = !resident && sl.n == 0 && M >= 256 && N >= 256;
+    if (pair_enabled() && (resident || stream)) {
         // Each CTA of a pair loads 128 columns (two chunks) of A and of B.  The
         // group-indexed maps have exactly C rows per group, and with ksplit the
         // residual gets a map of its own (base C rows in, group stride 2C rows),
@@ -1223,8 +1481,13 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
                                                 2 * (uint64_t)C * N))) {
             return VMOE_ERR_CUDA;
         }
-        a.tiles_m = M / 256;
-        a.tiles_n = N / 256;
+        a.tiles_m = (M + 255) / 256;
+        a.tiles_n = (N + 255) / 256;
+        if (stream) {
+            const long long tiles = (long long)a.G * a.tiles_m * a.tiles_n;
+            return ksplit ? launch_pair_stream<true>(ma, mb, mblo, md, a, tiles, s, name)
+                          : launch_pair_stream<false>(ma, mb, mblo, md, a, tiles, s, name);
+        }
         const long long units = (long long)a.G * a.tiles_n;
         if (C <= 2 * BK)
             return ksplit ? launch_pair<true, 2>(ma, mb, mblo, md, a, units, s, name, sched)
@@ -1244,15 +1507,8 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
     a.tiles_m = M / BM;
     long long max_tiles = (long long)a.G * a.tiles_m * a.tiles_n;
     const TailMaps unused{};  // the streaming kernel loads full k-blocks
-    auto go = [&](auto kern_launch) { return kern_launch(ma, mb, md, mblo, unused, a, max_tiles, s, name); };
-    // Dynamic tiles where the gradient is larger than L2 twice over, so that its
-    // stores run at DRAM's rate (17-task step, dW2 474 -> 424 us); a layer whose
-    // gradient stays in L2 has nothing to gain (ViT-S 37.2 us with a fixed stride,
-    // 39.5 with), nor have 128-wide tiles, bound by their operands (d 384: 139 both).
-    constexpr long long CLC_MIN_BYTES = 256LL << 20;
-    if (wide && max_tiles * BM * BN * 2 >= CLC_MIN_BYTES) return go(launch<256, MODE_WGRAD, true, true, EPI_STORE, true>);
-    return wide ? go(launch<256, MODE_WGRAD, true, true, EPI_STORE>)
-                : go(launch<128, MODE_WGRAD, true, true, EPI_STORE>);
+    return wide ? launch<256, MODE_WGRAD, true, true, EPI_STORE>(ma, mb, md, mblo, unused, a, max_tiles, s, name)
+                : launch<128, MODE_WGRAD, true, true, EPI_STORE>(ma, mb, md, mblo, unused, a, max_tiles, s, name);
 }
 
 }  // namespace tc
