@@ -109,6 +109,7 @@ struct PlanChunk {
 
 __global__ void __launch_bounds__(PLAN_CHUNK) plan_write_kernel(const __grid_constant__ PlanChunk c,
                                                                int32_t *__restrict__ plan) {
+    pdl_wait();  // so that what waits for this kernel has waited for the one before
     const int i = threadIdx.x;
     if (i < c.n) {
         plan[c.pos + i] = c.g[i];
@@ -200,8 +201,7 @@ int launch_expert_bwd_bf16_sliced(const Dims &p, const __nv_bfloat16 *xe, const 
                 row += w[slice[k0 + i]] * BW_UNIT;
             }
             trace_before(s, "bwd_plan");
-            plan_write_kernel<<<1, PLAN_CHUNK, 0, s>>>(c, dplan);
-            st = launch_result();
+            st = launch_kernel(plan_write_kernel, dim3(1), dim3(PLAN_CHUNK), 0, s, c, dplan);
             trace_after(s);
         }
         if (st != VMOE_OK) break;
