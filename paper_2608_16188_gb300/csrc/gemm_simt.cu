@@ -56,7 +56,8 @@ struct SimtTile {
 // a vector is wholly inside or wholly outside (zeros).
 template <int W, int NT, bool CONTIG_K>
 struct SimtChunk {
-    static constexpr int V = W * ST_BK / 4 / NT;
+    static constexpr int N4 = W * ST_BK / 4;  // vectors of a chunk
+    static constexpr int V = (N4 + NT - 1) / NT;
     float4 v[V];
     __device__ __forceinline__ void load(const float *p, int ld, int w0, int wn, int k0, int kn) {
 #pragma unroll
@@ -65,7 +66,7 @@ struct SimtChunk {
             const int w = w0 + (CONTIG_K ? u / (ST_BK / 4) : u % (W / 4) * 4);
             const int k = k0 + (CONTIG_K ? u % (ST_BK / 4) * 4 : u / (W / 4));
             v[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (w < wn && k < kn)
+            if (u < N4 && w < wn && k < kn)
                 v[i] = __ldg(reinterpret_cast<const float4 *>(
                     p + (CONTIG_K ? (long long)w * ld + k : (long long)k * ld + w)));
         }
@@ -74,6 +75,7 @@ struct SimtChunk {
 #pragma unroll
         for (int i = 0; i < V; ++i) {
             const int u = threadIdx.x + i * NT;
+            if (N4 % NT != 0 && u >= N4) continue;
             if (CONTIG_K) {
                 const int w = u / (ST_BK / 4), k = u % (ST_BK / 4) * 4;
                 s[k][w] = v[i].x;
@@ -256,16 +258,23 @@ int run_tile(SimtArgs a, int G, int mmax, int split, cudaStream_t s, const char 
 // the CUDA cores' 80); the 8-expert layer of d 64, f 256: FC2 37 -> 11, dX 38 ->
 // 10, the others 12-16 -> 8-11.  Row mode stays at 47% of the FMA pipe: half of
 // its second 64-row tile is padding, and shared-memory reads fill 75% of the L1.
+// Groups of at most 32 rows take tiles of 16 or 32 rows instead of computing 64 (6
+// tasks of 30 experts of at most 13 rows, d 336, f 1168: the step 1807 -> 607 us).
 // kmax: the longest reduction (row mode: K; weight gradients: C rows).
 template <int EPI, bool A_T, bool B_T>
 int run(const SimtArgs &a, int G, int mmax, cudaStream_t s, const char *name) {
     const int kmax = a.row_mode ? a.K : a.C;
     const long long sms = num_sms();
     const long long big = (long long)((a.N + 127) / 128) * ((mmax + 127) / 128) * G;
-    if (big >= 2 * sms) return run_tile<128, 128, 16, 8, EPI, A_T, B_T>(a, G, mmax, 1, s, name);
-    const long long small = (long long)((a.N + 63) / 64) * ((mmax + 63) / 64) * G;
+    if (big >= 2 * sms && !(a.row_mode && mmax <= 32)) return run_tile<128, 128, 16, 8, EPI, A_T, B_T>(a, G, mmax, 1, s, name);
+    const bool few = a.row_mode && mmax <= 32;  // one tile of 16 or 32 rows a group
+    const long long small = few ? (long long)((a.N + 127) / 128) * G
+                                : (long long)((a.N + 63) / 64) * ((mmax + 63) / 64) * G;
     int split = 1;
     while (split < 8 && small * split < 3 * sms && kmax >= 2 * split * 3 * ST_BK) split *= 2;
+    if (few && !A_T)
+        return mmax <= 16 ? run_tile<16, 128, 4, 4, EPI, false, B_T>(a, G, mmax, split, s, name)
+                          : run_tile<32, 128, 8, 4, EPI, false, B_T>(a, G, mmax, split, s, name);
     return run_tile<64, 64, 8, 4, EPI, A_T, B_T>(a, G, mmax, split, s, name);
 }
 

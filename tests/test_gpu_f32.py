@@ -18,6 +18,9 @@ CASES = [
     Config("f32_split", 91, T=1, N=66, d=128, f=516, E=2, k=2, cf=1.0, dtype="f32", flags=4),
     # 70 experts (two router passes of 64), d = 136 (a chunk of 8), empty groups
     Config("f32_experts70", 92, T=2, N=45, d=136, f=64, E=70, k=3, cf=1.0, dtype="f32", bias="zipf", flags=2),
+    # 13 and 27 rows a group: tiles of 16 and 32 rows, d and f off the 128-wide columns, with and without a split
+    Config("f32_rows13", 89, T=3, N=124, d=136, f=428, E=30, k=2, cf=1.5, dtype="f32", bias="drift"),
+    Config("f32_rows27", 88, T=1, N=50, d=200, f=260, E=4, k=1, cf=2.1, dtype="f32"),
     Config("f32_one_token", 93, T=1, N=1, d=8, f=4, E=2, k=1, cf=1.0, dtype="f32"),
 ]
 
