@@ -550,12 +550,21 @@ struct Tile {
     int khalf;  // weight-gradient mode: k-blocks per half (kblocks = 2 * khalf with ksplit)
     int gr;     // the real group of entry g
     int crow;   // entry g's first row in the compact buffer
+    int col0, bn;  // row mode: first column and columns (BN, or BN >> cut from tile `wide` on)
 };
 
-template <int MODE>
-__device__ __forceinline__ Tile decode_tile(const Args &a, const int *prefix, int u) {
+// Row mode with CUT: tiles from index `wide` on are halves (cut = 1) of BN / 2 columns.
+template <int MODE, int BN, bool CUT>
+__device__ __forceinline__ Tile decode_tile(const Args &a, const int *prefix, int u, int wide, int cut) {
     Tile t;
     if (MODE == MODE_ROW) {
+        int piece = 0;
+        t.bn = BN;
+        if (CUT && u >= wide) {
+            piece = (u - wide) & ((1 << cut) - 1);
+            u = wide + ((u - wide) >> cut);
+            t.bn = BN >> cut;
+        }
         int lo = 0, hi = a.G;  // prefix[lo] <= u < prefix[hi]
         while (hi - lo > 1) {
             int mid = (lo + hi) >> 1;
@@ -567,6 +576,7 @@ __device__ __forceinline__ Tile decode_tile(const Args &a, const int *prefix, in
         int local = u - prefix[lo];
         t.m_blk = local / a.tiles_n;
         t.n_blk = local - t.m_blk * a.tiles_n;
+        t.col0 = t.n_blk * BN + piece * t.bn;
         t.kblocks = a.K_fixed / BK;
         t.khalf = t.kblocks;
         t.kvalid = a.K_fixed;
@@ -637,6 +647,9 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     constexpr int STAGES = S::STAGES;
     constexpr int NT = S::NT;
     constexpr uint32_t IDESC = idesc_bf16(BM, BN, A_MN, B_MN);
+    // the last wave in pieces; not dA + GELU', whose prefetch of H needs fixed bounds
+    // (with run-time ones it spills: 269 -> 344 us at the 6-task ViT-B step)
+    constexpr bool CUT = MODE == MODE_ROW && EPI != EPI_DGELU;
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -730,6 +743,20 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     __syncthreads();
     tc_fence_after();
     total = (MODE == MODE_ROW) ? misc[2] : args.G * args.tiles_m * args.tiles_n;
+    // Row mode: a last wave that fills at most half of the SMs is cut into tiles of
+    // half the columns, so that it ends sooner; no element's sums change.  One
+    // image through a ViT-S layer (48 and 24 tiles) 32.8 -> 30.3 us, attention at C
+    // 247 1134 -> 1129.  Quarters, which would also shorten fuller last waves, cost
+    // more than they gave (6-task ViT-B, FC2 201 -> 222 us).
+    int wide = total, cut = 0;
+    if (CUT) {
+        const int rem = total % (int)gridDim.x;
+        if (rem > 0 && 2 * rem <= (int)gridDim.x) {
+            cut = 1;
+            wide = total - rem;
+            total += rem;
+        }
+    }
     const uint32_t tmem_base = (uint32_t)misc[0];
 
     if (warp == 0 || warp == Roles<MODE, EPI>::EW + 2) {
@@ -743,7 +770,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             int issued = 0;  // copies so far: slot s has had those of index s, s + STAGES, ...
             bool ok = true;
             const bool cmpa = (args.compact & CMP_A) != 0, cmpb = (args.compact & CMP_B) != 0;
-            Tile t = decode_tile<MODE>(args, prefix, blockIdx.x < total ? blockIdx.x : 0);
+            Tile t = decode_tile<MODE, BN, CUT>(args, prefix, blockIdx.x < total ? blockIdx.x : 0, wide, cut);
             for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
                 Tile tn = t;  // the next tile, looked up behind this one's first copy
                 const bool last = u + (int)gridDim.x >= total;
@@ -754,7 +781,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 const int rem_rows = t.rows_valid - t.m_blk * BM;
                 const int rn = MODE != MODE_ROW || rem_rows >= BM ? BM : ((rem_rows + 15) & ~15);
                 const int r0 = (cmpa ? t.crow : 0) + t.m_blk * BM, gz = cmpa ? 0 : t.gr;
-                const uint32_t bytes = isA ? (uint32_t)rn * (BK * 2) : S::B_BYTES;
+                const int bn = CUT ? t.bn : BN;
+                const uint32_t bytes = isA ? (uint32_t)rn * (BK * 2) : (uint32_t)bn * (BK * 2);
                 // Weight gradients: the first K row of k-block 0 (<= 0, see below)
                 const int k0 = t.kvalid - t.khalf * BK;
                 for (int kb = 0; kb < t.kblocks; ++kb) {
@@ -783,6 +811,11 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                                 if (rn & 16)
                                     tma_load_3d(sa + off * (BK * 2), &tmAt.a[2], fb, kb * BK, r0 + off, gz);
                             }
+                        } else if (CUT && bn != BN) {  // tmD: B's map with boxes of 64 columns
+                            for (int c = 0; c < bn; c += 64) {
+                                if (B_MN) tma_load_4d(sb + c * (BK * 2), &tmD, fb, 0, kb * BK, (t.col0 + c) / 64, t.gr);
+                                else tma_load_3d(sb + c * (BK * 2), &tmD, fb, kb * BK, t.col0 + c, t.gr);
+                            }
                         } else if (B_MN) {  // one 4-D box: BN/64 column chunks of 64 rows
                             tma_load_4d(sb, &tmB, fb, 0, kb * BK, t.n_blk * (BN / 64), t.gr);
                         } else {
@@ -804,14 +837,14 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         else
                             tma_load_4d(sb, hi ? &tmD2 : &tmB, fb, 0, ka, t.n_blk * (BN / 64), t.gr);
                     }
-                    if (kb == 0 && !last) tn = decode_tile<MODE>(args, prefix, u + gridDim.x);
+                    if (kb == 0 && !last) tn = decode_tile<MODE, BN, CUT>(args, prefix, u + gridDim.x, wide, cut);
                     ++issued;
                     if (++stage == STAGES) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
-                if (t.kblocks == 0 && !last) tn = decode_tile<MODE>(args, prefix, u + gridDim.x);
+                if (t.kblocks == 0 && !last) tn = decode_tile<MODE, BN, CUT>(args, prefix, u + gridDim.x, wide, cut);
                 t = tn;
             }
             if (*abort_flag) {  // let copies in flight land before the CTA exits
@@ -831,15 +864,16 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         int it = 0;
         bool ok = true;
         const bool cmpb = MODE == MODE_WGRAD && (args.compact & CMP_B) != 0;
+        const uint32_t idesc_cut = idesc_bf16(BM, BN >> cut, A_MN, B_MN);
         const bool one = elect_one();
         // Waits for slot `stage` and issues its MMAs from 16-row step k0 on.
-        auto k_block = [&](uint32_t dtmem, int k0, bool accumulate) {
+        auto k_block = [&](uint32_t dtmem, int k0, bool accumulate, uint32_t idesc) {
             const uint32_t sa = tiles_addr + stage * S::STAGE_BYTES;
             const uint64_t da = operand_desc(sa, 0, A_MN), db = operand_desc(sa + S::A_BYTES, 0, B_MN);
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
                 if (MODE == MODE_ROW || kk >= k0)
-                    mma_bf16(dtmem, desc_step(da, kk, A_MN), desc_step(db, kk, B_MN), IDESC,
+                    mma_bf16(dtmem, desc_step(da, kk, A_MN), desc_step(db, kk, B_MN), idesc,
                              accumulate || kk > k0 ? 1u : 0u);
             mma_commit(bar_empty(stage));
         };
@@ -853,7 +887,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             for (int u = blockIdx.x; one && u < total && ok; u += gridDim.x, ++it) {
                 int kblocks = args.K_fixed / BK, skip = 0;
                 if (MODE == MODE_WGRAD) {
-                    const Tile t = decode_tile<MODE>(args, prefix, u);
+                    const Tile t = decode_tile<MODE, BN, CUT>(args, prefix, u, wide, cut);
                     kblocks = t.kblocks;
                     skip = (t.khalf * BK - t.kvalid) >> 4;  // all-zero 16-row steps of k-block 0
                 }
@@ -866,7 +900,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         break;
                     }
                     tc_fence_after();
-                    k_block(tmem_base + (uint32_t)(acc * BN), (kb >> args.ksplit) == 0 ? skip : 0, kb > 0);
+                    k_block(tmem_base + (uint32_t)(acc * BN), (kb >> args.ksplit) == 0 ? skip : 0, kb > 0,
+                            !CUT || u < wide ? IDESC : idesc_cut);
                     next_stage();
                 }
                 if (!ok) break;
@@ -875,7 +910,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
         } else {  // compact B: the warp zeroes the rows of k-block 0 (both parts) that belong to a neighbour
             for (int u = blockIdx.x; u < total && ok; u += gridDim.x, ++it) {
-                const Tile t = decode_tile<MODE>(args, prefix, u);
+                const Tile t = decode_tile<MODE, BN, CUT>(args, prefix, u, wide, cut);
                 const int z = t.khalf * BK - t.kvalid;
                 const int acc = it & 1;
                 if (!wait_phase(bar_tempty(acc), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag, args.status)) break;
@@ -897,7 +932,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         fence_proxy_async();
                     }
                     __syncwarp();
-                    if (one) k_block(tmem_base + (uint32_t)(acc * BN), first ? z >> 4 : 0, kb > 0);
+                    if (one) k_block(tmem_base + (uint32_t)(acc * BN), first ? z >> 4 : 0, kb > 0, IDESC);
                     __syncwarp();
                     next_stage();
                 }
@@ -933,7 +968,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         int it = 0;
         bool zeroed = false;  // the first staging tile holds zeros that copies in flight read
         for (int u = blockIdx.x; u < total; u += gridDim.x, ++it) {
-            const Tile t = decode_tile<MODE>(args, prefix, u);
+            const Tile t = decode_tile<MODE, BN, CUT>(args, prefix, u, wide, cut);
             const int acc = it & 1;
             const uint32_t aph = (uint32_t)((it >> 1) & 1);
             if (!wait_phase(bar_tfull(acc), aph, abort_flag, args.status)) break;
@@ -978,7 +1013,6 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         constexpr int EW = Roles<MODE, EPI>::EW;
         constexpr int WPQ = EW / 4;                 // warps per lane quarter
         constexpr int CH = ROW_CH;                  // columns per chunk
-        constexpr int NCH = BN / CH;                // chunks per tile row
         constexpr int PITCH = Roles<MODE, EPI>::PITCH;   // staging row pitch (bytes)
         constexpr int PIECES = CH * 2 / 16;         // 16-byte pieces of a staged row
         constexpr int RPI = 32 / PIECES;            // rows per store instruction
@@ -1025,11 +1059,11 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
         };
         int it = 0;
-        Tile t = decode_tile<MODE>(args, prefix, blockIdx.x < total ? blockIdx.x : 0);
+        Tile t = decode_tile<MODE, BN, CUT>(args, prefix, blockIdx.x < total ? blockIdx.x : 0, wide, cut);
         if (EPI == EPI_DGELU && blockIdx.x < total) load_h(t, jw, hcur);
         for (int u = blockIdx.x; u < total; u += gridDim.x, ++it) {
             const bool have_next = u + (int)gridDim.x < total;
-            const Tile tn = decode_tile<MODE>(args, prefix, have_next ? u + gridDim.x : u);
+            const Tile tn = decode_tile<MODE, BN, CUT>(args, prefix, have_next ? u + gridDim.x : u, wide, cut);
             const int acc = it & 1;
             const uint32_t aph = (uint32_t)((it >> 1) & 1);
             if (!wait_phase(bar_tfull(acc), aph, abort_flag, args.status)) break;
@@ -1041,13 +1075,14 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             // residual) after its load rows; else the group's slab
             const bool cmpd = (args.compact & CMP_D) != 0;
             const long long gofs = (cmpd ? (long long)t.crow * args.ldd : (long long)t.gr * args.sD) +
-                                   (long long)row0 * args.ldd + t.n_blk * BN;
+                                   (long long)row0 * args.ldd + (CUT ? t.col0 : t.n_blk * BN);
             const long long gofs2 = cmpd ? gofs + (long long)t.rows_valid * args.ldd : gofs;
             const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
+            const int nch = (CUT ? t.bn : BN) / CH;  // chunks of this tile's rows
 #pragma unroll 1
-            for (int c = jw; c < NCH; c += WPQ) {
+            for (int c = jw; c < nch; c += WPQ) {
                 if (EPI == EPI_DGELU) {
-                    if (c + WPQ < NCH) load_h(t, c + WPQ, hnxt);
+                    if (c + WPQ < nch) load_h(t, c + WPQ, hnxt);
                     else if (have_next) load_h(tn, jw, hnxt);
                 }
                 if (nvalid > 0) {
@@ -1114,7 +1149,9 @@ int launch(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &md,
     static std::atomic<int> smem_limit[64];
     if (const int st = raise_smem_limit((const void *)kern, smem_limit, (int)S::SMEM_BYTES)) return st;
     if (max_tiles <= 0) return VMOE_OK;
-    const long long grid = max_tiles < num_sms() ? max_tiles : num_sms();
+    // row mode may cut every tile in two
+    const long long most = MODE == MODE_ROW && EPI != EPI_DGELU ? 2 * max_tiles : max_tiles;
+    const long long grid = most < num_sms() ? most : num_sms();
     trace_before(s, name);
     const int st = launch_kernel(kern, dim3((unsigned)grid), dim3(S::NT), S::SMEM_BYTES, s, ma, mb,
                                  md, md2, mat, a);

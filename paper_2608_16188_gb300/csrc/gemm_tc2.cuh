@@ -1422,7 +1422,11 @@ int row_gemm(const Dims &p, const __nv_bfloat16 *act, int K, const __nv_bfloat16
     if (pair)
         return wide ? launch_row_pair<256, B_MN, EPI>(ma, mb, mat, a, max_tiles, s, name)
                     : launch_row_pair<128, B_MN, EPI>(ma, mb, mat, a, max_tiles, s, name);
-    const CUtensorMap md = {}, md2 = {};  // row mode stores with st.global: no output maps
+    // row mode stores with st.global: no output maps, md carries B's map with boxes of 64 columns
+    CUtensorMap md;
+    const CUtensorMap md2 = {};
+    okb = B_MN ? make_map_chunked(&md, w, N, K, G, 64, 1) : make_map(&md, w, K, N, G, 64);
+    if (!okb) return VMOE_ERR_CUDA;
     return wide ? launch<256, MODE_ROW, false, B_MN, EPI>(ma, mb, md, md2, mat, a, max_tiles, s, name)
                 : launch<128, MODE_ROW, false, B_MN, EPI>(ma, mb, md, md2, mat, a, max_tiles, s, name);
 }
