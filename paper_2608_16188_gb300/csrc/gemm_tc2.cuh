@@ -283,7 +283,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     tc_fence_before();
     cluster_sync_all();  // barriers initialised and TMEM allocated in both CTAs
     tc_fence_after();
-    pdl_wait();  // the predecessor's outputs are complete from here on
+    wait_for_predecessor(args, false);  // the predecessor's outputs are complete from here on
     const uint32_t tmem_base = (uint32_t)misc[0];
     const int cid = blockIdx.x >> 1;
     const int total = args.G * args.tiles_n;
@@ -594,6 +594,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     cluster_sync_all();  // no MMA, copy or remote arrive of either CTA is still in flight
     tc_fence_after();
     if (warp == 0) tmem_dealloc_pair(tmem_base, S::TMEM_COLS);
+    wait_for_predecessor(args, true);
 }
 
 // ---------------------------------------------------------------------------
@@ -677,7 +678,7 @@ wgrad_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     tc_fence_before();
     cluster_sync_all();  // barriers initialised and TMEM allocated in both CTAs
     tc_fence_after();
-    pdl_wait();  // the predecessor's outputs are complete from here on
+    wait_for_predecessor(args, false);  // the predecessor's outputs are complete from here on
     const uint32_t tmem_base = (uint32_t)misc[0];
     const int tpg = args.tiles_m * args.tiles_n;  // tiles a group
     struct Unit {
@@ -849,6 +850,7 @@ wgrad_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     cluster_sync_all();  // no MMA, copy or remote arrive of either CTA is still in flight
     tc_fence_after();
     if (warp == 0) tmem_dealloc_pair(tmem_base, 512);
+    wait_for_predecessor(args, true);
 }
 
 // ---------------------------------------------------------------------------
@@ -1433,6 +1435,8 @@ int row_gemm(const Dims &p, const __nv_bfloat16 *act, int K, const __nv_bfloat16
 
 // Weight-gradient GEMM: D[g][M][N] = act1[g][C][M]^T * act2[g][C][N], summed
 // over each group's load[g] rows; both operands MN-major.
+// late: nothing that this reads is written by the launch just before it, of the
+// same entry point (wait_for_predecessor).
 // ksplit: act2 is [G, 2C, N] -- a bf16 part in rows [0, C) and its residual in
 // rows [C, 2C) -- and D = act1^T (hi + lo), summed over both halves.
 // Kernel choice:
@@ -1447,7 +1451,7 @@ int row_gemm(const Dims &p, const __nv_bfloat16 *act, int K, const __nv_bfloat16
 // VMOE_PAIR=0 in the environment turns the pair kernels off.
 inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __nv_bfloat16 *act2,
                       int N, const int32_t *load, __nv_bfloat16 *D, cudaStream_t s,
-                      const char *name, bool ksplit = false, const Slice &sl = Slice(),
+                      const char *name, bool late, bool ksplit = false, const Slice &sl = Slice(),
                       const PairSchedule *sched = nullptr) {
     const int G = p.G(), C = p.C;
     const bool wide = N % 256 == 0;
@@ -1462,6 +1466,7 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
     a.sD = (long long)M * N;
     a.ldd = N;
     a.ksplit = ksplit ? 1 : 0;
+    a.late_wait = late ? 1 : 0;
     if (sl.n > 0) {
         a.G = sl.n;
         a.glist = sl.glist;

@@ -72,8 +72,8 @@ int launch_expert_bwd_bf16(const Dims &p, const __nv_bfloat16 *xe, const __nv_bf
     if ((st = row_gemm<EPI_STORE, false>(p, dh_hi, p.f, w1, p.d, load, dxe, nullptr, nullptr, s,
                                          "tc_dx", 0, 0, 2 * C * f)) != VMOE_OK)
         return st;
-    if ((st = wgrad_gemm(p, xe, p.d, dh, p.f, load, dw1, s, "tc_dw1", true)) != VMOE_OK) return st;
-    return wgrad_gemm(p, act, p.f, dye, p.d, load, dw2, s, "tc_dw2");
+    if ((st = wgrad_gemm(p, xe, p.d, dh, p.f, load, dw1, s, "tc_dw1", true, true)) != VMOE_OK) return st;
+    return wgrad_gemm(p, act, p.f, dye, p.d, load, dw2, s, "tc_dw2", true);
 }
 
 // The backward under a dH budget (the expert groups' temporary memory, Section
@@ -151,7 +151,7 @@ int launch_expert_bwd_bf16_sliced(const Dims &p, const __nv_bfloat16 *xe, const 
     int st = planner.init(G, w.data(), r.data(), cap_units, 0.0, 0.0);
     if (st != VMOE_OK) return st;
     // dW2 first: it needs no dH, and it runs while the first slice is planned
-    if ((st = wgrad_gemm(p, act, p.f, dye, p.d, load, dw2, s, "tc_dw2")) != VMOE_OK) return st;
+    if ((st = wgrad_gemm(p, act, p.f, dye, p.d, load, dw2, s, "tc_dw2", false)) != VMOE_OK) return st;
     int32_t *dplan = reinterpret_cast<int32_t *>(workspace);
     __nv_bfloat16 *dh = reinterpret_cast<__nv_bfloat16 *>(static_cast<uint8_t *>(workspace) + plan_bytes);
     // dW1 of a slice on SM pairs, optionally (VMOE_SHARES=1) with each group's
@@ -221,7 +221,7 @@ int launch_expert_bwd_bf16_sliced(const Dims &p, const __nv_bfloat16 *xe, const 
         sl.compact = CMP_B;
         PairSchedule sc;
         slice_schedule(slice, sc);
-        st = wgrad_gemm(p, xe, p.d, dh, p.f, load, dw1, s, "tc_dw1", true, sl, &sc);
+        st = wgrad_gemm(p, xe, p.d, dh, p.f, load, dw1, s, "tc_dw1", true, true, sl, &sc);
         pos += n;
         ++ns;
     }
@@ -250,13 +250,13 @@ int launch_attn_expert_bwd(const Dims &p, int H, const __nv_bfloat16 *xe, const 
     float *dsum = reinterpret_cast<float *>(dqkv + rows * 3 * hd);
     int st = row_gemm<EPI_STORE, false>(p, dye, p.d, wo, hd, load, dout, nullptr, nullptr, s, "attn_dout");
     if (st != VMOE_OK) return st;
-    if ((st = wgrad_gemm(p, o, hd, dye, p.d, load, dwo, s, "attn_dwo")) != VMOE_OK) return st;
+    if ((st = wgrad_gemm(p, o, hd, dye, p.d, load, dwo, s, "attn_dwo", true)) != VMOE_OK) return st;
     if ((st = launch_attn_core_bwd(p.G(), p.C, H, load, qkv, o, lse, dout, dsum, dqkv, s)) != VMOE_OK)
         return st;
     if ((st = row_gemm<EPI_STORE, false>(p, dqkv, 3 * hd, wqkv, p.d, load, dxe, nullptr, nullptr, s,
                                          "attn_dxe")) != VMOE_OK)
         return st;
-    return wgrad_gemm(p, xe, p.d, dqkv, 3 * hd, load, dwqkv, s, "attn_dwqkv");
+    return wgrad_gemm(p, xe, p.d, dqkv, 3 * hd, load, dwqkv, s, "attn_dwqkv", true);
 }
 
 }  // namespace vmoe
