@@ -36,7 +36,8 @@ inline int launch_result() {
 
 // Programmatic dependent launch for the kernels of a step: each launches with
 // programmatic stream serialisation and waits for its predecessor's results
-// (pdl_wait) only after its own set-up -- barriers, TMEM, tensor-map prefetch.
+// (pdl_wait) only after its own set-up -- barriers, TMEM, tensor-map prefetch
+// (a weight gradient that reads none of them waits at its end: late_wait).
 // The grouped GEMMs let their successor launch once every CTA has reached its
 // last tile (pdl_launch_dependents); the other kernels at exit.  Letting it
 // launch at the start measured slower: the waiting CTAs of the successor hold

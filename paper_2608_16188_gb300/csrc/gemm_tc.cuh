@@ -100,7 +100,7 @@ struct Shape {
     static constexpr int STAGES_FIT = (int)((232448 - FIXED) / STAGE_BYTES);
     static constexpr int STAGES_MAX = TMA_EPI ? (BN == 256 ? 3 : 4) : (BN == 256 ? 4 : 6);
     static constexpr int STAGES = STAGES_FIT < STAGES_MAX ? STAGES_FIT : STAGES_MAX;
-    static constexpr uint32_t TMEM_COLS = 2 * BN;
+    static constexpr uint32_t TMEM_COLS = BN == 192 ? 512 : 2 * BN;  // a power of two
     static constexpr int NUM_BARS = 2 * STAGES + 5;
     static constexpr size_t SMEM_BYTES = 1024 + (size_t)STAGES * STAGE_BYTES + EPI_BYTES +
                                          NUM_BARS * 8 + 16 + NT * 4 + (MAX_G + 1) * 4;
@@ -652,6 +652,13 @@ __device__ __forceinline__ void epilogue_chunk(f32x2 (&v)[CH / 2], const uint4 *
     }
 }
 
+// Row mode runs a last wave in halves of its tiles; not dA + GELU', whose prefetch
+// of H needs fixed bounds (with run-time ones it spills: 269 -> 344 us at the 6-task
+// ViT-B step), and not 192 columns, whose half is not a whole number of 64-column boxes.
+constexpr bool cuts_last_wave(int bn, int mode, int epi) {
+    return mode == MODE_ROW && epi != EPI_DGELU && bn != 192;
+}
+
 template <int BN, int MODE, bool A_MN, bool B_MN, int EPI>
 __global__ void __launch_bounds__(Roles<MODE, EPI>::NT, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -661,9 +668,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     constexpr int STAGES = S::STAGES;
     constexpr int NT = S::NT;
     constexpr uint32_t IDESC = idesc_bf16(BM, BN, A_MN, B_MN);
-    // the last wave in pieces; not dA + GELU', whose prefetch of H needs fixed bounds
-    // (with run-time ones it spills: 269 -> 344 us at the 6-task ViT-B step)
-    constexpr bool CUT = MODE == MODE_ROW && EPI != EPI_DGELU;
+    constexpr bool CUT = cuts_last_wave(BN, MODE, EPI);
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -968,7 +973,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
         }
         __syncwarp();
-    } else if (MODE == MODE_WGRAD) {
+    } else if constexpr (MODE == MODE_WGRAD) {
         // ------------------------------------------------------------ epilogue (weight gradients)
         // Every tile is full.  Each warp reads all BN/2 accumulator columns of its
         // 32 rows with back-to-back tcgen05.ld before one wait, then writes 64-
@@ -1166,8 +1171,8 @@ int launch(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &md,
     static std::atomic<int> smem_limit[64];
     if (const int st = raise_smem_limit((const void *)kern, smem_limit, (int)S::SMEM_BYTES)) return st;
     if (max_tiles <= 0) return VMOE_OK;
-    // row mode may cut every tile in two
-    const long long most = MODE == MODE_ROW && EPI != EPI_DGELU ? 2 * max_tiles : max_tiles;
+    // every tile may be cut in two
+    const long long most = cuts_last_wave(BN, MODE, EPI) ? 2 * max_tiles : max_tiles;
     const long long grid = most < num_sms() ? most : num_sms();
     trace_before(s, name);
     const int st = launch_kernel(kern, dim3((unsigned)grid), dim3(S::NT), S::SMEM_BYTES, s, ma, mb,
