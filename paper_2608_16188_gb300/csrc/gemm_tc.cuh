@@ -213,6 +213,38 @@ __device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volati
                                            unsigned long long limit_ns = TIMEOUT_NS) {
     return mbar_try_wait(bar, parity) || wait_phase_slow(bar, parity, abort_flag, status, limit_ns);
 }
+// Arrive on an mbarrier that may live in the peer CTA (release at cluster scope).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
+                 : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Bounded wait with acquire at cluster scope (barriers the peer CTA arrives on).
+static __device__ __noinline__ bool wait_phase_cluster(uint32_t bar, uint32_t parity,
+                                                       volatile int *abort_flag, int *status) {
+    const unsigned long long t0 = global_ns();
+    for (uint32_t i = 1;; ++i) {
+        if (mbar_try_wait_cluster(bar, parity)) return true;
+        if ((i & 63u) == 0) {
+            if (*abort_flag) return false;
+            if (global_ns() - t0 > TIMEOUT_NS) {
+                *abort_flag = 1;
+                if (status) atomicExch(status, (int)VMOE_ERR_DEVICE_TIMEOUT);
+                return false;
+            }
+        }
+    }
+}
 // One lane of a converged warp, the same one every time.  The compiler takes
 // the branch as run by one thread, which a test of the lane index does not tell
 // it: a k-block of four 128 x 128 MMAs with its wait and commit then issues in
@@ -300,7 +332,10 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map
 //
 // One thread a CTA asks (clc_scheduler), CLC_DEPTH answers ahead of the roles;
 // every role reads each answer (clc_take) and frees its slot.  In a pair the
-// leader asks and the answer goes to both CTAs.
+// leader asks and the answer goes to both CTAs, so a slot is free only once every
+// reader in both has read it: the roles of both, and the peer's scheduler, which
+// reads each answer too and would leave early if a later one, the last, overwrote
+// it (the leader's own scheduler reads an answer before it asks for the next).
 constexpr int CLC_DEPTH = 4;
 struct ClcQueue {
     uint4 resp[CLC_DEPTH + 1];  // the last one: draining after an abort
@@ -335,7 +370,7 @@ __device__ __forceinline__ bool clc_query(uint32_t resp, uint32_t &x) {
         : "memory");
     return ok != 0;
 }
-// consumers: arrivals that free a slot (a pair's leader counts both CTAs' roles)
+// consumers: arrivals that free a slot (a pair's leader counts both CTAs' roles and its peer's scheduler)
 __device__ __forceinline__ void clc_init(ClcQueue &q, int consumers) {
     for (int i = 0; i < CLC_DEPTH; ++i) {
         mbar_init(smem_u32(q.full + i), 1);
@@ -343,20 +378,24 @@ __device__ __forceinline__ void clc_init(ClcQueue &q, int consumers) {
     }
     mbar_init(smem_u32(&q.drain), 1);
 }
-// One thread a CTA.  `issue`: this CTA asks (a pair's peer only receives).
+// One thread a CTA.  leader_empty: 0 in the CTA that asks; in a pair's peer, which
+// only receives, the leader's `empty` barriers.
 // After an abort the CTAs not launched yet are taken and dropped, so that none
 // of them starts and runs into the same wait.
 template <bool PAIR>
-__device__ __forceinline__ void clc_scheduler(ClcQueue &q, bool issue, volatile int *abort_flag, int *status) {
+__device__ __forceinline__ void clc_scheduler(ClcQueue &q, uint32_t leader_empty, volatile int *abort_flag,
+                                              int *status) {
+    const bool issue = leader_empty == 0;
     uint32_t ph = 0, x;
     int s = 0;
     bool more = true, ok = true;
     while (more) {
-        if (!wait_phase(smem_u32(q.empty + s), ph ^ 1u, abort_flag, status)) {
+        const uint32_t eb = smem_u32(q.empty + s);  // the peer's readers too: acquire at cluster scope
+        if (!mbar_try_wait_cluster(eb, ph ^ 1u) && !wait_phase_cluster(eb, ph ^ 1u, abort_flag, status)) {
             ok = false;
             break;
         }
-        fence_proxy_async();  // the roles' reads of the slot before it is written again
+        fence_proxy_async();  // the readers' reads of the slot before it is written again
         mbar_expect_tx(smem_u32(q.full + s), 16);
         if (issue) clc_try<PAIR>(smem_u32(q.resp + s), smem_u32(q.full + s));
         if (!wait_phase(smem_u32(q.full + s), ph, abort_flag, status)) {
@@ -367,6 +406,10 @@ __device__ __forceinline__ void clc_scheduler(ClcQueue &q, bool issue, volatile 
             break;
         }
         more = clc_query(smem_u32(q.resp + s), x);
+        if (!issue) {
+            fence_proxy_async();  // this read, too, before the leader's next answer lands in the slot
+            mbar_arrive_cluster(leader_empty + 8u * (uint32_t)s);
+        }
         if (++s == CLC_DEPTH) {
             s = 0;
             ph ^= 1u;
@@ -399,8 +442,7 @@ __device__ __forceinline__ bool clc_take(ClcQueue &q, ClcPos &c, uint32_t &x, vo
     if (WARP) __syncwarp();
     if (!WARP || (threadIdx.x & 31) == 0) {
         mbar_arrive(smem_u32(q.empty + c.s));
-        if (leader_empty)
-            asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(leader_empty + 8u * (uint32_t)c.s) : "memory");
+        if (leader_empty) mbar_arrive_cluster(leader_empty + 8u * (uint32_t)c.s);
     }
     if (++c.s == CLC_DEPTH) {
         c.s = 0;

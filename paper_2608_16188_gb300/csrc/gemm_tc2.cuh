@@ -58,38 +58,6 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-// Arrive on an mbarrier that may live in the peer CTA (release at cluster scope).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait with acquire at cluster scope (barriers the peer CTA arrives on).
-static __device__ __noinline__ bool wait_phase_cluster(uint32_t bar, uint32_t parity,
-                                                       volatile int *abort_flag, int *status) {
-    const unsigned long long t0 = global_ns();
-    for (uint32_t i = 1;; ++i) {
-        if (mbar_try_wait_cluster(bar, parity)) return true;
-        if ((i & 63u) == 0) {
-            if (*abort_flag) return false;
-            if (global_ns() - t0 > TIMEOUT_NS) {
-                *abort_flag = 1;
-                if (status) atomicExch(status, (int)VMOE_ERR_DEVICE_TIMEOUT);
-                return false;
-            }
-        }
-    }
-}
 __device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v) {
     asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
@@ -252,7 +220,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const uint32_t leader_empty = leader ? 0u : mapa_shared(smem_u32(clc.empty), 0);
 
     if (tid == 0) {
-        clc_init(clc, leader ? 2 * PAIR_ROLES : PAIR_ROLES);
+        clc_init(clc, leader ? 2 * PAIR_ROLES + 1 : PAIR_ROLES);  // + 1: the peer's scheduler
         for (int i = 0; i < AS; ++i) {
             mbar_init(bar_afull(i), 1);
             mbar_init(bar_aempty(i), 1);
@@ -429,7 +397,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         give_up();
     } else if (warp == THREADS / 32 + 1) {
         // ------------------------------------------------------------ scheduler
-        if (!sched.enabled && elect_one()) clc_scheduler<true>(clc, leader, abort_flag, args.status);
+        if (!sched.enabled && elect_one()) clc_scheduler<true>(clc, leader_empty, abort_flag, args.status);
         __syncwarp();
         give_up();
     } else if (warp == 1) {
@@ -653,7 +621,7 @@ wgrad_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     const uint32_t leader_empty = leader ? 0u : mapa_shared(smem_u32(clc.empty), 0);
 
     if (tid == 0) {
-        clc_init(clc, leader ? 2 * PAIR_ROLES : PAIR_ROLES);
+        clc_init(clc, leader ? 2 * PAIR_ROLES + 1 : PAIR_ROLES);  // + 1: the peer's scheduler
         for (int i = 0; i < STAGES; ++i) {
             mbar_init(bar_full(i), 2);  // the leader's A and B producers
             mbar_init(bar_empty(i), 1);
@@ -750,7 +718,7 @@ wgrad_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         give_up();
     } else if (warp == THREADS / 32 + 1) {
         // ------------------------------------------------------------ scheduler
-        if (elect_one()) clc_scheduler<true>(clc, leader, abort_flag, args.status);
+        if (elect_one()) clc_scheduler<true>(clc, leader_empty, abort_flag, args.status);
         __syncwarp();
         give_up();
     } else if (warp == 1) {
