@@ -381,7 +381,8 @@ __device__ __forceinline__ void clc_init(ClcQueue &q, int consumers) {
 // One thread a CTA.  leader_empty: 0 in the CTA that asks; in a pair's peer, which
 // only receives, the leader's `empty` barriers.
 // After an abort the CTAs not launched yet are taken and dropped, so that none
-// of them starts and runs into the same wait.
+// of them starts and runs into the same wait -- as long as each answer has been
+// read and held a CTA: asking again after "none left" is undefined.
 template <bool PAIR>
 __device__ __forceinline__ void clc_scheduler(ClcQueue &q, uint32_t leader_empty, volatile int *abort_flag,
                                               int *status) {
@@ -401,8 +402,9 @@ __device__ __forceinline__ void clc_scheduler(ClcQueue &q, uint32_t leader_empty
         if (!wait_phase(smem_u32(q.full + s), ph, abort_flag, status)) {
             ok = false;
             const unsigned long long t0 = global_ns();  // the answer in flight lands before the CTA exits
-            while (!mbar_try_wait(smem_u32(q.full + s), ph) && global_ns() - t0 < 100000000ull) {
-            }
+            bool landed = false;
+            while (!landed && global_ns() - t0 < 100000000ull) landed = mbar_try_wait(smem_u32(q.full + s), ph);
+            more = landed && clc_query(smem_u32(q.resp + s), x);
             break;
         }
         more = clc_query(smem_u32(q.resp + s), x);
@@ -416,7 +418,7 @@ __device__ __forceinline__ void clc_scheduler(ClcQueue &q, uint32_t leader_empty
         }
     }
     pdl_launch_dependents();  // nothing is left to take
-    for (uint32_t n = 0; !ok && issue && n < (1u << 28); ++n) {
+    for (uint32_t n = 0; !ok && more && issue && n < (1u << 28); ++n) {
         const unsigned long long t0 = global_ns();
         fence_proxy_async();
         mbar_expect_tx(smem_u32(&q.drain), 16);

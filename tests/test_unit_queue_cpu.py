@@ -6,6 +6,8 @@ A small model of that protocol (one role a CTA, a ring of two, every interleavin
 which readers have to be among them, and the arrivals are counted in the kernels' source."""
 import os
 import re
+import shutil
+import subprocess
 
 import pytest
 
@@ -82,3 +84,77 @@ def test_the_kernels_count_every_reader(kernel):
     read = sched.index("more = clc_query(")
     assert "mbar_arrive_cluster(leader_empty" in sched[read:]
     assert re.search(r"clc_scheduler[^;(]*\(clc, leader_empty,", body)
+
+
+# clc_scheduler as host code, its primitives played by a script: answer i holds a CTA while i < hold,
+# the wait for answer `fail` gives up, and that answer lands late or never.
+HARNESS = r"""
+#include <cstdint>
+#include <cstdio>
+#include <cstdlib>
+#define __device__
+#define __forceinline__ inline
+struct ClcQueue { int resp[%(depth)d + 1]; uint64_t full[%(depth)d], empty[%(depth)d], drain; };
+constexpr int CLC_DEPTH = %(depth)d;
+static ClcQueue q;
+static int hold, fail, lands, asked, waits, wrong;
+static bool unread, none;
+static unsigned long long now;
+static uint32_t smem_u32(const void *p) { return (uint32_t)((const char *)p - (const char *)&q); }
+static unsigned long long global_ns() { return now += 10000000ull; }
+static bool is(uint32_t bar, const uint64_t *b) { return bar >= smem_u32(b) && bar < smem_u32(b + CLC_DEPTH); }
+static bool wait_phase(uint32_t bar, uint32_t, volatile int *, int *) { return !(is(bar, q.full) && waits++ == fail); }
+static bool mbar_try_wait(uint32_t bar, uint32_t) { return bar == smem_u32(&q.drain) || lands; }
+static bool mbar_try_wait_cluster(uint32_t, uint32_t) { return true; }
+static bool wait_phase_cluster(uint32_t, uint32_t, volatile int *, int *) { return true; }
+static void mbar_expect_tx(uint32_t, uint32_t) {}
+static void mbar_arrive_cluster(uint32_t) {}
+static void fence_proxy_async() {}
+static void pdl_launch_dependents() {}
+template <bool> void clc_try(uint32_t, uint32_t) {
+    if (unread || none) ++wrong;  // asked before the last answer was read, or after "none left"
+    unread = true;
+    ++asked;
+}
+static bool clc_query(uint32_t, uint32_t &x) {
+    unread = false;
+    x = 0;
+    none = asked > hold;
+    return !none;
+}
+%(code)s
+int main(int, char **v) {
+    hold = atoi(v[1]), fail = atoi(v[2]), lands = atoi(v[3]);
+    int flag = 0;
+    clc_scheduler%(args)s;
+    printf("%%d %%d\n", wrong, asked);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def scheduler(tmp_path_factory):
+    if shutil.which("g++") is None:
+        pytest.skip("no host compiler")
+    src = open(os.path.join(CSRC, "gemm_tc.cuh")).read()
+    at = src.index("clc_scheduler(ClcQueue &q")
+    begin = src.rindex("\n//", 0, at)  # behind the comment above it
+    code = src[src.index("\n", begin + 1):src.index("\n}\n", at) + 3].strip()
+    depth = int(re.search(r"constexpr int CLC_DEPTH = (\d+);", src).group(1))
+    args = "<true>" if code.startswith("template") else ""
+    args += "(q, %s, &flag, nullptr)" % ("true" if "bool issue," in code else "0u")
+    d = tmp_path_factory.mktemp("sched")
+    (d / "s.cpp").write_text(HARNESS % {"depth": depth, "code": code, "args": args})
+    subprocess.run(["g++", "-std=c++17", "-O1", "-o", str(d / "s"), str(d / "s.cpp")], check=True)
+    return lambda *a: [int(w) for w in subprocess.run([str(d / "s"), *map(str, a)], check=True, capture_output=True,
+                                                      text=True).stdout.split()]
+
+
+@pytest.mark.parametrize("hold", [0, 1, 7])
+@pytest.mark.parametrize("fail", [-1, 0, 1, 7])
+@pytest.mark.parametrize("lands", [0, 1])
+def test_the_scheduler_never_asks_past_the_last_answer(scheduler, hold, fail, lands):
+    wrong, asked = scheduler(hold, fail, lands)
+    assert wrong == 0
+    if fail < 0 or lands:  # every CTA that was left has been taken, and "none left" read once
+        assert asked == hold + 1
