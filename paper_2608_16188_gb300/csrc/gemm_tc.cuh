@@ -143,19 +143,30 @@ enum { CMP_A = 1, CMP_B = 2, CMP_D = 4 };
 struct TailMaps {
     CUtensorMap a[3];
 };
-__device__ __forceinline__ int real_group(const Args &a, int i) { return a.glist ? __ldg(a.glist + i) : i; }
+__device__ __forceinline__ int real_group(const Args &a, int i) { return a.glist ? a.glist[i] : i; }
 
-// A weight gradient launched right behind a kernel of the same entry point whose
-// outputs it does not read (dW1 behind dX, dW2 behind dW1, ...) starts on the SMs
-// which that kernel's last wave leaves idle: it waits for its predecessor at its
-// end (late_wait) instead of its start.  What it does read was written by kernels
-// that the predecessor itself waited for before it let this one launch, and by
-// waiting before it exits it hands on "complete" to whatever waits for it.
+// A late weight gradient (launch_chain.h: nothing that may still be running writes
+// what it reads, or touches what it writes) starts on the SMs which its predecessor's
+// last wave leaves idle, and waits for its predecessor at its end (late_wait) instead
+// of its start.  By waiting before it exits it hands on "complete" to whatever waits
+// for it.
+// What it reads was written by kernels that had completed before the last launch that
+// waited at its start let its successor start (dW1 behind dX: dH by dA, which dX waited
+// for; dW2 behind a late dW1 that has not waited yet: A and dYe, through dX again).
+// Complete, so performed in L2; but without a wait of its own nothing documented
+// makes that visible here, so it starts with an acquire at GPU scope, for its plain
+// loads (loads, slice plans: never through the non-coherent path), and a proxy fence
+// for its TMA loads, which read L2.
 // Measured on GB300 (us a step or call): ViT-S 214 -> 210, ragged top-3 255 -> 250,
 // 17 tasks 2837 -> 2819, the budgeted backward 2153 -> 2128, attention at C 247
 // 1130 -> 1116.
 __device__ __forceinline__ void wait_for_predecessor(const Args &a, bool at_end) {
-    if ((a.late_wait != 0) == at_end) pdl_wait();
+    if ((a.late_wait != 0) == at_end) {
+        pdl_wait();
+    } else if (!at_end) {
+        __threadfence();
+        asm volatile("fence.proxy.async;" ::: "memory");
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -644,11 +655,11 @@ __device__ __forceinline__ Tile decode_tile(const Args &a, const int *prefix, in
         int tpg = a.tiles_m * a.tiles_n;
         t.g = u / tpg;
         t.gr = real_group(a, t.g);
-        t.crow = a.crow ? __ldg(a.crow + t.g) : 0;
+        t.crow = a.crow ? a.crow[t.g] : 0;
         int local = u - t.g * tpg;
         t.m_blk = local / a.tiles_n;
         t.n_blk = local - t.m_blk * a.tiles_n;
-        int L = __ldg(a.load + t.gr);
+        int L = a.load[t.gr];
         L = L < 0 ? 0 : (L > a.C ? a.C : L);
         t.kvalid = L;
         t.khalf = (L + BK - 1) / BK;

@@ -273,9 +273,9 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     auto decode = [&](int u, int &g, int &n_blk, int &L) {
         const int i = u / args.tiles_n;
         g = real_group(args, i);
-        crow = args.crow ? __ldg(args.crow + i) : 0;
+        crow = args.crow ? args.crow[i] : 0;
         n_blk = u - i * args.tiles_n;
-        L = __ldg(args.load + g);
+        L = args.load[g];
         L = L < 0 ? 0 : (L > args.C ? args.C : L);
     };
     auto give_up = [&]() {
@@ -658,7 +658,7 @@ wgrad_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         const int local = u - t.g * tpg;
         t.m = local / args.tiles_n;
         t.n = local - t.m * args.tiles_n;
-        t.L = __ldg(args.load + t.g);
+        t.L = args.load[t.g];
         t.L = t.L < 0 ? 0 : (t.L > args.C ? args.C : t.L);
         t.nkb = (t.L + BK - 1) / BK;
         return t;
@@ -1415,8 +1415,8 @@ int row_gemm(const Dims &p, const __nv_bfloat16 *act, int K, const __nv_bfloat16
 
 // Weight-gradient GEMM: D[g][M][N] = act1[g][C][M]^T * act2[g][C][N], summed
 // over each group's load[g] rows; both operands MN-major.
-// late: nothing that this reads is written by the launch just before it, of the
-// same entry point (wait_for_predecessor).
+// late: it waits for the launch just before it at its end (wait_for_predecessor); only
+// what LaunchChain::late answers.
 // ksplit: act2 is [G, 2C, N] -- a bf16 part in rows [0, C) and its residual in
 // rows [C, 2C) -- and D = act1^T (hi + lo), summed over both halves.
 // Kernel choice:

@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "gemm_tc2.cuh"
+#include "launch_chain.h"
 #include "planner.cuh"
 
 namespace vmoe {
@@ -55,6 +56,27 @@ int pair_clusters(const void *kern, size_t smem) {
 
 using namespace tc;
 
+namespace {
+// The FFN backward's buffers, as address ranges.
+struct FfnSpans {
+    Span xe, h, act, w1, w2, dye, load, dxe, dw1, dw2;
+    FfnSpans(const Dims &p, const void *xe_, const void *h_, const void *act_, const void *w1_, const void *w2_,
+             const void *dye_, const void *load_, const void *dxe_, const void *dw1_, const void *dw2_) {
+        const size_t rows = (size_t)p.G() * p.C, w = (size_t)p.G() * p.d * p.f * 2;
+        xe = {xe_, rows * p.d * 2};
+        h = {h_, rows * p.f * 2};
+        act = {act_, rows * p.f * 2};
+        w1 = {w1_, w};
+        w2 = {w2_, w};
+        dye = {dye_, rows * p.d * 2};
+        load = {load_, (size_t)p.G() * sizeof(int32_t)};
+        dxe = {dxe_, rows * p.d * 2};
+        dw1 = {dw1_, w};
+        dw2 = {dw2_, w};
+    }
+};
+}  // namespace
+
 int launch_expert_bwd_bf16(const Dims &p, const __nv_bfloat16 *xe, const __nv_bfloat16 *h,
                            const __nv_bfloat16 *act, const __nv_bfloat16 *w1,
                            const __nv_bfloat16 *w2, const __nv_bfloat16 *dye,
@@ -66,14 +88,21 @@ int launch_expert_bwd_bf16(const Dims &p, const __nv_bfloat16 *xe, const __nv_bf
     // (groups with a few rows, where terms cancel) at fp32-like accuracy.
     const long long C = p.C, f = p.f;
     __nv_bfloat16 *dh_hi = dh, *dh_lo = dh + C * f;
+    const FfnSpans b(p, xe, h, act, w1, w2, dye, load, dxe, dw1, dw2);
+    const Span dhs{dh, (size_t)p.G() * 2 * C * f * 2};
+    LaunchChain chain;
     int st = row_gemm<EPI_DGELU, false>(p, dye, p.d, w2, p.f, load, dh_hi, dh_lo, h, s,
                                         "tc_da_dgelu", 2 * C * f, C * f);
     if (st != VMOE_OK) return st;
+    chain.on_time({b.dye, b.w2, b.h, b.load}, {dhs});
     if ((st = row_gemm<EPI_STORE, false>(p, dh_hi, p.f, w1, p.d, load, dxe, nullptr, nullptr, s,
                                          "tc_dx", 0, 0, 2 * C * f)) != VMOE_OK)
         return st;
-    if ((st = wgrad_gemm(p, xe, p.d, dh, p.f, load, dw1, s, "tc_dw1", true, true)) != VMOE_OK) return st;
-    return wgrad_gemm(p, act, p.f, dye, p.d, load, dw2, s, "tc_dw2", true);
+    chain.on_time({dhs, b.w1, b.load}, {b.dxe});
+    const bool late1 = chain.late({b.xe, dhs, b.load}, {b.dw1});
+    if ((st = wgrad_gemm(p, xe, p.d, dh, p.f, load, dw1, s, "tc_dw1", late1, true)) != VMOE_OK) return st;
+    const bool late2 = chain.late({b.act, b.dye, b.load}, {b.dw2});  // beside dX still, behind a late dW1
+    return wgrad_gemm(p, act, p.f, dye, p.d, load, dw2, s, "tc_dw2", late2);
 }
 
 // The backward under a dH budget (the expert groups' temporary memory, Section
@@ -150,6 +179,9 @@ int launch_expert_bwd_bf16_sliced(const Dims &p, const __nv_bfloat16 *xe, const 
     SlicePlanner planner;
     int st = planner.init(G, w.data(), r.data(), cap_units, 0.0, 0.0);
     if (st != VMOE_OK) return st;
+    const FfnSpans b(p, xe, h, act, w1, w2, dye, load, dxe, dw1, dw2);
+    const Span ws{workspace, workspace_bytes};  // the plan and the slices' dH
+    LaunchChain chain;
     // dW2 first: it needs no dH, and it runs while the first slice is planned
     if ((st = wgrad_gemm(p, act, p.f, dye, p.d, load, dw2, s, "tc_dw2", false)) != VMOE_OK) return st;
     int32_t *dplan = reinterpret_cast<int32_t *>(workspace);
@@ -218,10 +250,12 @@ int launch_expert_bwd_bf16_sliced(const Dims &p, const __nv_bfloat16 *xe, const 
         st = row_gemm<EPI_STORE, false>(p, dh, p.f, w1, p.d, load, dxe, nullptr, nullptr, s, "tc_dx", 0,
                                         0, 0, sl);
         if (st != VMOE_OK) break;
+        chain.on_time({ws, b.w1, b.load}, {b.dxe});  // dX; the plan's launch and dA wait at their start too
         sl.compact = CMP_B;
         PairSchedule sc;
         slice_schedule(slice, sc);
-        st = wgrad_gemm(p, xe, p.d, dh, p.f, load, dw1, s, "tc_dw1", true, true, sl, &sc);
+        const bool late = chain.late({b.xe, ws, b.load}, {b.dw1});
+        st = wgrad_gemm(p, xe, p.d, dh, p.f, load, dw1, s, "tc_dw1", late, true, sl, &sc);
         pos += n;
         ++ns;
     }
@@ -248,15 +282,24 @@ int launch_attn_expert_bwd(const Dims &p, int H, const __nv_bfloat16 *xe, const 
     __nv_bfloat16 *dout = static_cast<__nv_bfloat16 *>(workspace);
     __nv_bfloat16 *dqkv = dout + rows * hd;
     float *dsum = reinterpret_cast<float *>(dqkv + rows * 3 * hd);
+    const size_t wbytes = (size_t)p.G() * p.d * hd * 2;
+    const Span sxe{xe, rows * p.d * 2}, sdye{dye, rows * p.d * 2}, so{o, rows * hd * 2}, swo{wo, wbytes},
+        swqkv{wqkv, 3 * wbytes}, sload{load, (size_t)p.G() * sizeof(int32_t)}, sdxe{dxe, rows * p.d * 2},
+        sdwo{dwo, wbytes}, sdwqkv{dwqkv, 3 * wbytes}, sdout{dout, rows * hd * 2}, sdqkv{dqkv, rows * 3 * hd * 2};
+    LaunchChain chain;
     int st = row_gemm<EPI_STORE, false>(p, dye, p.d, wo, hd, load, dout, nullptr, nullptr, s, "attn_dout");
     if (st != VMOE_OK) return st;
-    if ((st = wgrad_gemm(p, o, hd, dye, p.d, load, dwo, s, "attn_dwo", true)) != VMOE_OK) return st;
+    chain.on_time({sdye, swo, sload}, {sdout});
+    const bool late_o = chain.late({so, sdye, sload}, {sdwo});
+    if ((st = wgrad_gemm(p, o, hd, dye, p.d, load, dwo, s, "attn_dwo", late_o)) != VMOE_OK) return st;
     if ((st = launch_attn_core_bwd(p.G(), p.C, H, load, qkv, o, lse, dout, dsum, dqkv, s)) != VMOE_OK)
         return st;
     if ((st = row_gemm<EPI_STORE, false>(p, dqkv, 3 * hd, wqkv, p.d, load, dxe, nullptr, nullptr, s,
                                          "attn_dxe")) != VMOE_OK)
         return st;
-    return wgrad_gemm(p, xe, p.d, dqkv, 3 * hd, load, dwqkv, s, "attn_dwqkv", true);
+    chain.on_time({sdqkv, swqkv, sload}, {sdxe});  // the core's launches wait at their start too
+    const bool late_qkv = chain.late({sxe, sdqkv, sload}, {sdwqkv});
+    return wgrad_gemm(p, xe, p.d, dqkv, 3 * hd, load, dwqkv, s, "attn_dwqkv", late_qkv);
 }
 
 }  // namespace vmoe
