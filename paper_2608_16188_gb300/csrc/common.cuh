@@ -327,11 +327,13 @@ __device__ __forceinline__ f32x2 gelu_deriv2(f32x2 h, bool tanh_form) {
     const float k = -2.0f * 1.4426950408889634f * GELU_TANH_C;
     const f32x2 h2 = mul2(h, h);
     const float2 z = unpk2(mul2(h, fma2(h2, pk2(k * 0.044715f), pk2(k))));
-    // exp(-2u) below overflow, so that (1 - s) s stays 0 and not 0 * inf for large negative h
-    const f32x2 e = exp2_2(pk2(fminf(z.x, 125.0f), fminf(z.y, 125.0f)));
+    const f32x2 e = exp2_2(pk2(z.x, z.y));
     const f32x2 s = rcp2(add2(e, pk2(1.0f)));
     const f32x2 du = fma2(h2, pk2(2.0f * GELU_TANH_C * 3.0f * 0.044715f), pk2(2.0f * GELU_TANH_C));
-    return fma2(mul2(mul2(h, mul2(e, s)), du), s, s);
+    const float2 r = unpk2(fma2(mul2(mul2(h, mul2(e, s)), du), s, s)), hv = unpk2(h);
+    // beyond exp(-2u) = 2^125 (h < -9.8) GELU' is 0 to 1e-34, while e overflows and h du grows
+    // past what s takes back (-5 at h = -1e13); 0 h keeps NaN
+    return pk2(z.x < 125.0f ? r.x : 0.0f * hv.x, z.y < 125.0f ? r.y : 0.0f * hv.y);
 }
 
 }  // namespace vmoe
