@@ -1,4 +1,7 @@
-"""GELU' of the tensor-core epilogues where it is 0 or 1: large |h|, up to where h^2 overflows."""
+"""GELU of the tensor-core epilogues relative to its value in the negative tail, and GELU' where it is 0 or 1: large
+|h|, up to where h^2 overflows."""
+import math
+
 import pytest
 import torch
 
@@ -28,3 +31,31 @@ def test_derivative_far_from_zero(tanh):
     step = (h > 0).double()
     assert torch.isnan(dh[nan]).all()
     assert ((dh - step).abs()[~nan] <= 1e-7).all(), (dh - step).abs()[~nan].max()
+
+
+@pytest.mark.parametrize("tanh", [False, True], ids=["erf", "tanh"])
+def test_gelu_relative_in_the_negative_tail(tanh):
+    """Every bf16 h in [-5, -2^-8]: within half a bf16 ulp of the value (2^-8) and what the approximation adds --
+    formula 7.1.26 evaluated in 64 bits is at most 1.59e-3 of the tail off down to -5; the tanh form has four
+    fp32 roundings in its exponent, |2 u| <= 17 at -5, and two approximate instructions: 17 * 2^-22 + 2^-21."""
+    bits = torch.arange(0x3B80, 0x40A1, dtype=torch.int32)
+    v = (bits | 0x8000).to(torch.int16).view(torch.bfloat16)
+    rows = -(-v.numel() // D)
+    x = torch.zeros(128, D, dtype=torch.bfloat16)
+    x.view(-1)[:v.numel()] = v
+    assert v.double().min() == -5.0 and rows <= 128
+    p = vm.problem(1, D, D, D, 1, 1, 1.0, "bf16", vm.VMOE_GELU_TANH if tanh else 0)
+    load = torch.tensor([[D]], dtype=torch.int32, device="cuda")
+    eye = torch.eye(D, dtype=torch.bfloat16, device="cuda")
+    h, a, ye = (torch.empty(D, D, dtype=torch.bfloat16, device="cuda") for _ in range(3))
+    vm.vmoe_expert_fwd(p, x.cuda(), eye, eye, load, h, a, ye)
+    torch.cuda.synchronize()
+    hv = v.double()
+    if tanh:
+        u = math.sqrt(2.0 / math.pi) * (hv + 0.044715 * hv ** 3)
+        want, more = hv / (1.0 + torch.exp(-2.0 * u)), 17 * 2.0 ** -22 + 2.0 ** -21
+    else:
+        want, more = hv * 0.5 * torch.special.erfc(-hv / math.sqrt(2.0)), 1.6e-3
+    got = a.cpu().double().view(-1)[:v.numel()]
+    off = ((got - want) / want).abs()
+    assert (off <= 2.0 ** -8 + more).all(), (hv[off.argmax()], off.max())
