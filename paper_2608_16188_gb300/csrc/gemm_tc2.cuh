@@ -1211,9 +1211,9 @@ row_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     if (warp == 0) tmem_dealloc_pair(tmem_base, S::TMEM_COLS);
 }
 
-// Clusters of two that fit on the device at once (cached per device); 0 if
-// the query fails.
-int pair_clusters(const void *kern, size_t smem);
+// Clusters of two CTAs of `threads` threads that fit on the device at once (cached
+// per device); 0 if the query fails.
+int pair_clusters(const void *kern, int threads, size_t smem);
 
 template <bool KSPLIT, int NKB>
 int launch_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mblo, const CUtensorMap &md,
@@ -1228,7 +1228,7 @@ int launch_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap 
     PairSchedule sc;
     sc.enabled = 0;
     if (sched && sched->enabled) {  // a share schedule names its own pairs
-        const int ncl = pair_clusters((const void *)kern, S::SMEM_BYTES);
+        const int ncl = pair_clusters((const void *)kern, PAIR_THREADS, S::SMEM_BYTES);
         if (ncl <= 0) return VMOE_ERR_CUDA;
         sc = *sched;
         int used = 0;
@@ -1294,7 +1294,7 @@ int launch_row_pair(const CUtensorMap &ma, const CUtensorMap &mb, const TailMaps
     static std::atomic<int> smem_limit[64];
     if (const int st = raise_smem_limit((const void *)kern, smem_limit, (int)S::SMEM_BYTES)) return st;
     if (max_tiles <= 0) return VMOE_OK;
-    const int ncl = pair_clusters((const void *)kern, S::SMEM_BYTES);
+    const int ncl = pair_clusters((const void *)kern, THREADS, S::SMEM_BYTES);
     if (ncl <= 0) return VMOE_ERR_CUDA;
     const long long clusters = max_tiles < ncl ? max_tiles : ncl;
     cudaLaunchConfig_t cfg = {};
@@ -1325,12 +1325,12 @@ int pair_wgrad_capacity(int C) {
         using S = PairShape<KSPLIT, 2>;
         static std::atomic<int> lim[64];
         if (raise_smem_limit((const void *)wgrad_pair_kernel<KSPLIT, 2>, lim, (int)S::SMEM_BYTES)) return 0;
-        return pair_clusters((const void *)wgrad_pair_kernel<KSPLIT, 2>, S::SMEM_BYTES);
+        return pair_clusters((const void *)wgrad_pair_kernel<KSPLIT, 2>, PAIR_THREADS, S::SMEM_BYTES);
     }
     using S = PairShape<KSPLIT, 4>;
     static std::atomic<int> lim[64];
     if (raise_smem_limit((const void *)wgrad_pair_kernel<KSPLIT, 4>, lim, (int)S::SMEM_BYTES)) return 0;
-    return pair_clusters((const void *)wgrad_pair_kernel<KSPLIT, 4>, S::SMEM_BYTES);
+    return pair_clusters((const void *)wgrad_pair_kernel<KSPLIT, 4>, PAIR_THREADS, S::SMEM_BYTES);
 }
 
 // Row-mode GEMM: D[g][C rows][N] = act[g][C][K] * B, B MN-major ([K][N]) or

@@ -15,7 +15,7 @@ int plan_shares(int n, const double *work, const int32_t *minimum, const int32_t
                 int32_t budget, int32_t *shares);                      // planner.cu
 
 namespace tc {
-int pair_clusters(const void *kern, size_t smem) {
+int pair_clusters(const void *kern, int threads, size_t smem) {
     // per device and kernel: the kernels are few, a small table does
     struct Entry {
         std::atomic<const void *> kern;
@@ -28,7 +28,7 @@ int pair_clusters(const void *kern, size_t smem) {
         if (e.kern.load(std::memory_order_acquire) == kern) return e.n.load(std::memory_order_relaxed);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)num_sms());
-    cfg.blockDim = dim3(PAIR_THREADS);  // the larger of the pair kernels: one CTA an SM either way
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
