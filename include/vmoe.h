@@ -250,12 +250,14 @@ size_t vmoe_attn_expert_bwd_workspace_size(const vmoe_problem *p, int heads);
  *   dXe = dQKV W_qkv^T,  dW_qkv = Xe^T dQKV,
  * P rebuilt from qkv and lse, D formed from the stored o.  The attention core's
  * products take fp16 operands, each staged tile of Q, K, V and dO scaled by a
- * power of two (exact for bf16 values), so P and dS enter dV, dQ and dK with 11
- * significant bits; for C > 128, dQ = dS K instead takes dS as a value plus its
- * residual (fp16, or bf16 for C > 256).  Sums accumulate in fp32.  Inputs as written by the
- * forward (xe, qkv, o, lse) and dye [T,E,C,d] (vmoe_dispatch of dY with the
- * gates); outputs dxe [T,E,C,d]
- * (rows >= load not written), dwqkv [T,E,d,3H64] and dwo [T,E,H64,d] (zero for an
+ * power of two (exact for bf16 values down to 2^-29 of the tile's largest), so P
+ * and dS enter dV, dQ and dK with 11 significant bits; for C > 128, dQ instead
+ * takes bf16 operands and dS as a bf16 value plus its residual.  A row of Q or dO
+ * that is infinite, NaN or 2^29 times the others thus reaches dK and dV of its
+ * whole group and head, and, for C <= 128, the other rows' dQ.  Sums accumulate in
+ * fp32.  Inputs as written by the forward (xe, qkv, o, lse) and dye [T,E,C,d]
+ * (vmoe_dispatch of dY with the gates); outputs dxe [T,E,C,d] (rows >= load not
+ * written), dwqkv [T,E,d,3H64] and dwo [T,E,H64,d] (zero for an
  * empty group).  workspace: caller-owned device scratch of at least
  * vmoe_attn_expert_bwd_workspace_size(p, heads) bytes (else VMOE_ERR_INVALID),
  * its contents clobbered.  Asynchronous on `cuda_stream`. */

@@ -23,12 +23,10 @@
 // The tiles arrive by cp.async; in the forward and the dQ kernel, one commit
 // group per block of 64 keys, so the work on block j overlaps the copies of the
 // blocks after it (dK/dV and the fused backward wait for all of theirs: their
-// operand scales span every row).  The dQ kernel of groups above 256 tokens
-// keeps bf16 operands and takes dS as a bf16 value plus its bf16 residual, two
-// products.  In fp16, every query block's CTA would scale the whole of K and V
-// (measured at 8 tasks and C 248: 245 us with the residual, against 297 us
-// with K and V scaled once all keys have landed, 326 us with each key block
-// scaled as it lands, and 206 us for bf16 with a single product).
+// operand scales span every row).  For groups above 128 tokens S, dP and dQ keep
+// bf16 operands, dS entering dQ as a bf16 value plus its bf16 residual, two products:
+// nothing of a row's dQ then hangs on the other rows' magnitudes, and K and V need
+// no conversion.
 // Keys (or queries) past the load are masked; rows past it are never stored.
 // There are no atomics: dQ is one kernel over query blocks, dK and dV another
 // over key blocks, so every sum runs in a fixed order.
@@ -122,7 +120,7 @@ __device__ __forceinline__ void at_cp_wait(int pending) {
     __syncthreads();
 }
 
-// The backward runs its products on fp16 operands (see the backward's notes
+// The backward runs most of its products on fp16 operands (see the backward's notes
 // below); the forward on bf16.  F16 selects the operand type of a product.
 template <bool F16>
 __device__ __forceinline__ void at_mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
@@ -309,9 +307,10 @@ __global__ void __launch_bounds__(AT_THREADS) attn_fwd_kernel(AtArgs a) {
 
 // ------------------------------------------------------------------ backward operands
 // The fused backward and the dK/dV kernel take fp16 operands, each staged tile
-// scaled by its own power of two (the dQ kernel keeps bf16, see the header).  The inputs are bf16 (8 significant bits), so a bf16 value
-// times 2^e converts to fp16 (11 bits) exactly while it stays an fp16 normal;
-// the products, exact in either type, are then those of the bf16 path.  What
+// scaled by its own power of two (above 128 tokens S, dP and dQ keep bf16, see the
+// header).  The inputs are bf16 (8 significant bits), so a bf16 value times 2^e
+// converts to fp16 (11 bits) exactly while it stays an fp16 normal; the products,
+// exact in either type, are then those of the bf16 path.  What
 // changes is the two values the kernels round for the second products, P (for
 // dV = P^T dO) and dS (for dQ = dS K and dK = dS^T Q): 11 bits instead of 8.
 // Rounded to bf16, the two took 12 heads of 64 at C 124 to 0.021 of a group's
@@ -597,8 +596,10 @@ __global__ void __launch_bounds__(AT_THREADS, AT_MIN_CTAS_BWD) attn_bwd_dkv_kern
 // keys past L), dQ += dS K in registers; P and dS (fp16, as the MMAs round them)
 // go to shared memory, and half of the warps form dV = P^T dO and half dK = dS^T Q
 // for the block's 64 keys, summed over the queries in increasing order.  With 256
-// rows dQ takes dS as an fp16 value and its fp16 residual, as the dQ kernel of
-// larger groups takes it as two bf16 values.
+// rows S, dP and dQ are the dQ kernel's: bf16 operands, dS in dQ as a bf16 value and
+// its residual; each warp holds its rows of Q and dO as bf16 fragments, and the tiles
+// turn to fp16 for dV and dK alone.  (On one fp16 scale for the group, a query row
+// 2^40 times the others', or NaN, left the others' dQ wrong.)
 // Rows, keys and queries past the load rounded up to 32 (16 for the queries) are
 // neither loaded nor multiplied: loads vary from group to group.
 // Measured on GB300 (us): 17 tasks, 12 heads, C 124: 304 with every row of the
@@ -629,22 +630,24 @@ __device__ __forceinline__ void at_mma_tb(float (&acc)[2 * NDP][4], const __nv_b
     }
 }
 
-// A warp's 16 x 8 NT fp32 tile as fp16 into rows row0.. and columns col0.. of a
-// shared [rows][AT_PITCH] tile.
+// A warp's 16 x 8 NT fp32 tile, times mul, as fp16 into rows row0.. and columns
+// col0.. of a shared [rows][AT_PITCH] tile.
 template <int NT>
-__device__ __forceinline__ void at_put(__nv_bfloat16 *tile, int row0, int col0, const float (&v)[NT][4]) {
+__device__ __forceinline__ void at_put(__nv_bfloat16 *tile, int row0, int col0, const float (&v)[NT][4],
+                                       float mul = 1.0f) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
     for (int h = 0; h < 2; ++h)
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
             *reinterpret_cast<uint32_t *>(tile + (row0 + g + 8 * h) * AT_PITCH + col0 + nt * 8 + 2 * t) =
-                at_pack<true>(v[nt][2 * h], v[nt][2 * h + 1]);
+                at_pack<true>(v[nt][2 * h] * mul, v[nt][2 * h + 1] * mul);
 }
 
 template <int ROWS>
 __global__ void __launch_bounds__(2 * ROWS, ROWS == 128 ? 2 : 1) attn_bwd_fused_kernel(AtArgs a) {
     constexpr int NT = 2 * ROWS, W = ROWS / 16;
+    constexpr bool F16 = ROWS == 128;  // S, dP and dQ on fp16 operands too
     pdl_wait();
     const int h = blockIdx.y, g = blockIdx.z;
     const int L = clamp_load(a.load, g, a.C);
@@ -687,20 +690,27 @@ __global__ void __launch_bounds__(2 * ROWS, ROWS == 128 ? 2 : 1) attn_bwd_fused_
         if ((threadIdx.x & 1) == 0 && r < L32) dsh[r] = acc;
         mx[4] = __float_as_uint(fabsf(acc));
     }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & 3, g8 = lane >> 2;
+    const int row0 = warp * 16;
+    const bool active = row0 < L;  // this warp has queries
+    uint32_t qa[4][4] = {}, da[4][4] = {};
+    if (!F16 && active) {  // this warp's rows of Q and dO in bf16, before the tiles turn to fp16
+        at_afrag(qa, qs, row0);
+        at_afrag(da, dos, row0);
+    }
     mx[0] = at_tile_absmax<NT>(qs, L32);
-    mx[1] = at_tile_absmax<NT>(ks, L32);
+    if (F16) mx[1] = at_tile_absmax<NT>(ks, L32);
     mx[2] = at_tile_absmax<NT>(vs, L32);
     mx[3] = at_tile_absmax<NT>(dos, L32);
     at_block_max<5, W>(mx, red);
     const AtScales sc = at_scales(mx, a.scale);
     at_tile_to_f16<NT>(qs, L32, sc.q);
-    at_tile_to_f16<NT>(ks, L32, sc.k);
-    at_tile_to_f16<NT>(vs, L32, sc.v);
     at_tile_to_f16<NT>(dos, L32, sc.dO);
+    if (F16) {
+        at_tile_to_f16<NT>(ks, L32, sc.k);
+        at_tile_to_f16<NT>(vs, L32, sc.v);
+    }
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & 3, g8 = lane >> 2;
-    const int row0 = warp * 16;
-    const bool active = row0 < L;  // this warp has queries
     float lse[2] = {0.0f, 0.0f}, dd[2] = {0.0f, 0.0f};
     bool rv[2];
 #pragma unroll
@@ -709,7 +719,7 @@ __global__ void __launch_bounds__(2 * ROWS, ROWS == 128 ? 2 : 1) attn_bwd_fused_
         rv[h2] = r < L;
         if (active) {
             lse[h2] = lse_s[r];
-            dd[h2] = dsh[r] * sc.d;
+            dd[h2] = F16 ? dsh[r] * sc.d : dsh[r];
         }
     }
     float dq[8][4];
@@ -719,33 +729,30 @@ __global__ void __launch_bounds__(2 * ROWS, ROWS == 128 ? 2 : 1) attn_bwd_fused_
         // in two halves of 32 keys, which holds S and dP in half the registers
 #pragma unroll 1
         for (int k32 = 0; active && k32 < AT_BLK && kb + k32 < L; k32 += 32) {
-            uint32_t fa[4][4];
             float s[4][4], dp[4][4];
             at_zero(s);
             at_zero(dp);
-            at_afrag(fa, qs, row0);
-            at_mma_abt<true, 4>(s, fa, ks, kb + k32);
-            at_afrag(fa, dos, row0);
-            at_mma_abt<true, 4>(dp, fa, vs, kb + k32);
+            if (F16) at_afrag(qa, qs, row0);
+            at_mma_abt<F16, 4>(s, qa, ks, kb + k32);
+            if (F16) at_afrag(qa, dos, row0);
+            at_mma_abt<F16, 4>(dp, F16 ? qa : da, vs, kb + k32);
 #pragma unroll
             for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int key = kb + k32 + nt * 8 + 2 * t + (j & 1);
                     const bool in = key < L && rv[j >> 1];
-                    const float p = in ? __expf(s[nt][j] * sc.s - lse[j >> 1]) : 0.0f;
-                    s[nt][j] = p;                                                  // P
-                    dp[nt][j] = in ? p * (dp[nt][j] * sc.dp - dd[j >> 1]) : 0.0f;  // dS, scaled
+                    const float p = in ? __expf(s[nt][j] * (F16 ? sc.s : a.scale) - lse[j >> 1]) : 0.0f;
+                    s[nt][j] = p;  // P
+                    // dS, with fp16 operands scaled
+                    dp[nt][j] = in ? p * ((F16 ? dp[nt][j] * sc.dp : dp[nt][j]) - dd[j >> 1]) : 0.0f;
                 }
-            at_mma_pb<true, 4>(dq, dp, ks, kb + k32);
             at_put<4>(ps, row0, k32, s);
-            at_put<4>(dss, row0, k32, dp);
-            if (ROWS > 128) {
-#pragma unroll
-                for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) dp[nt][j] -= __half2float(__float2half_rn(dp[nt][j]));
-                at_mma_pb<true, 4>(dq, dp, ks, kb + k32);
+            at_put<4>(dss, row0, k32, dp, F16 ? 1.0f : sc.d);
+            at_mma_pb<F16, 4>(dq, dp, ks, kb + k32);
+            if (!F16) {
+                at_residual(dp);
+                at_mma_pb<false, 4>(dq, dp, ks, kb + k32);
             }
         }
         __syncthreads();
@@ -768,7 +775,7 @@ __global__ void __launch_bounds__(2 * ROWS, ROWS == 128 ? 2 : 1) attn_bwd_fused_
         }
         __syncthreads();  // P and dS of this block are read; the next block rewrites them
     }
-    if (active) at_store(dq, sc.dq, dst, ld, row0, L, h * AT_DK);
+    if (active) at_store(dq, F16 ? sc.dq : a.scale, dst, ld, row0, L, h * AT_DK);
 }
 
 size_t at_smem_fwd(int C) {
