@@ -224,37 +224,11 @@ __device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volati
                                            unsigned long long limit_ns = TIMEOUT_NS) {
     return mbar_try_wait(bar, parity) || wait_phase_slow(bar, parity, abort_flag, status, limit_ns);
 }
-// Arrive on an mbarrier that may live in the peer CTA (release at cluster scope).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait with acquire at cluster scope (barriers the peer CTA arrives on).
-static __device__ __noinline__ bool wait_phase_cluster(uint32_t bar, uint32_t parity,
-                                                       volatile int *abort_flag, int *status) {
-    const unsigned long long t0 = global_ns();
-    for (uint32_t i = 1;; ++i) {
-        if (mbar_try_wait_cluster(bar, parity)) return true;
-        if ((i & 63u) == 0) {
-            if (*abort_flag) return false;
-            if (global_ns() - t0 > TIMEOUT_NS) {
-                *abort_flag = 1;
-                if (status) atomicExch(status, (int)VMOE_ERR_DEVICE_TIMEOUT);
-                return false;
-            }
-        }
-    }
+// Arrive on an mbarrier of another CTA of the cluster without a release at cluster
+// scope, for barriers whose waiter orders through tcgen05 or proxy fences rather than
+// through memory.
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // One lane of a converged warp, the same one every time.  The compiler takes
 // the branch as run by one thread, which a test of the lane index does not tell
@@ -346,7 +320,9 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map
 // leader asks and the answer goes to both CTAs, so a slot is free only once every
 // reader in both has read it: the roles of both, and the peer's scheduler, which
 // reads each answer too and would leave early if a later one, the last, overwrote
-// it (the leader's own scheduler reads an answer before it asks for the next).
+// it (the leader's own scheduler reads an answer before it asks for the next).  Each
+// reader's proxy fence orders its read before its arrive; releases at cluster scope
+// would stall the SM's bulk stores (by every role: 17 tasks 2850 -> 3168 us).
 constexpr int CLC_DEPTH = 4;
 struct ClcQueue {
     uint4 resp[CLC_DEPTH + 1];  // the last one: draining after an abort
@@ -402,8 +378,7 @@ __device__ __forceinline__ void clc_scheduler(ClcQueue &q, uint32_t leader_empty
     int s = 0;
     bool more = true, ok = true;
     while (more) {
-        const uint32_t eb = smem_u32(q.empty + s);  // the peer's readers too: acquire at cluster scope
-        if (!mbar_try_wait_cluster(eb, ph ^ 1u) && !wait_phase_cluster(eb, ph ^ 1u, abort_flag, status)) {
+        if (!wait_phase(smem_u32(q.empty + s), ph ^ 1u, abort_flag, status)) {
             ok = false;
             break;
         }
@@ -421,7 +396,7 @@ __device__ __forceinline__ void clc_scheduler(ClcQueue &q, uint32_t leader_empty
         more = clc_query(smem_u32(q.resp + s), x);
         if (!issue) {
             fence_proxy_async();  // this read, too, before the leader's next answer lands in the slot
-            mbar_arrive_cluster(leader_empty + 8u * (uint32_t)s);
+            mbar_arrive_remote(leader_empty + 8u * (uint32_t)s);
         }
         if (++s == CLC_DEPTH) {
             s = 0;
@@ -455,10 +430,7 @@ __device__ __forceinline__ bool clc_take(ClcQueue &q, ClcPos &c, uint32_t &x, vo
     if (WARP) __syncwarp();
     if (!WARP || (threadIdx.x & 31) == 0) {
         mbar_arrive(smem_u32(q.empty + c.s));
-        // the read above came before it (fence, and the arrive's own release); a release at
-        // cluster scope would wait for the warp's bulk stores too: 17 tasks 2850 -> 3168 us
-        if (leader_empty)
-            asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(leader_empty + 8u * (uint32_t)c.s) : "memory");
+        if (leader_empty) mbar_arrive_remote(leader_empty + 8u * (uint32_t)c.s);
     }
     if (++c.s == CLC_DEPTH) {
         c.s = 0;

@@ -82,7 +82,7 @@ def test_the_kernels_count_every_reader(kernel):
     sched = queue[queue.index("void clc_scheduler("):]
     sched = sched[:sched.index("pdl_launch_dependents();")]
     read = sched.index("more = clc_query(")
-    assert "mbar_arrive_cluster(leader_empty" in sched[read:]
+    assert "mbar_arrive_remote(leader_empty" in sched[read:]
     assert re.search(r"clc_scheduler[^;(]*\(clc, leader_empty,", body)
 
 
@@ -105,10 +105,8 @@ static unsigned long long global_ns() { return now += 10000000ull; }
 static bool is(uint32_t bar, const uint64_t *b) { return bar >= smem_u32(b) && bar < smem_u32(b + CLC_DEPTH); }
 static bool wait_phase(uint32_t bar, uint32_t, volatile int *, int *) { return !(is(bar, q.full) && waits++ == fail); }
 static bool mbar_try_wait(uint32_t bar, uint32_t) { return bar == smem_u32(&q.drain) || lands; }
-static bool mbar_try_wait_cluster(uint32_t, uint32_t) { return true; }
-static bool wait_phase_cluster(uint32_t, uint32_t, volatile int *, int *) { return true; }
 static void mbar_expect_tx(uint32_t, uint32_t) {}
-static void mbar_arrive_cluster(uint32_t) {}
+static void mbar_arrive_remote(uint32_t) {}
 static void fence_proxy_async() {}
 static void pdl_launch_dependents() {}
 template <bool> void clc_try(uint32_t, uint32_t) {
