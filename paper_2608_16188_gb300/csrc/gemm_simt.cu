@@ -108,7 +108,7 @@ __device__ __forceinline__ void simt_store(const SimtArgs &a, int g, long long o
 }
 
 template <int BM, int BN, int TM, int TN, int EPI, bool A_T, bool B_T>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 2 : 6) simt_gemm_kernel(const SimtArgs a) {
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), 6) simt_gemm_kernel(const SimtArgs a) {
     constexpr int NT = (BM / TM) * (BN / TN), CT = BN / TN;
     __shared__ __align__(16) SimtTile<BM, BN> sm;
     pdl_wait();
@@ -174,36 +174,35 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 2 : 6) simt
 #pragma unroll
         for (int j = 0; j < TN; ++j)
             asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[i][j]), "=f"(acc[i + 1][j]) : "l"(acc2[i / 2][j]));
-    if constexpr (BM * BN * sizeof(float) <= sizeof(SimtTile<BM, BN>)) {
-        if (S > 1) {
-            float *red = reinterpret_cast<float *>(&sm);  // [BM][BN]
-            __syncthreads();
+    static_assert(BM * BN * sizeof(float) <= sizeof(SimtTile<BM, BN>), "a partial tile fits the buffers");
+    if (S > 1) {
+        float *red = reinterpret_cast<float *>(&sm);  // [BM][BN]
+        __syncthreads();
 #pragma unroll
-            for (int i = 0; i < TM; ++i)
+        for (int i = 0; i < TM; ++i)
 #pragma unroll
-                for (int r = 0; r < CB; ++r)
-                    *reinterpret_cast<float4 *>(red + ((i / 4) * (BM / RB) + 4 * tm + i % 4) * BN + r * (BN / CB) + 4 * tn) =
-                        make_float4(acc[i][4 * r], acc[i][4 * r + 1], acc[i][4 * r + 2], acc[i][4 * r + 3]);
-            cg::cluster_group cluster = cg::this_cluster();
-            cluster.sync();
-            // rank r finishes rows [BM r / S, BM (r + 1) / S), the ranks' parts summed in order
-            const int rows = BM / S;
-            for (int u = threadIdx.x; u < rows * (BN / 4); u += NT) {
-                const int r = rank * rows + u / (BN / 4), n = u % (BN / 4) * 4;
-                if (m0 + r >= M || n0 + n >= a.N) continue;
-                float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                for (int q = 0; q < S; ++q) {
-                    const float4 w = *reinterpret_cast<const float4 *>(cluster.map_shared_rank(red, q) + r * BN + n);
-                    v.x += w.x;
-                    v.y += w.y;
-                    v.z += w.z;
-                    v.w += w.w;
-                }
-                simt_store<EPI>(a, g, (long long)(m0 + r) * a.ldd + n0 + n, v);
+            for (int r = 0; r < CB; ++r)
+                *reinterpret_cast<float4 *>(red + ((i / 4) * (BM / RB) + 4 * tm + i % 4) * BN + r * (BN / CB) + 4 * tn) =
+                    make_float4(acc[i][4 * r], acc[i][4 * r + 1], acc[i][4 * r + 2], acc[i][4 * r + 3]);
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();
+        // rank r finishes rows [BM r / S, BM (r + 1) / S), the ranks' parts summed in order
+        const int rows = BM / S;
+        for (int u = threadIdx.x; u < rows * (BN / 4); u += NT) {
+            const int r = rank * rows + u / (BN / 4), n = u % (BN / 4) * 4;
+            if (m0 + r >= M || n0 + n >= a.N) continue;
+            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (int q = 0; q < S; ++q) {
+                const float4 w = *reinterpret_cast<const float4 *>(cluster.map_shared_rank(red, q) + r * BN + n);
+                v.x += w.x;
+                v.y += w.y;
+                v.z += w.z;
+                v.w += w.w;
             }
-            cluster.sync();  // the parts stay until every rank has read them
-            return;
+            simt_store<EPI>(a, g, (long long)(m0 + r) * a.ldd + n0 + n, v);
         }
+        cluster.sync();  // the parts stay until every rank has read them
+        return;
     }
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
@@ -246,18 +245,21 @@ int run_tile(SimtArgs a, int G, int mmax, int split, cudaStream_t s, const char 
     return e == cudaSuccess ? VMOE_OK : VMOE_ERR_CUDA;
 }
 
-// Tile choice.  A warp's shared-memory reads cost TM + TN wavefronts a k against
-// TM * TN / 4 cycles of its scheduler's FMA pipe, so 16 x 8 outputs a thread run
-// nearest the FMA rate: 128 x 128 tiles wherever they give every SM two CTAs.
-// Below that 64 x 64 tiles of 8 x 4 (8 x 8 left too few warps: 16-wide rows of
-// K = 256 took 13 us instead of 10), and a K split over up to 8 CTAs while the
-// tiles give an SM fewer than three CTAs and a part keeps 3 chunks or more.
+// Tile choice: 64 x 64 tiles of 8 x 4 outputs a thread (8 x 8 left too few warps:
+// 16-wide rows of K = 256 took 13 us instead of 10), and a K split over up to 8 CTAs
+// while the tiles give an SM fewer than three CTAs and a part keeps 3 chunks or more.
+// 128 x 128 tiles of 16 x 8, nearer the FMA rate on paper (a warp's shared-memory
+// reads cost TM + TN wavefronts a k against TM * TN / 4 cycles of its scheduler's FMA
+// pipe), run two CTAs an SM and multiply 128 rows for any load: over 12 layers, C 33
+// to 2400 and loads of a third to all of C they took 0.9 to 4 times these tiles'
+// time, above 1 but for the weight gradients of d 384, f 1536 and d 512, f 2048
+// (0.95-0.97) and row GEMMs with 2400 rows in every group.
 // Measured on GB300 (us; the 64 x 64 kernel of 4 x 4 outputs that this replaced
-// -> now), ViT-S in fp32, 16 groups of about 98 rows: FC1 178 -> 70, FC2 344 ->
-// 70, dA 132 -> 73, dX 311 -> 72, dW1 102 -> 48, dW2 112 -> 48 (39 TFLOP/s of
-// the CUDA cores' 80); the 8-expert layer of d 64, f 256: FC2 37 -> 11, dX 38 ->
-// 10, the others 12-16 -> 8-11.  Row mode stays at 47% of the FMA pipe: half of
-// its second 64-row tile is padding, and shared-memory reads fill 75% of the L1.
+// -> now), 512 groups of 10 rows at C 33, d 64, f 256: FC2 69 -> 33, dX 57 -> 33, dA
+// 51 -> 33 (100, 93 and 67 with 128 x 128); 48 groups of 300 at C 500, d 200, f 800:
+// FC1 297 -> 119, dW1 330 -> 129.
+// Row mode stays at 47% of the FMA pipe: half of its second 64-row tile is padding,
+// and shared-memory reads fill 75% of the L1.
 // Groups of at most 32 rows take tiles of 16 or 32 rows instead of computing 64 (6
 // tasks of 30 experts of at most 13 rows, d 336, f 1168: the step 1807 -> 607 us).
 // kmax: the longest reduction (row mode: K; weight gradients: C rows).
@@ -265,8 +267,6 @@ template <int EPI, bool A_T, bool B_T>
 int run(const SimtArgs &a, int G, int mmax, cudaStream_t s, const char *name) {
     const int kmax = a.row_mode ? a.K : a.C;
     const long long sms = num_sms();
-    const long long big = (long long)((a.N + 127) / 128) * ((mmax + 127) / 128) * G;
-    if (big >= 2 * sms && !(a.row_mode && mmax <= 32)) return run_tile<128, 128, 16, 8, EPI, A_T, B_T>(a, G, mmax, 1, s, name);
     const bool few = a.row_mode && mmax <= 32;  // one tile of 16 or 32 rows a group
     const long long small = few ? (long long)((a.N + 127) / 128) * G
                                 : (long long)((a.N + 63) / 64) * ((mmax + 63) / 64) * G;
