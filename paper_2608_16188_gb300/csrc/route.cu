@@ -56,45 +56,49 @@ route_given_kernel(Dims p, const float *__restrict__ logits, int32_t *__restrict
     topk_rows(p, smem, E + 1, ntok, t, n0, out_idx, out_gate, RT_THREADS);
 }
 
-// CUDA-core router for fp32 tokens: RF_TOK tokens x ECH experts a pass, 4 x 4
-// logits a thread.  d is swept in chunks of RF_KC staged in shared memory (the
-// next chunk's loads in registers meanwhile); RF_SLICES groups of threads take
-// a slice of every chunk each, and their partial logits are summed in slice
-// order.  A layer's few hundred tokens are a few dozen CTAs, so the chain of
-// chunks is what bounds it, not the arithmetic.
-constexpr int RF_TOK = 16;
-constexpr int RF_KC = 128;
-constexpr int RF_XP = RF_KC + 4;  // x row pitch (floats)
-template <int ECH>
+// CUDA-core router for fp32 tokens: TOK tokens x ECH experts a pass, 4 x 4 logits a
+// thread.  d is swept in chunks of KC staged in shared memory (the next chunk's
+// loads in registers meanwhile); SLICES groups of threads take a slice of every
+// chunk each, and their partial logits are summed in slice order.
+// Two forms.  Few tokens (a layer's few hundred are a few dozen CTAs) are bound by
+// the chain of chunks: 16 tokens a CTA, chunks of 128, 4 or 8 slices.  Many tokens
+// are bound by arithmetic, by the weights each CTA stages and by its top-k threads:
+// 64 tokens, chunks of 32, one slice (launch_route has the rule).
+template <int ECH, int TOK, int KC, int SLICES_>
 struct RouteF32 {
-    static constexpr int EG = ECH / 4;                         // threads along experts
-    static constexpr int SLICES = RT_THREADS / (EG * (RF_TOK / 4));
-    static constexpr int KS = RF_KC / SLICES;                  // d per slice and chunk
-    static constexpr int XV = RF_TOK * RF_KC / 4 / RT_THREADS;  // x vectors per thread
-    static constexpr int WV = RF_KC * ECH / RT_THREADS;        // weights per thread
+    static constexpr int SLICES = SLICES_;
+    static constexpr int XP = KC + 4;                // x row pitch (floats)
+    static constexpr int EG = ECH / 4;               // threads along experts
+    static constexpr int NT = EG * (TOK / 4) * SLICES;  // threads
+    static constexpr int CTAS = SLICES > 1 ? 2 : NT == 128 ? 7 : 4;  // an SM
+    static constexpr int KS = KC / SLICES;           // d per slice and chunk
+    static constexpr int XV = TOK * KC / 4 / NT;     // x vectors per thread
+    static constexpr int WV = KC * ECH / NT;         // weights per thread
+    static constexpr int PARTS = SLICES > 1 ? SLICES * TOK * ECH : 0;
     static constexpr size_t smem(int E) {
-        return sizeof(float) * ((size_t)RF_TOK * RF_XP + (size_t)RF_KC * ECH +
-                                (size_t)SLICES * RF_TOK * ECH + (size_t)RF_TOK * (E + 1));
+        return sizeof(float) * ((size_t)TOK * XP + (size_t)KC * ECH + PARTS + (size_t)TOK * (E + 1));
     }
     static_assert(KS % 4 == 0, "a slice is swept four values of d at a time");
+    static_assert(XV * NT * 4 == TOK * KC && WV * NT == KC * ECH, "every thread stages as much");
 };
 
-template <int ECH>
-__global__ void __launch_bounds__(RT_THREADS)
+template <int ECH, int TOK, int KC, int SLICES>
+__global__ void __launch_bounds__(RouteF32<ECH, TOK, KC, SLICES>::NT, RouteF32<ECH, TOK, KC, SLICES>::CTAS)
 route_f32_kernel(Dims p, const float *__restrict__ x, const float *__restrict__ wr,
                  const float *__restrict__ bias, float *__restrict__ logits,
                  int32_t *__restrict__ out_idx, float *__restrict__ out_gate) {
-    using S = RouteF32<ECH>;
+    using S = RouteF32<ECH, TOK, KC, SLICES>;
+    constexpr int NT = S::NT, UNROLL = SLICES == 1 ? 1 : 2;
     pdl_wait();
     extern __shared__ __align__(16) float smem[];
-    float *xs = smem;                            // [RF_TOK][RF_XP]
-    float *ws = xs + RF_TOK * RF_XP;             // [RF_KC][ECH]
-    float *part = ws + RF_KC * ECH;              // [SLICES][RF_TOK][ECH]
-    float *lg = part + S::SLICES * RF_TOK * ECH;  // [RF_TOK][E + 1]
-    const int t = blockIdx.y, n0 = blockIdx.x * RF_TOK;
+    float *xs = smem;               // [TOK][S::XP]
+    float *ws = xs + TOK * S::XP;   // [KC][ECH]
+    float *part = ws + KC * ECH;    // [SLICES][TOK][ECH], with more than one slice
+    float *lg = part + S::PARTS;    // [TOK][E + 1]
+    const int t = blockIdx.y, n0 = blockIdx.x * TOK;
     const int E = p.E, d = p.d, N = p.N, ldl = E + 1, tid = threadIdx.x;
-    const int ntok = min(RF_TOK, N - n0);
-    const int eg = tid % S::EG, tg = tid / S::EG % (RF_TOK / 4), sl = tid / (S::EG * (RF_TOK / 4));
+    const int ntok = min(TOK, N - n0);
+    const int eg = tid % S::EG, tg = tid / S::EG % (TOK / 4), sl = tid / (S::EG * (TOK / 4));
     const float *xt = x + ((long long)t * N + n0) * d;
     const float *wt = wr + (long long)t * d * E;
     float4 xv[S::XV];
@@ -448,6 +452,8 @@ int launch_mma_router(const Dims &p, const __nv_bfloat16 *x, const float *wr, co
 // a warp turns its own ranks into slots (us: ViT-S, 4 tasks of 1576 tokens, top-2
 // 10.2 -> 7.9; 6 of 3152 14.3 -> 13.4; 17 of 1576, where its loads wait for DRAM,
 // 10.6 either way).
+// The counters' pitch is odd: a warp scans one expert's column.
+__host__ __device__ constexpr int cs_pitch(int E) { return E | 1; }
 template <bool SMEM_IDX, int CS_THREADS>
 __global__ void __launch_bounds__(CS_THREADS)
 capacity_scan_kernel(Dims p, const int32_t *__restrict__ idx, int32_t *__restrict__ slot,
@@ -455,13 +461,14 @@ capacity_scan_kernel(Dims p, const int32_t *__restrict__ idx, int32_t *__restric
     constexpr int CS_WARPS = CS_THREADS / 32;
     pdl_wait();
     extern __shared__ int cs_smem[];
-    int *cnt = cs_smem;  // [CS_WARPS][E]
     const int t = blockIdx.x;
     const int E = p.E, N = p.N, k = p.k, C = p.C;
+    const int ldc = cs_pitch(E);
+    int *cnt = cs_smem;  // [CS_WARPS][ldc]
     const int total = k * N;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long tb = (long long)t * N * k;
-    int *sidx = cs_smem + CS_WARPS * E;  // [N*k] in token-major (memory) order
+    int *sidx = cs_smem + CS_WARPS * ldc;  // [N*k] in token-major (memory) order
     int *srank = sidx + total;           // [N*k]
     if (SMEM_IDX) {
         constexpr int U = 4;  // loads in flight a thread
@@ -475,14 +482,14 @@ capacity_scan_kernel(Dims p, const int32_t *__restrict__ idx, int32_t *__restric
                 if (i0 + u * CS_THREADS < total) sidx[i0 + u * CS_THREADS] = v[u];
         }
     }
-    for (int i = threadIdx.x; i < CS_WARPS * E; i += CS_THREADS) cnt[i] = 0;
+    for (int i = threadIdx.x; i < CS_WARPS * ldc; i += CS_THREADS) cnt[i] = 0;
     __syncthreads();
     const int32_t *src = SMEM_IDX ? sidx : idx + tb;
     int32_t *rank = SMEM_IDX ? srank : slot + tb;
 
     const int per = ((total + CS_WARPS - 1) / CS_WARPS + 31) & ~31;
     const int beg = min(total, warp * per), end = min(total, beg + per);
-    int *my = cnt + warp * E;
+    int *my = cnt + warp * ldc;
     const unsigned lt = (1u << lane) - 1u;
     // the lane's first position beg + lane of the choice-major sequence p = j*N + n
     const int j_beg = (beg + lane) / N, n_beg = (beg + lane) - j_beg * N;
@@ -505,23 +512,50 @@ capacity_scan_kernel(Dims p, const int32_t *__restrict__ idx, int32_t *__restric
         __syncwarp();  // every lane has read its counter
         if (valid && before == 0) my[e] = base + __popc(peers);
         __syncwarp();
-        advance(n, j);
+        if (p0 + 32 < end) advance(n, j);
     }
     __syncthreads();
-    // Exclusive scan over warps, per expert: a warp an expert, lane w its counter of warp w.
-    for (int e = warp; e < E; e += CS_WARPS) {
-        const int c = lane < CS_WARPS ? cnt[lane * E + e] : 0;
-        int incl = c;
+    // Exclusive scan over warps, per expert: a warp an expert, lane w its counter of
+    // warp w; with 8 warps a thread an expert.
+    if (CS_WARPS == 32) {
+        for (int e = warp; e < E; e += CS_WARPS) {
+            const int c = cnt[lane * ldc + e];
+            int incl = c;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            cnt[lane * ldc + e] = incl - c;
+            if (lane == 31) load[(long long)t * E + e] = min(incl, C);
         }
-        if (lane < CS_WARPS) cnt[lane * E + e] = incl - c;
-        if (lane == 31) load[(long long)t * E + e] = min(incl, C);
+    } else {
+        for (int e = threadIdx.x; e < E; e += CS_THREADS) {
+            int run = 0;
+#pragma unroll 8
+            for (int w = 0; w < CS_WARPS; ++w) {
+                const int c = cnt[w * ldc + e];
+                cnt[w * ldc + e] = run;
+                run += c;
+            }
+            load[(long long)t * E + e] = min(run, C);
+        }
     }
     __syncthreads();
-    // Pass 2: each warp's ranks -> slots.
+    // Pass 2: ranks -> slots, each warp its own; from four choices on, whose places lie
+    // apart, in memory order, the warp that ranked a place looked up: w = pos / per (both
+    // quotients by a reciprocal: exact, as they lie half a part from an integer and total
+    // is below 2^14).
+    if (SMEM_IDX && k > 3) {
+        const float rk = 1.0f / (float)k, rper = 1.0f / (float)per;
+        for (int i = threadIdx.x; i < total; i += CS_THREADS) {
+            const int q = (int)(((float)i + 0.5f) * rk);
+            const int w = (int)(((float)((i - q * k) * N + q) + 0.5f) * rper);
+            const int r = srank[i] + cnt[w * ldc + sidx[i]];
+            slot[tb + i] = r < C ? r : -1;
+        }
+        return;
+    }
     n = n_beg;
     j = j_beg;
     for (int p0 = beg; p0 < end; p0 += 32) {
@@ -529,7 +563,7 @@ capacity_scan_kernel(Dims p, const int32_t *__restrict__ idx, int32_t *__restric
             const int i = n * k + j, r = rank[i] + my[src[i]];
             slot[tb + i] = r < C ? r : -1;
         }
-        advance(n, j);
+        if (p0 + 32 < end) advance(n, j);
     }
 }
 
@@ -560,7 +594,7 @@ int launch_f32(const Dims &p, const float *x, const float *wr, const float *bias
 template <int CS_THREADS>
 int launch_scan(const Dims &p, const int32_t *idx, int32_t *slot, int32_t *load, cudaStream_t s) {
     const size_t total = (size_t)p.N * p.k;
-    const size_t smem_small = sizeof(int) * (size_t)(CS_THREADS / 32) * p.E;
+    const size_t smem_small = sizeof(int) * (size_t)(CS_THREADS / 32) * cs_pitch(p.E);
     const size_t smem_big = smem_small + sizeof(int) * 2 * total;
     if (smem_big <= 96 * 1024) {
         static std::atomic<int> smem_limit[64];
