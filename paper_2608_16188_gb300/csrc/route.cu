@@ -107,36 +107,36 @@ route_f32_kernel(Dims p, const float *__restrict__ x, const float *__restrict__ 
         auto load = [&](int k0) {
 #pragma unroll
             for (int q = 0; q < S::XV; ++q) {  // d % 8 == 0: a vector is inside its row or past it
-                const int i = tid + q * RT_THREADS, r = i / (RF_KC / 4), c = i % (RF_KC / 4) * 4;
+                const int i = tid + q * NT, r = i / (KC / 4), c = i % (KC / 4) * 4;
                 xv[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 if (r < ntok && k0 + c < d)
                     xv[q] = __ldg(reinterpret_cast<const float4 *>(xt + (long long)r * d + k0 + c));
             }
 #pragma unroll
             for (int q = 0; q < S::WV; ++q) {
-                const int i = tid + q * RT_THREADS, r = i / ECH, c = i % ECH;
+                const int i = tid + q * NT, r = i / ECH, c = i % ECH;
                 wv[q] = k0 + r < d && e0 + c < E ? __ldg(wt + (long long)(k0 + r) * E + e0 + c) : 0.0f;
             }
         };
         float acc[4][4] = {};
         load(0);
-        for (int k0 = 0; k0 < d; k0 += RF_KC) {
+        for (int k0 = 0; k0 < d; k0 += KC) {
             __syncthreads();  // the previous chunk has been read
 #pragma unroll
             for (int q = 0; q < S::XV; ++q) {
-                const int i = tid + q * RT_THREADS;
-                *reinterpret_cast<float4 *>(xs + i / (RF_KC / 4) * RF_XP + i % (RF_KC / 4) * 4) = xv[q];
+                const int i = tid + q * NT;
+                *reinterpret_cast<float4 *>(xs + i / (KC / 4) * S::XP + i % (KC / 4) * 4) = xv[q];
             }
 #pragma unroll
-            for (int q = 0; q < S::WV; ++q) ws[tid + q * RT_THREADS] = wv[q];
+            for (int q = 0; q < S::WV; ++q) ws[tid + q * NT] = wv[q];
             __syncthreads();
-            if (k0 + RF_KC < d) load(k0 + RF_KC);
-#pragma unroll 2
+            if (k0 + KC < d) load(k0 + KC);
+#pragma unroll UNROLL
             for (int kk = sl * S::KS; kk < (sl + 1) * S::KS; kk += 4) {
                 float4 a[4], b[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    a[i] = *reinterpret_cast<const float4 *>(xs + (4 * tg + i) * RF_XP + kk);
+                    a[i] = *reinterpret_cast<const float4 *>(xs + (4 * tg + i) * S::XP + kk);
                     b[i] = *reinterpret_cast<const float4 *>(ws + (kk + i) * ECH + 4 * eg);
                 }
 #pragma unroll
@@ -152,24 +152,37 @@ route_f32_kernel(Dims p, const float *__restrict__ x, const float *__restrict__ 
                 }
             }
         }
+        if (SLICES == 1) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int r = 4 * tg + i, e = e0 + 4 * eg + q;
+                    if (r < ntok && e < E) lg[r * ldl + e] = acc[i][q] + (bias ? bias[(long long)t * E + e] : 0.0f);
+                }
+            continue;
+        }
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            *reinterpret_cast<float4 *>(part + (sl * RF_TOK + 4 * tg + i) * ECH + 4 * eg) =
+            *reinterpret_cast<float4 *>(part + (sl * TOK + 4 * tg + i) * ECH + 4 * eg) =
                 make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
         __syncthreads();
-        for (int i = tid; i < RF_TOK * ECH; i += RT_THREADS) {
+        for (int i = tid; i < TOK * ECH; i += NT) {
             const int r = i / ECH, e = e0 + i % ECH;
             if (r >= ntok || e >= E) continue;
             float v = part[i];
 #pragma unroll
-            for (int q = 1; q < S::SLICES; ++q) v += part[q * RF_TOK * ECH + i];
+            for (int q = 1; q < SLICES; ++q) v += part[q * TOK * ECH + i];
             if (bias) v += bias[(long long)t * E + e];
             lg[r * ldl + e] = v;
             logits[((long long)t * N + n0 + r) * E + e] = v;
         }
     }
     __syncthreads();
-    topk_rows(p, lg, ldl, ntok, t, n0, out_idx, out_gate, RT_THREADS);
+    if (SLICES == 1)
+        for (int i = tid; i < ntok * E; i += NT)
+            logits[((long long)t * N + n0) * E + i] = lg[i / E * ldl + i % E];
+    topk_rows(p, lg, ldl, ntok, t, n0, out_idx, out_gate, NT);
 }
 
 // Tensor-core router for bf16 tokens.  x is exactly representable in bf16, so
@@ -578,15 +591,17 @@ int launch_given(const Dims &p, const float *logits, int32_t *idx, float *gate, 
     return st;
 }
 
-template <int ECH>
+template <int ECH, int TOK, int KC, int SLICES>
 int launch_f32(const Dims &p, const float *x, const float *wr, const float *bias, float *logits,
                int32_t *idx, float *gate, cudaStream_t s) {
-    const size_t smem = RouteF32<ECH>::smem(p.E);
+    using S = RouteF32<ECH, TOK, KC, SLICES>;
+    const size_t smem = S::smem(p.E);
     static std::atomic<int> smem_limit[64];
-    if (const int st = raise_smem_limit((const void *)route_f32_kernel<ECH>, smem_limit, (int)smem)) return st;
+    auto kern = route_f32_kernel<ECH, TOK, KC, SLICES>;
+    if (const int st = raise_smem_limit((const void *)kern, smem_limit, (int)smem)) return st;
     trace_before(s, "route_topk");
-    const int st = launch_kernel(route_f32_kernel<ECH>, dim3((p.N + RF_TOK - 1) / RF_TOK, p.T), dim3(RT_THREADS),
-                                 smem, s, p, x, wr, bias, logits, idx, gate);
+    const int st = launch_kernel(kern, dim3((p.N + TOK - 1) / TOK, p.T), dim3(S::NT), smem, s, p, x, wr, bias,
+                                 logits, idx, gate);
     trace_after(s);
     return st;
 }
@@ -625,8 +640,17 @@ int launch_route(const Dims &p, const void *x, const float *w_router, const floa
         st = launch_given(p, logits, idx, gate, s);
     } else {
         const float *xf = (const float *)x;
-        st = p.E <= 32 ? launch_f32<32>(p, xf, w_router, bias, logits, idx, gate, s)
-                       : launch_f32<64>(p, xf, w_router, bias, logits, idx, gate, s);
+        // measured against the 16-token form (us, with the scan; 3 to 6000 tokens a task, d 8 to
+        // 640, 4 to 256 experts): 100 tiles, E 64, d 8: 23.8 -> 14, d 264: 33.9 -> 25, but E 32, d
+        // 640: 26.3 -> 30.1; 752 tiles, E 128, d 16: 197 -> 65; 50 tiles, d 136: slower from there on
+        const long long tiles = (long long)((p.N + 63) / 64) * p.T;
+        const bool many = tiles >= num_sms() || (2 * tiles >= num_sms() && p.d <= 512);
+        if (many)
+            st = p.E <= 32 ? launch_f32<32, 64, 32, 1>(p, xf, w_router, bias, logits, idx, gate, s)
+                           : launch_f32<64, 64, 32, 1>(p, xf, w_router, bias, logits, idx, gate, s);
+        else
+            st = p.E <= 32 ? launch_f32<32, 16, 128, 8>(p, xf, w_router, bias, logits, idx, gate, s)
+                           : launch_f32<64, 16, 128, 4>(p, xf, w_router, bias, logits, idx, gate, s);
     }
     if (st != VMOE_OK) return st;
     trace_before(s, "capacity_scan");
