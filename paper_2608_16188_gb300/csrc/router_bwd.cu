@@ -722,13 +722,14 @@ constexpr int RT = 64;
 constexpr int RKC = 32;
 constexpr int RD_THREADS = 256;
 
+template <bool SPLIT>
 __global__ void __launch_bounds__(RD_THREADS)
-router_dw_simt_kernel(Dims p, int split, const float *__restrict__ x, const float *__restrict__ dl,
+router_dw_simt_kernel(Dims p, int nsplit, const float *__restrict__ x, const float *__restrict__ dl,
                       float *__restrict__ dw, float *__restrict__ dbias) {
     __shared__ __align__(16) float buf[2][RKC][RT];  // x and dlogit rows of a chunk; then the partial tile [RT][RT]
     __shared__ float bias_part[RT];
     float(*xs)[RT] = buf[0], (*ds)[RT] = buf[1];
-    const int rank = (int)(blockIdx.x % split);
+    const int split = SPLIT ? nsplit : 1, rank = (int)(blockIdx.x % split);
     const int t = blockIdx.z, i0 = (int)(blockIdx.x / split) * RT, e0 = blockIdx.y * RT;
     const int tid = threadIdx.x, ti = tid / 16, tj = tid % 16;
     const int d = p.d, E = p.E, N = p.N;
@@ -780,6 +781,21 @@ router_dw_simt_kernel(Dims p, int split, const float *__restrict__ x, const floa
         }
         __syncthreads();
     }
+    float *dwt = dw + (long long)t * d * E;
+    if (!SPLIT) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int i = i0 + ti * 4 + a;
+            if (i >= d) continue;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int e = e0 + tj * 4 + b;
+                if (e < E) dwt[(long long)i * E + e] = acc[a][b];
+            }
+        }
+        if (do_bias && tid < RT && e0 + tid < E) dbias[(long long)t * E + e0 + tid] = bacc;
+        return;
+    }
     float *part = &buf[0][0][0];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
@@ -787,7 +803,6 @@ router_dw_simt_kernel(Dims p, int split, const float *__restrict__ x, const floa
     if (tid < RT) bias_part[tid] = bacc;
     cg::cluster_group cluster = cg::this_cluster();
     cluster.sync();
-    float *dwt = dw + (long long)t * d * E;
     for (int i = rank * RD_THREADS + tid; i < RT * RT; i += split * RD_THREADS) {
         const int r = i / RT, c = i % RT;
         if (i0 + r >= d || e0 + c >= E) continue;
@@ -807,6 +822,10 @@ int launch_router_dw_simt(const Dims &p, const float *x, const float *dl, float 
     const int tiles_d = (p.d + RT - 1) / RT, tiles_e = (p.E + RT - 1) / RT;
     int split = 1;  // more CTAs a tile while SMs are idle and each keeps two chunks
     while (split < 8 && (long long)tiles_d * tiles_e * p.T * split < 2LL * num_sms() && p.N >= split * 4 * RKC) split *= 2;
+    if (split == 1) {
+        router_dw_simt_kernel<false><<<dim3(tiles_d, tiles_e, p.T), RD_THREADS, 0, s>>>(p, 1, x, dl, dw, dbias);
+        return launch_result();
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(tiles_d * split), tiles_e, p.T);
     cfg.blockDim = dim3(RD_THREADS);
@@ -818,8 +837,9 @@ int launch_router_dw_simt(const Dims &p, const float *x, const float *dl, float 
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, router_dw_simt_kernel, p, split, x, dl, dw, dbias) == cudaSuccess ? VMOE_OK
-                                                                                                     : VMOE_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, router_dw_simt_kernel<true>, p, split, x, dl, dw, dbias) == cudaSuccess
+               ? VMOE_OK
+               : VMOE_ERR_CUDA;
 }
 
 // ---------------------------------------------------------------------------
