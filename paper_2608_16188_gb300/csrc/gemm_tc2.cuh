@@ -1456,6 +1456,25 @@ int row_gemm(const Dims &p, const __nv_bfloat16 *act, int K, const __nv_bfloat16
 //     second line): the one-SM streaming grouped GEMM.
 // All sum a group's rows in the same order, k-block by k-block, value then residual.
 // VMOE_PAIR=0 in the environment turns the pair kernels off.
+enum WgradKernel { WGRAD_RESIDENT, WGRAD_STREAM, WGRAD_ONE_SM };
+inline WgradKernel wgrad_kernel(const Dims &p, int M, int N, bool ksplit, bool slices) {
+    const bool pair_pays = ksplit || p.C <= 32 || p.C > 2 * BK;
+    if (!pair_enabled()) return WGRAD_ONE_SM;
+    if (pair_pays && M % 256 == 0 && N % 256 == 0 && p.C <= 4 * BK) return WGRAD_RESIDENT;
+    return !slices && M >= 256 && N >= 256 ? WGRAD_STREAM : WGRAD_ONE_SM;
+}
+// Whether it pays to launch it late (LaunchChain).  Not on the resident kernel with few
+// units, each a pair's chain of M / 256 row tiles; beside its predecessor it loses more
+// than the start gains.  Measured on GB300 (us a backward, every gradient that may be
+// late against those with two units a pair against none): 45 groups of d 256, f 3840,
+// C 256: 242, 169, 181, and C 1 with 5 tokens: 116, 58, 64 (dW2: 45 units); 16 groups of
+// d 768, f 3072, C 4 with 8 tokens: 103, 75, 73 (48 units); attention, 28 groups of d
+// 1280, 4 heads, C 8: 72, 56, 56 (84 and 140 units).  From two units a pair on, and on
+// the other kernels, late gains 1 to 17% (groups = entries of the launch).
+inline bool wgrad_late_pays(const Dims &p, int M, int N, bool ksplit, int groups, bool slices) {
+    return wgrad_kernel(p, M, N, ksplit, slices) != WGRAD_RESIDENT || (long long)groups * (N / 256) >= num_sms();
+}
+
 inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __nv_bfloat16 *act2,
                       int N, const int32_t *load, __nv_bfloat16 *D, cudaStream_t s,
                       const char *name, bool late, bool ksplit = false, const Slice &sl = Slice(),
@@ -1480,10 +1499,8 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
         a.crow = sl.crow;
         a.compact = sl.compact;
     }
-    const bool pair_pays = ksplit || C <= 32 || C > 2 * BK;
-    const bool resident = pair_pays && M % 256 == 0 && N % 256 == 0 && C <= 4 * BK;
-    const bool stream = !resident && sl.n == 0 && M >= 256 && N >= 256;
-    if (pair_enabled() && (resident || stream)) {
+    const WgradKernel kernel = wgrad_kernel(p, M, N, ksplit, sl.n > 0);
+    if (kernel != WGRAD_ONE_SM) {
         // Each CTA of a pair loads 128 columns (two chunks) of A and of B.  The
         // group-indexed maps have exactly C rows per group, and with ksplit the
         // residual gets a map of its own (base C rows in, group stride 2C rows),
@@ -1499,7 +1516,7 @@ inline int wgrad_gemm(const Dims &p, const __nv_bfloat16 *act1, int M, const __n
         }
         a.tiles_m = (M + 255) / 256;
         a.tiles_n = (N + 255) / 256;
-        if (stream) {
+        if (kernel == WGRAD_STREAM) {
             const long long tiles = (long long)a.G * a.tiles_m * a.tiles_n;
             return ksplit ? launch_pair_stream<true>(ma, mb, mblo, md, a, tiles, s, name)
                           : launch_pair_stream<false>(ma, mb, mblo, md, a, tiles, s, name);

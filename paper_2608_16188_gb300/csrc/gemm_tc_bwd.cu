@@ -99,9 +99,10 @@ int launch_expert_bwd_bf16(const Dims &p, const __nv_bfloat16 *xe, const __nv_bf
                                          "tc_dx", 0, 0, 2 * C * f)) != VMOE_OK)
         return st;
     chain.on_time({dhs, b.w1, b.load}, {b.dxe});
-    const bool late1 = chain.late({b.xe, dhs, b.load}, {b.dw1});
+    const bool late1 = chain.late({b.xe, dhs, b.load}, {b.dw1}, wgrad_late_pays(p, p.d, p.f, true, p.G(), false));
     if ((st = wgrad_gemm(p, xe, p.d, dh, p.f, load, dw1, s, "tc_dw1", late1, true)) != VMOE_OK) return st;
-    const bool late2 = chain.late({b.act, b.dye, b.load}, {b.dw2});  // beside dX still, behind a late dW1
+    // beside dX still, behind a late dW1
+    const bool late2 = chain.late({b.act, b.dye, b.load}, {b.dw2}, wgrad_late_pays(p, p.f, p.d, false, p.G(), false));
     return wgrad_gemm(p, act, p.f, dye, p.d, load, dw2, s, "tc_dw2", late2);
 }
 
@@ -254,7 +255,7 @@ int launch_expert_bwd_bf16_sliced(const Dims &p, const __nv_bfloat16 *xe, const 
         sl.compact = CMP_B;
         PairSchedule sc;
         slice_schedule(slice, sc);
-        const bool late = chain.late({b.xe, ws, b.load}, {b.dw1});
+        const bool late = chain.late({b.xe, ws, b.load}, {b.dw1}, wgrad_late_pays(p, p.d, p.f, true, n, true));
         st = wgrad_gemm(p, xe, p.d, dh, p.f, load, dw1, s, "tc_dw1", late, true, sl, &sc);
         pos += n;
         ++ns;
@@ -290,7 +291,7 @@ int launch_attn_expert_bwd(const Dims &p, int H, const __nv_bfloat16 *xe, const 
     int st = row_gemm<EPI_STORE, false>(p, dye, p.d, wo, hd, load, dout, nullptr, nullptr, s, "attn_dout");
     if (st != VMOE_OK) return st;
     chain.on_time({sdye, swo, sload}, {sdout});
-    const bool late_o = chain.late({so, sdye, sload}, {sdwo});
+    const bool late_o = chain.late({so, sdye, sload}, {sdwo}, wgrad_late_pays(p, hd, p.d, false, p.G(), false));
     if ((st = wgrad_gemm(p, o, hd, dye, p.d, load, dwo, s, "attn_dwo", late_o)) != VMOE_OK) return st;
     if ((st = launch_attn_core_bwd(p.G(), p.C, H, load, qkv, o, lse, dout, dsum, dqkv, s)) != VMOE_OK)
         return st;
@@ -298,7 +299,7 @@ int launch_attn_expert_bwd(const Dims &p, int H, const __nv_bfloat16 *xe, const 
                                          "attn_dxe")) != VMOE_OK)
         return st;
     chain.on_time({sdqkv, swqkv, sload}, {sdxe});  // the core's launches wait at their start too
-    const bool late_qkv = chain.late({sxe, sdqkv, sload}, {sdwqkv});
+    const bool late_qkv = chain.late({sxe, sdqkv, sload}, {sdwqkv}, wgrad_late_pays(p, p.d, 3 * hd, false, p.G(), false));
     return wgrad_gemm(p, xe, p.d, dqkv, 3 * hd, load, dwqkv, s, "attn_dwqkv", late_qkv);
 }
 

@@ -37,10 +37,11 @@ class LaunchChain {
         open(writes, true);
     }
 
-    // Whether the next launch may be late; if not, it is an on-time one.  An entry
-    // point's first launch never is: what runs before it is not known here.
-    bool late(Spans reads, Spans writes) {
-        if (!anchored_ || n_ + (int)(reads.size() + writes.size()) > MAX || touches(reads, false) ||
+    // Whether the next launch is a late one: `wanted`, and it may be; if not, it is an
+    // on-time one.  An entry point's first launch never is late: what runs before it
+    // is not known here.
+    bool late(Spans reads, Spans writes, bool wanted = true) {
+        if (!wanted || !anchored_ || n_ + (int)(reads.size() + writes.size()) > MAX || touches(reads, false) ||
             touches(writes, true)) {
             on_time(reads, writes);
             return false;
