@@ -50,14 +50,14 @@ constexpr int EPI_WARP_BYTES = 32 * 80;  // 32 rows x (64 data + 16 pad) bytes
 
 // Row-mode epilogue of the one-SM grouped GEMM: the two-output epilogues
 // (FC1 + GELU, dA + GELU') run 16 epilogue warps (4 per TMEM lane quarter),
-// the plain store 8, all in 32-column chunks.  The two-output epilogues are
-// issue-bound at 8 warps (about 31 instructions per output element); 16 warps
-// leave room for 3 pipeline stages instead of 4, which the plain-store GEMMs,
-// bound by their operand stream, cannot spare.  Measured on GB300 (ms; 8 -> 16
-// warps): dA 0.536 -> 0.518 and FC1 0.485 -> 0.477 at the 17-task ViT-B step,
-// 0.370 -> 0.321 and 0.301 -> 0.285 at the 6-task one; FC2 / dX 0.425 ->
-// 0.433 / 0.434 -> 0.445 at 17 tasks, hence 8 there.  16-column chunks (4
-// stages with 16 warps) gained nothing.
+// the plain store 8, all in 32-column chunks.  The two-output epilogues spend
+// about 26 instructions per output element, which 8 warps do not issue fast
+// enough; 16 warps leave room for 3 pipeline stages instead of 4, which the
+// plain-store GEMMs, bound by their operand stream, cannot spare.  Measured on
+// GB300 (ms; 8 -> 16 warps, then at 31 to 38 instructions an element): dA 0.536 ->
+// 0.518 and FC1 0.485 -> 0.477 at the 17-task ViT-B step, 0.370 -> 0.321 and 0.301
+// -> 0.285 at the 6-task one; FC2 / dX 0.425 -> 0.433 / 0.434 -> 0.445 at 17 tasks,
+// hence 8 there.  16-column chunks (4 stages with 16 warps) gained nothing.
 constexpr int EPI_WARP_BYTES_TMA = 2 * 4096;  // two 32 x 64 bf16 tiles, 128-byte swizzle
 constexpr int MAX_G = 1024;
 constexpr unsigned long long TIMEOUT_NS = 4000000000ull;
@@ -87,8 +87,9 @@ struct UseTmaStore {
 
 template <int BN, int MODE, int EPI>
 struct Shape {
-    // Weight-gradient tiles have K = load <= 2 slots, so 3 slots suffice and
-    // leave room for the double-buffered 128-byte-swizzled TMA-store staging.
+    // Weight gradients are bound by their stores, not by the ring (their K is a
+    // group's load): 3 slots at BN 256 leave room for the double-buffered
+    // 128-byte-swizzled TMA-store staging.
     static constexpr bool TMA_EPI = UseTmaStore<MODE, EPI>::value;
     static constexpr int NT = Roles<MODE, EPI>::NT;
     static constexpr int EPI_BYTES =
@@ -328,9 +329,11 @@ struct ClcQueue {
     uint4 resp[CLC_DEPTH + 1];  // the last one: draining after an abort
     uint64_t full[CLC_DEPTH], empty[CLC_DEPTH], drain;
 };
-template <bool PAIR>
+// One request, its answer to `resp` and `bar` of both CTAs of the pair (BOTH), or of
+// this one alone.
+template <bool BOTH>
 __device__ __forceinline__ void clc_try(uint32_t resp, uint32_t bar) {
-    if (PAIR)
+    if (BOTH)
         asm volatile(
             "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.multicast::cluster::all.b128 "
             "[%0], [%1];" ::"r"(resp),
@@ -370,7 +373,6 @@ __device__ __forceinline__ void clc_init(ClcQueue &q, int consumers) {
 // After an abort the CTAs not launched yet are taken and dropped, so that none
 // of them starts and runs into the same wait -- as long as each answer has been
 // read and held a CTA: asking again after "none left" is undefined.
-template <bool PAIR>
 __device__ __forceinline__ void clc_scheduler(ClcQueue &q, uint32_t leader_empty, volatile int *abort_flag,
                                               int *status) {
     const bool issue = leader_empty == 0;
@@ -384,7 +386,7 @@ __device__ __forceinline__ void clc_scheduler(ClcQueue &q, uint32_t leader_empty
         }
         fence_proxy_async();  // the readers' reads of the slot before it is written again
         mbar_expect_tx(smem_u32(q.full + s), 16);
-        if (issue) clc_try<PAIR>(smem_u32(q.resp + s), smem_u32(q.full + s));
+        if (issue) clc_try<true>(smem_u32(q.resp + s), smem_u32(q.full + s));
         if (!wait_phase(smem_u32(q.full + s), ph, abort_flag, status)) {
             ok = false;
             const unsigned long long t0 = global_ns();  // the answer in flight lands before the CTA exits

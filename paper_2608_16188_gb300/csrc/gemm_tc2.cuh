@@ -424,7 +424,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         give_up();
     } else if (warp == THREADS / 32 + 1) {
         // ------------------------------------------------------------ scheduler
-        if (!sched.enabled && elect_one()) clc_scheduler<true>(clc, leader_empty, abort_flag, args.status);
+        if (!sched.enabled && elect_one()) clc_scheduler(clc, leader_empty, abort_flag, args.status);
         __syncwarp();
         give_up();
     } else if (warp == 1) {
@@ -745,7 +745,7 @@ wgrad_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         give_up();
     } else if (warp == THREADS / 32 + 1) {
         // ------------------------------------------------------------ scheduler
-        if (elect_one()) clc_scheduler<true>(clc, leader_empty, abort_flag, args.status);
+        if (elect_one()) clc_scheduler(clc, leader_empty, abort_flag, args.status);
         __syncwarp();
         give_up();
     } else if (warp == 1) {

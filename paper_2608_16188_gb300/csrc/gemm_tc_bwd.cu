@@ -191,7 +191,7 @@ int launch_expert_bwd_bf16_sliced(const Dims &p, const __nv_bfloat16 *xe, const 
     // column tiles on a share of the pairs from the fill-clamp-refill allocation
     // (Section 3.2.2): work = its tiles x (output bytes + load x input bytes per
     // row), at least one pair, at most one pair per tile; slices with more
-    // groups than pairs keep the round-robin schedule.
+    // groups than pairs keep the default one, units by cluster launch control.
     const bool use_shares = shares_enabled() && pair_enabled() && p.d % 256 == 0 && p.f % 256 == 0 &&
                             p.C <= 4 * BK;
     const int pairs = use_shares ? pair_wgrad_capacity<true>(p.C) : 0;

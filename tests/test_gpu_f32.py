@@ -1,4 +1,4 @@
-"""fp32 problems where the CUDA-core kernels change path: 128- and 64-wide tiles with ragged edges, K ranges
+"""fp32 problems where the CUDA-core kernels change path: row tiles of 16, 32 and 64 with ragged edges, K ranges
 split over a cluster, router chunks and expert passes with remainders, one token.  Held to the fp32 bars of the
 parity tests (1e-5 of an output's RMS: sums of a few hundred to a few thousand fp32 products in any order stay
 under 1e-6)."""
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 Config = workloads.Config
 CASES = [
-    # 64 groups: 128 x 128 tiles; d = 72 and f = 1028 end inside a tile and a K chunk
+    # 64 groups: no K split; d = 72 and f = 1028 end inside a tile and a K chunk
     Config("f32_wide_tiles", 90, T=2, N=300, d=72, f=1028, E=32, k=2, cf=1.25, dtype="f32", bias="drift"),
     # 2 groups, K = 516 (33 chunks) over 8 CTAs; row tiles of 64 and of 2 rows
     Config("f32_split", 91, T=1, N=66, d=128, f=516, E=2, k=2, cf=1.0, dtype="f32", flags=4),

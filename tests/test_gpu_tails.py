@@ -1,9 +1,9 @@
 """Group tails of the expert GEMMs against the fp64 oracle.
 
 The grouped GEMMs load only a group's valid rows: row-mode A tiles load
-16 ceil(load / 16) rows as 64-, 32- and 16-row boxes, and the resident-B
-weight-gradient kernels (one SM, and SM pairs) load a group's last k-block
-with a 16-, 32- or 48-row box.  Here every group of one launch has its own
+16 ceil(load / 16) rows as 64-, 32- and 16-row boxes, and the weight gradients
+take a group's rows in k-blocks of 64 that end at its last row, the first one's
+missing rows before row 0 read as zeros.  Here every group of one launch has its own
 load, covering each residue (0, 1, 15-17, 31-33, ..., 127, 128 rows of a
 128-row capacity; up to 256 rows of a 256-row one), and every
 padding row of the inputs (rows s >= load of xe, dye and the workspace) holds
@@ -61,12 +61,12 @@ def _zero_pad(t, valid):
     return t
 
 
-# d 128 / f 256 and d 256 / f 384: the one-SM weight-gradient kernels (resident B,
-# and streaming with 128-column tiles); d 256 / f 512 and d 512 / f 256: the
-# SM-pair kernel for dW1 (C 128: two resident B tiles; C 256: one) and for dW2
-# (C 32 and C 256; with C 128 dW2 streams).  With C 256 the row-mode GEMMs run on
-# SM pairs (256-row tiles), with 256-column tiles (d 512 / f 256) and 128-column
-# ones (d 384 / f 640, whose weight gradients stream).
+# d 128 / f 256: the one-SM weight-gradient kernel; d 256 / f 384 and d 384 / f 640:
+# the streaming SM-pair kernel with ragged edge tiles; d 256 / f 512 and d 512 / f
+# 256: the resident SM-pair kernel for dW1 (C 128: two B tiles; C 256: one) and for
+# dW2 (C 32 and C 256; with C 128 dW2 streams).  With C 256 the row-mode GEMMs have
+# two row tiles a group, 256 columns wide (f 256, 512) and 128 (f 640); with
+# VMOE_ROW_PAIR=1 (test_gpu_schedules.py) they run on SM pairs.
 @pytest.mark.parametrize("dtype,d,f,C", [("bf16", 128, 256, 128), ("bf16", 256, 384, 128),
                                          ("bf16", 256, 512, 128), ("bf16", 512, 256, 256),
                                          ("bf16", 256, 512, 32), ("bf16", 384, 640, 256),

@@ -10,8 +10,8 @@ import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_16188_gb300", "csrc")
 
-# Lines "w reads... / writes..." (on time) or "l reads... / writes..." (late if it may be); a
-# buffer is "address:bytes".  Prints 1 or 0 for each l.
+# Lines "w reads... / writes..." (on time), "l reads... / writes..." (late if it may be) or "u ..."
+# (it may be, but is not wanted); a buffer is "address:bytes".  Prints 1 or 0 for each l and u.
 PROGRAM = r"""
 #include <cstdio>
 #include <iostream>
@@ -38,7 +38,7 @@ int main() {
         for (auto &v : s) v.resize(4, none);
         LaunchChain::Spans r = {s[0][0], s[0][1], s[0][2], s[0][3]}, q = {s[1][0], s[1][1], s[1][2], s[1][3]};
         if (kind == "w") c.on_time(r, q);
-        else printf("%d\n", (int)c.late(r, q));
+        else printf("%d\n", (int)c.late(r, q, kind != "u"));
     }
 }
 """
@@ -86,6 +86,12 @@ def test_the_output_of_an_open_launch_is_waited_for(chain):
     # ... and what a late one writes; behind an on-time launch it is complete
     assert chain("w %s / %s\nl %s / %s\nl %s / %s\n" % (XE, DXE, ACT, DW1, DW1, DW2)) == [1, 0]
     assert chain("w %s / %s\nl %s / %s\nw %s / %s\nl %s / %s\n" % (XE, DXE, ACT, DW1, XE, DH, DXE, DW2)) == [1, 1]
+
+
+def test_an_unwanted_late_launch_is_on_time(chain):
+    lines = "w %s / %s\n%s %s / %s\nl %s / %s\n"
+    assert chain(lines % (XE, DXE, "l", ACT, DW1, DXE, DW2)) == [1, 0]
+    assert chain(lines % (XE, DXE, "u", ACT, DW1, DXE, DW2)) == [0, 1]  # it has waited: dX has completed
 
 
 def test_more_buffers_than_the_chain_holds(chain):
